@@ -37,6 +37,11 @@ __global__ void k_batch_advance(int64_t* clocks, const int* every, int n_ctx, in
 cudaError_t launch_sweep_batch(const BatchArgs& b, int n_tasks, int cluster, int threads, size_t smem, int modes,
                                cudaStream_t st) {
     const BatchKernel kernel = batch_kernel(cluster > 1, modes, threads);
+    int dev = 0, reserved = 0;  // (the canonical members' table addresses: see kReservedSmem)
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess ||
+        reserved != kReservedSmem)
+        return cudaErrorInvalidConfiguration;
     if (smem > 48 * 1024) {
         const cudaError_t e =
             cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));

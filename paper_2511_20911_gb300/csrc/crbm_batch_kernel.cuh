@@ -45,21 +45,21 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_sweep_batch(const __grid_con
         else
             bp::sweep_bitplane_body<false>(a, hrec, vrec, task.y, t0, a.n_sweeps, a.clock[1]);
     } else if ((kModes & kBatchPaper) && a.g.paper) {  // whole words
-        if (b.smem_rec)
-            canon::sweep_canon_body<true, false, true>(a, task.y, t0, a.n_sweeps, a.clock[1]);
+        if (b.canon_mode == kCanonRec)
+            canon::sweep_canon_body<kCanonRec, false, true>(a, task.y, t0, a.n_sweeps, a.clock[1]);
         else
-            canon::sweep_canon_body<false, false, true>(a, task.y, t0, a.n_sweeps, a.clock[1]);
+            canon::sweep_canon_body<kCanonPacked, false, true>(a, task.y, t0, a.n_sweeps, a.clock[1]);
     } else if (kCluster && task.w > 1) {
         const int rank = static_cast<int>(cg::this_cluster().block_rank());
         const int rank0 = task.z < task.w ? rank - task.z : 0;
-        if (b.smem_rec)
-            canon::sweep_canon_body<true, true>(a, task.y, t0, a.n_sweeps, a.clock[1], task.z, rank0);
+        if (b.canon_mode == kCanonRec)
+            canon::sweep_canon_body<kCanonRec, true>(a, task.y, t0, a.n_sweeps, a.clock[1], task.z, rank0);
         else
-            canon::sweep_canon_body<false, true>(a, task.y, t0, a.n_sweeps, a.clock[1], task.z, rank0);
-    } else if (b.smem_rec) {
-        canon::sweep_canon_body<true, false>(a, task.y, t0, a.n_sweeps, a.clock[1]);
+            canon::sweep_canon_body<kCanonPacked, true>(a, task.y, t0, a.n_sweeps, a.clock[1], task.z, rank0);
+    } else if (b.canon_mode == kCanonRec) {
+        canon::sweep_canon_body<kCanonRec, false>(a, task.y, t0, a.n_sweeps, a.clock[1]);
     } else {
-        canon::sweep_canon_body<false, false>(a, task.y, t0, a.n_sweeps, a.clock[1]);
+        canon::sweep_canon_body<kCanonPacked, false>(a, task.y, t0, a.n_sweeps, a.clock[1]);
     }
 }
 

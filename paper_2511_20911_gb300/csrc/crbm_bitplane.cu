@@ -40,7 +40,7 @@ constexpr int kBpMaxThreads = CRBM_SWEEP_MAX_THREADS;  // largest CTA the launch
 // the L=18 grid tunes to) fit on an SM; CTAs of up to kBpMaxThreads threads.
 template <bool kSmemRec, bool kSwap>
 __global__ void __maxnreg__(56) k_sweep_bitplane(const SweepArgs a, int chunk, int* state) {
-    extern __shared__ __align__(16) uint32_t smem[];
+    extern __shared__ __align__(128) uint32_t smem[];
     __shared__ int s_word, s_chunk;
     const Geometry& g = a.g;
     const int lane = threadIdx.x & 31;

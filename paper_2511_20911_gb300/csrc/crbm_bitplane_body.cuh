@@ -47,7 +47,7 @@ __host__ __device__ inline size_t bp_strag_words(const Geometry& g) { return 2 *
 template <bool kSwap>
 __device__ __forceinline__ void sweep_bitplane_body(const SweepArgs& a, const uint32_t* hrec, const uint32_t* vrec,
                                                     int word, uint32_t t0, int n_sweeps, int64_t meas) {
-    extern __shared__ __align__(16) uint32_t smem[];
+    extern __shared__ __align__(128) uint32_t smem[];
     const Geometry& g = a.g;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
     // the warp that keeps the running sums and finishes each measurement: the last, which has the
@@ -248,14 +248,21 @@ __device__ __forceinline__ void sweep_bitplane_body(const SweepArgs& a, const ui
             atomicAdd(&s_cnt[32 + lane], anti1);
             atomicAdd(&s_cnt[64 + lane], pos);
             __syncthreads();
-            if (warp == post_warp) post_sweep_warp(a, s_cnt, s_sob, s_bos, lane, word, t, do_meas, do_swap, meas, s_acc);
-            if (do_meas) ++meas;
+            RungCounts rc{0, 0, 0};
+            if (warp == post_warp) {
+                rc = rung_counts(a, s_cnt, s_sob, lane);
+                if (do_swap) swap_rungs(a, rc, s_sob, s_bos, lane, word, t, swap_uniform(a, lane, word, t));
+            }
             // a measurement alone touches only warp post_warp's sums and the counts, which the next
             // measurement reaches after the next sweep's barriers; a swap round re-permutes the planes
             if (do_swap) {
                 __syncthreads();
                 permute_planes();
                 __syncthreads();
+            }
+            if (do_meas) {
+                if (warp == post_warp) add_measurement(a, rc, lane, word, t, meas, s_acc);
+                ++meas;
             }
         }
     }

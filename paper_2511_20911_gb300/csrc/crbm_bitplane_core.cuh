@@ -8,6 +8,7 @@
 namespace crbm {
 namespace bp {
 
+using dev::transpose32;
 using dev::U4;
 
 // One plane of the comparison u < t, most significant bit first: lt collects
@@ -60,20 +61,6 @@ __device__ __forceinline__ uint4 visible_planes(const uint32_t* tb, uint32_t hp,
     const uint4 m01 = mux(n.c0, sel(1), sel(0));
     const uint4 m23 = mux(n.c0, sel(3), sel(2));
     return mux(n.c2, sel(4), mux(n.c1, m23, m01));
-}
-
-// 32 x 32 bit transpose across a warp: lane c returns the word whose bit l is
-// bit c of lane l's x (block swaps of 16, 8, 4, 2 and 1 rows and columns).
-__device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
-    constexpr uint32_t kLow[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
-#pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        const int j = 16 >> i;
-        const uint32_t m = kLow[i];
-        const uint32_t y = __shfl_xor_sync(0xffffffffu, x, j);
-        x = (lane & j) ? ((x & ~m) | ((y >> j) & m)) : ((x & m) | ((y << j) & ~m));
-    }
-    return x;
 }
 
 // Appends the lanes whose comparison is still open (open != 0: its

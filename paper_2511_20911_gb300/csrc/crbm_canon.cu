@@ -2,7 +2,7 @@
 // (32 chains) -- the whole even, periodic lattice, its hidden layer and the
 // lane-expanded tables -- in shared memory and runs a chunk of sweeps on it.
 // The sweep body is in crbm_canon_body.cuh, the per-cell cores in
-// crbm_canon_core.cuh.
+// crbm_row_core.cuh.
 #include <algorithm>
 
 #include "crbm_canon_body.cuh"
@@ -26,25 +26,34 @@ using namespace canon;
 // the word's spins and sums, then releases it with the new count and claims
 // again.  A CTA that finds no free unfinished word exits: every unfinished
 // word is then held by a running CTA, which claims again after its chunk, so
-// no work is left behind and nothing waits.
+// no work is left behind and nothing waits.  A launch with a CTA for every word
+// has no states (nullptr) and one item per CTA.
 //
-// Two instantiations per variant: one for CTAs of at most kSmallCta threads
-// (12 warps, the shape the L=18 grid tunes to) at two CTAs per SM, which may
-// take 80 registers a thread and keeps the sweep loop free of spills, and one
-// for any CTA, at 64 registers.  A launch takes the first wherever its CTA
-// fits it and it holds as many CTAs per SM as the second.
-constexpr int kSmallCta = 384;
-template <bool kSmemRec, bool kPaper, int kMaxThreads>
-__global__ void __launch_bounds__(kMaxThreads, kMaxThreads <= kSmallCta ? 2 : CRBM_SWEEP_MIN_BLOCKS)
+// Three instantiations per variant: kCtaWide, CTAs of at most 512 threads alone
+// on their SM, which may take 128 registers a thread (ladders of the L=18
+// lattice, 96 words in CTAs of 16 warps: 4.67 us per sweep against 4.88 at 64
+// registers); kCtaPair, CTAs of at most 384 threads at two or more per SM, 80
+// registers (L=18 grid, 500 sweeps in CTAs of 8 warps: 5.28 ms; 5.41 at 128
+// registers); kCtaAny, any CTA at 64 registers.
+constexpr int kCtaAny = CRBM_SWEEP_MAX_THREADS, kCtaPair = 384, kCtaWide = 512;
+template <int kMode, bool kPaper, int kMaxThreads>
+__global__ void __launch_bounds__(kMaxThreads, kMaxThreads == kCtaPair ? 2 : CRBM_SWEEP_MIN_BLOCKS)
     k_sweep_canon_persistent(const SweepArgs a, int chunk, int* state) {
-    __shared__ int s_word, s_chunk;
+    extern __shared__ __align__(128) uint32_t smem[];  // (no static shared memory: see kReservedSmem)
+    int& s_word = reinterpret_cast<int*>(smem + canon_smem(a.g, kMode).seg)[33];
+    int& s_chunk = reinterpret_cast<int*>(smem + canon_smem(a.g, kMode).seg)[34];
     const int n_chunks = (a.n_sweeps + chunk - 1) / chunk;
     const int nw = a.n_words, nq = (nw + 3) / 4;
     const int K = a.measure_every;
     const int lane = threadIdx.x & 31;
     const unsigned int start = (blockIdx.x * 97u) % static_cast<unsigned int>(nw);
-    for (;;) {
-        if (threadIdx.x < 32) {
+    for (bool first = true;; first = false) {
+        if (state == nullptr) {  // a CTA per word: nothing to schedule
+            if (threadIdx.x == 0) {
+                s_word = first ? static_cast<int>(blockIdx.x) : -1;
+                s_chunk = 0;
+            }
+        } else if (threadIdx.x < 32) {
             int word = -1, c = 0;
             for (int tries = 0; tries < (1 << 20) && word < 0; ++tries) {
                 int best = 0x7fffffff, bk = 0x7fffffff, bw = -1;  // (chunks done, scan rank, word)
@@ -97,9 +106,9 @@ __global__ void __launch_bounds__(kMaxThreads, kMaxThreads <= kSmallCta ? 2 : CR
         const int n = min(chunk, a.n_sweeps - c * chunk);
         const int64_t meas0 =
             K > 0 ? a.meas0 + static_cast<int64_t>(t0 / K) - static_cast<int64_t>(a.t0 / K) : a.meas0;
-        sweep_canon_body<kSmemRec, false, kPaper>(a, word, t0, n, meas0);
+        sweep_canon_body<kMode, false, kPaper>(a, word, t0, n, meas0, 0, 0, first);
         __syncthreads();  // every thread's state stores are issued
-        if (threadIdx.x == 0) {
+        if (threadIdx.x == 0 && state != nullptr) {
             __threadfence();
             st_release(state + word, 2 * (c + 1));
         }
@@ -108,65 +117,154 @@ __global__ void __launch_bounds__(kMaxThreads, kMaxThreads <= kSmallCta ? 2 : CR
 
 }  // namespace
 
-bool canon_smem_records(const Geometry& g) {
-    constexpr size_t kSmemPerSm = 228 * 1024, kCtaMax = 227 * 1024, kReserve = 1024;
-    const size_t base = smem_bytes_canon(g);
-    const size_t with = sizeof(uint32_t) * canon_smem_rec_offset(g) + sizeof(uint4) * g.n_cells * kCellRec;
-    if (with > kCtaMax) return false;
-    const size_t per_sm_base = std::min<size_t>(2, kSmemPerSm / (base + kReserve));
-    return kSmemPerSm / (with + kReserve) >= per_sm_base;
+size_t smem_bytes_canon(const Geometry& g) {
+    const size_t words = static_cast<size_t>(kAccWords) + kCanonTab + g.N + static_cast<size_t>(g.n_cells) * 32 + 96 + 33 +
+                         32 + 64 + 3;
+    return sizeof(uint32_t) * ((words & ~static_cast<size_t>(3)) + (g.paper ? static_cast<size_t>(g.n_cells) * 64 : 0));
 }
-
-size_t smem_bytes_canon_launch(const Geometry& g) {
-    return canon_smem_records(g)
-               ? sizeof(uint32_t) * canon_smem_rec_offset(g) + sizeof(uint4) * g.n_cells * kCellRec
-               : smem_bytes_canon(g);
-}
-
-size_t smem_bytes_canon(const Geometry& g) { return sizeof(uint32_t) * canon_smem_rec_offset(g); }
 
 namespace {
-template <bool kSmemRec, bool kPaper>
-cudaError_t launch_persistent(const SweepArgs& a, int warps_per_cta, int chunk, int* sched, cudaStream_t st) {
-    const size_t smem = smem_bytes_canon_launch(a.g);
-    using Kernel = void (*)(const SweepArgs, int, int*);
-    const Kernel big = k_sweep_canon_persistent<kSmemRec, kPaper, CRBM_SWEEP_MAX_THREADS>;
-    const Kernel small = k_sweep_canon_persistent<kSmemRec, kPaper, kSmallCta>;
-    const int threads = warps_per_cta * 32;
-    // the spill-free instantiation where the CTA fits it and it keeps as many CTAs per SM
-    int per_sm = 0, per_sm_small = 0, dev = 0, sms = 0;
-    cudaError_t e = cudaSuccess;
-    for (const Kernel k : {big, small}) {
-        if (k == small && threads > kSmallCta) break;
-        if (smem > 48 * 1024)
-            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-        if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(k == big ? &per_sm : &per_sm_small, k, threads, smem);
-        if (e != cudaSuccess) return e;
+// Sweeps per work item: with a CTA per word, all of them; else the chunk with
+// the least (rounds of items over the grid) x (sweeps + the staging of a word,
+// 0.7 sweeps on the L=18 grid: 5.79 ms per 500 sweeps in chunks of 8, 5.56 in
+// chunks of 16).
+int pick_chunk(int n_sweeps, int n_words, int grid) {
+    if (n_words <= grid) return n_sweeps;
+    int best = n_sweeps;
+    double best_cost = 0.0;
+    for (int n_chunks = 1; n_chunks <= 64 && n_chunks <= n_sweeps; ++n_chunks) {
+        const int chunk = (n_sweeps + n_chunks - 1) / n_chunks;
+        const int64_t items = static_cast<int64_t>(n_words) * ((n_sweeps + chunk - 1) / chunk);
+        const double cost = static_cast<double>((items + grid - 1) / grid) * (chunk + 0.7);
+        if (n_chunks == 1 || cost < best_cost) {
+            best = chunk;
+            best_cost = cost;
+        }
     }
-    const Kernel kernel = per_sm_small >= per_sm && per_sm_small > 0 ? small : big;
-    if (kernel == small) per_sm = per_sm_small;
-    if (e == cudaSuccess) e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return best;
+}
+}  // namespace
+
+// The segments' length.  Warp w takes segments w, w + warps, ... of a half-step
+// and runs on SM sub-partition w % 4, so the half-step takes about what the
+// fullest sub-partition has to issue (its segments, each a fifth of a cell on top
+// of its cells), and a CTA alone on its SM also what its fullest warp has.
+size_t canon_plan(Geometry& g, int warps, int* mode, int bands) {
+    constexpr size_t kCtaMax = 227 * 1024;
+    auto bytes = [&](int m) { return sizeof(uint32_t) * static_cast<size_t>(canon_smem(g, m).total); };
+    auto cut = [&](int nseg) {
+        g.seg_cells = (g.Wc + nseg - 1) / nseg;
+        g.n_seg = (g.Wc + g.seg_cells - 1) / g.seg_cells;
+    };
+    const int min_seg = (g.Wc + kMaxSegCells - 1) / kMaxSegCells;
+    cut(min_seg);
+    for (*mode = kCanonRec; *mode < kCanonPacked && bytes(*mode) > kCtaMax;) ++*mode;
+    int best = min_seg;
+    double best_cost = 0.0;
+    for (int nseg = min_seg; nseg <= g.Wc; ++nseg) {
+        cut(nseg);
+        // a band does its boundary row of cells first, then the others
+        const int n = bands > 1 ? ((g.W + bands - 1) / bands - 1) * g.n_seg : g.W * g.n_seg;
+        int rounds = (n + warps - 1) / warps, fullest = bands > 1 ? (g.n_seg + 3) / 4 : 0;
+        if (bands > 1) rounds += (g.n_seg + warps - 1) / warps;
+        int most = 0;
+        for (int q = 0; q < 4; ++q) {
+            int c = 0;
+            for (int w = q; w < warps; w += 4) c += w < n ? (n - w + warps - 1) / warps : 0;
+            most = std::max(most, c);
+        }
+        fullest += most;
+        const double cost = (fullest + rounds) * (g.seg_cells + 0.2);
+        if (nseg == min_seg || (cost < best_cost && bytes(*mode) <= kCtaMax)) {
+            best = nseg;
+            best_cost = cost;
+        }
+    }
+    cut(best);
+    return bytes(*mode);
+}
+
+namespace {
+using PersistentKernel = void (*)(const SweepArgs, int, int*);
+template <int kMaxThreads>
+PersistentKernel persistent_kernel(int mode, int paper) {
+    if (paper)
+        return mode == kCanonRec     ? k_sweep_canon_persistent<kCanonRec, true, kMaxThreads>
+               : mode == kCanonPlain ? k_sweep_canon_persistent<kCanonPlain, true, kMaxThreads>
+                                     : k_sweep_canon_persistent<kCanonPacked, true, kMaxThreads>;
+    return mode == kCanonRec     ? k_sweep_canon_persistent<kCanonRec, false, kMaxThreads>
+           : mode == kCanonPlain ? k_sweep_canon_persistent<kCanonPlain, false, kMaxThreads>
+                                 : k_sweep_canon_persistent<kCanonPacked, false, kMaxThreads>;
+}
+PersistentKernel persistent_kernel(int mode, int paper, int cta) {
+    return cta == kCtaWide   ? persistent_kernel<kCtaWide>(mode, paper)
+           : cta == kCtaPair ? persistent_kernel<kCtaPair>(mode, paper)
+                             : persistent_kernel<kCtaAny>(mode, paper);
+}
+
+cudaError_t make_plan(const Geometry& g0, int n_words, int warps, int dev, CanonLaunch& p) {
+    Geometry g = g0;
+    p = CanonLaunch();
+    p.smem = canon_plan(g, warps, &p.mode);
+    p.seg_cells = g.seg_cells;
+    p.n_seg = g.n_seg;
+    int reserved = 0;
+    cudaError_t e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&p.sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    const int n_items = ((a.n_sweeps + chunk - 1) / chunk) * a.n_words;
-    const int grid = std::min(std::min(n_items, a.n_words), per_sm * sms);
-    e = cudaMemsetAsync(sched, 0, sizeof(int) * (4 + static_cast<size_t>(a.n_words)), st);
+    auto occupancy = [&](int cta, int* per_sm) {
+        const PersistentKernel k = persistent_kernel(p.mode, g.paper, cta);
+        // (always the most a CTA can have: contexts of other sizes share the kernel)
+        cudaError_t r = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        if (r == cudaSuccess) r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k, 32 * warps, p.smem);
+        return r;
+    };
+    int per_sm[3] = {0, 0, 0};  // kCtaAny, kCtaPair, kCtaWide
+    e = occupancy(kCtaAny, &per_sm[0]);
+    if (e == cudaSuccess && 32 * warps <= kCtaPair) e = occupancy(kCtaPair, &per_sm[1]);
+    if (e == cudaSuccess && 32 * warps <= kCtaWide) e = occupancy(kCtaWide, &per_sm[2]);
     if (e != cudaSuccess) return e;
-    kernel<<<grid, warps_per_cta * 32, smem, st>>>(a, chunk, sched);
-    return cudaGetLastError();
+    if (per_sm[2] > 0 && (n_words < 2 * p.sms || std::max(per_sm[0], per_sm[1]) == 1)) {
+        p.cta = kCtaWide;
+        p.per_sm = 1;
+    } else if (per_sm[1] >= per_sm[0]) {
+        p.cta = kCtaPair;
+        p.per_sm = per_sm[1];
+    } else {
+        p.cta = kCtaAny;
+        p.per_sm = per_sm[0];
+    }
+    if (p.per_sm < 1 || reserved != kReservedSmem) return cudaErrorInvalidConfiguration;
+    p.warps = warps;
+    p.device = dev;
+    return cudaSuccess;
 }
 
 }  // namespace
 
-cudaError_t launch_sweep_canon_persistent(const SweepArgs& a, int warps_per_cta, int chunk, int* sched,
+cudaError_t launch_sweep_canon_persistent(const SweepArgs& a0, int warps_per_cta, int* sched, CanonLaunch& plan,
                                           cudaStream_t st) {
-    if (a.g.paper)
-        return canon_smem_records(a.g) ? launch_persistent<true, true>(a, warps_per_cta, chunk, sched, st)
-                                       : launch_persistent<false, true>(a, warps_per_cta, chunk, sched, st);
-    return canon_smem_records(a.g) ? launch_persistent<true, false>(a, warps_per_cta, chunk, sched, st)
-                                   : launch_persistent<false, false>(a, warps_per_cta, chunk, sched, st);
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess && (plan.warps != warps_per_cta || plan.device != dev))
+        e = make_plan(a0.g, a0.n_words, warps_per_cta, dev, plan);
+    if (e != cudaSuccess) return e;
+    SweepArgs a = a0;
+    a.g.seg_cells = plan.seg_cells;
+    a.g.n_seg = plan.n_seg;
+    // no more CTAs per SM than whole words: were every word held at once, SMs with one word more
+    // than others would finish last with nothing to claim for the rest
+    const int per_sm = std::max(1, std::min(plan.per_sm, a.n_words / plan.sms));
+    const int grid = std::min(a.n_words, per_sm * plan.sms);
+    const int chunk = pick_chunk(a.n_sweeps, a.n_words, grid);
+    if (grid == a.n_words) {
+        sched = nullptr;
+    } else {
+        e = cudaMemsetAsync(sched, 0, sizeof(int) * (4 + static_cast<size_t>(a.n_words)), st);
+        if (e != cudaSuccess) return e;
+    }
+    persistent_kernel(plan.mode, a.g.paper, plan.cta)<<<grid, warps_per_cta * 32, plan.smem, st>>>(a, chunk, sched);
+    return cudaGetLastError();
 }
 
 }  // namespace crbm

@@ -1,26 +1,43 @@
 // Body of the canonical SMEM-resident sweep (one CTA = one 32-chain word, or
 // one band of cell rows of a word in a thread-block cluster), shared by the
 // persistent kernel (crbm_canon.cu) and the batched kernel (crbm_batch.cu).
+// The spins are kept in row form (crbm_row_core.cuh).
 #pragma once
+
+#include <type_traits>
 
 #include <cooperative_groups.h>
 
-#include "crbm_canon_core.cuh"
+#include "crbm_row_core.cuh"
 
 namespace crbm {
 namespace canon {
 
 namespace cg = cooperative_groups;
 
-template <bool kSmem>
-__device__ __forceinline__ uint4 ld_rec(const uint4* p) {
-    return kSmem ? *p : __ldg(p);
-}
-// The first word of a cell's record 5 (Q2.lo).
-template <bool kSmem>
-__device__ __forceinline__ uint32_t ld_rec5(const uint4* r) {
-    return kSmem ? reinterpret_cast<const uint32_t*>(r + 5)[0] : __ldg(reinterpret_cast<const uint32_t*>(r + 5));
-}
+// Cell records: in shared memory (an address) or read through the read-only
+// cache (a pointer).
+template <int kMode>
+struct CellRecs {
+    const uint4* p;
+    __device__ __forceinline__ CellRecs(uint32_t, const uint4* g, int cell) : p(g + static_cast<size_t>(cell) * kCellRec) {}
+    template <int k>
+    __device__ __forceinline__ uint4 get() const {
+        return __ldg(p + k);
+    }
+};
+template <>
+struct CellRecs<kCanonRec> {
+    uint32_t p;
+    __device__ __forceinline__ CellRecs(uint32_t s, const uint4*, int cell) : p(s + 16u * kCellRec * static_cast<uint32_t>(cell)) {}
+    template <int k>
+    __device__ __forceinline__ uint4 get() const {
+        return lds128<16 * k>(p);
+    }
+};
+
+template <int j>
+using Cell = std::integral_constant<int, j>;  // the j-th cell of a segment
 
 // The two halves of a cluster barrier, so that work no other CTA waits for
 // can run between them: arrive (release: this thread's earlier shared-memory
@@ -45,9 +62,8 @@ __device__ __forceinline__ void body_sync() {
 // measurement / replica exchange / correlations, write the state back.
 // State is read with L1-bypassing loads: under the persistent scheduler the
 // previous chunk of this word may have been written by another SM.
-// kSmemRec: the per-cell records are first copied into shared memory after
-// the replica tables (canon_smem_records() decides on the host), else read
-// through the read-only cache.
+// A warp's unit of work is a segment of a row of cells (a.g.seg_cells cells).
+// kMode: how the word is kept in shared memory (kCanon*, crbm_internal.h).
 // kCluster: the CTA holds band `band` of the word's a.n_bands bands of cell
 // rows; the word's bands are the cluster ranks rank0 .. rank0 + n_bands - 1
 // (a cluster may hold several words of one context, or padding ranks of that
@@ -67,37 +83,77 @@ __device__ __forceinline__ void body_sync() {
 // only ones that read rows a neighbour writes, and they run after the
 // previous barrier completed, so no band overwrites a row its neighbour has
 // yet to read.
+// first: false when this CTA's previous word was of the same context (its records
+// and expansion table are then in place).
 // kPaper: CRBM_PRECISION_PAPER draws (two Philox calls per cell, the visible
-// uniforms passed from the hidden half-step through shared memory).
-template <bool kSmemRec, bool kCluster, bool kPaper = false>
+// uniforms passed from the hidden half-step through shared memory, or drawn
+// again in the visible one with kCanonPacked).
+template <int kMode, bool kCluster, bool kPaper = false>
 __device__ __forceinline__ void sweep_canon_body(const SweepArgs& a, int word, uint32_t t0, int n_sweeps,
-                                                 int64_t meas0, int band = 0, int rank0 = 0) {
-    extern __shared__ __align__(16) uint32_t smem[];
+                                                 int64_t meas0, int band = 0, int rank0 = 0,
+                                                 bool first = true) {
+    extern __shared__ __align__(128) uint32_t smem[];
+    constexpr bool kPacked = kMode == kCanonPacked && !kPaper;  // 16-bit hidden words
+    constexpr bool kRedraw = kMode == kCanonPacked && kPaper;   // the visible call drawn again
+    constexpr uint32_t kWCell = kPacked ? 64u : 128u;           // bytes of a cell's hidden words
     const Geometry& g = a.g;
     const int W = g.W, Wc = g.Wc;  // rows and columns of cells
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+    const int nseg = g.n_seg, uc = g.seg_cells;
+    // (the shuffle tells the compiler that the warp index is warp-uniform: segment indices, loop counters
+    // and cell addresses then run on the uniform pipe)
+    const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);
+    const int nwarp = blockDim.x >> 5;
     // The warp that keeps the running sums and finishes each measurement: the
-    // last, which has the fewest cells when they do not divide evenly, so that
+    // last, which has the fewest segments when they do not divide evenly, so that
     // it can finish a measurement while the others start the next sweep.
     const int post_warp = nwarp - 1;
     const int nb = kCluster ? a.n_bands : 1;
     const bool active = band < nb;
     const int row0 = active ? band * W / nb : 0, row1 = active ? (band + 1) * W / nb : 0;
-    // (the two forms of the cell range compile to measurably faster code in
-    // the exact and the paper-precision sweep respectively; they are equal)
-    const int c_begin = (kCluster || kPaper) ? row0 * Wc : 0;
-    const int c_end = (kCluster || kPaper) ? row1 * Wc : g.n_cells;
-    int64_t* s_acc = reinterpret_cast<int64_t*>(smem);  // [kNSum][32] running sums
-    uint32_t* s_th = smem + kAccWords;          // [2][4][32]
-    uint32_t* s_tv = s_th + kCanonTh;           // [4][32][32]
-    uint32_t* s_v = s_th + kCanonTab;           // [N]
-    uint32_t* s_w = s_v + g.N;                  // [n_cells][32] per-lane hidden words
-    int* s_cnt = reinterpret_cast<int*>(s_w + g.n_cells * 32);   // [3][32]
-    int* s_seg = s_cnt + 96;                                      // [33]
-    uint32_t* s_segmask = reinterpret_cast<uint32_t*>(s_seg + 33); // [32]
-    int* s_sob = reinterpret_cast<int*>(s_segmask + 32);          // [32] slot of each rung
-    int* s_bos = s_sob + 32;                                        // [32] rung of each slot
+    const int u_begin = kCluster ? row0 * nseg : 0, u_end = kCluster ? row1 * nseg : W * nseg;
+    const CanonSmem cs = canon_smem(g, kMode);
+    int64_t* s_acc = reinterpret_cast<int64_t*>(smem + cs.acc);  // [kNSum][32] running sums
+    int* s_cnt = reinterpret_cast<int*>(smem + cs.cnt);          // [3][32]
+    int* s_sob = reinterpret_cast<int*>(smem + cs.sob);          // [32] slot of each rung
+    int* s_bos = s_sob + 32;                                     // [32] rung of each slot
+    uint32_t* s_u = smem + cs.u;                                 // [32] the swap round's uniforms
+    uint32_t* s_segmask = smem + cs.segmask;
+    int* s_seg = reinterpret_cast<int*>(smem + cs.seg);
     char* sm = reinterpret_cast<char*>(smem);
+    char* s_tab = sm + 4 * kCanonTabWord;
+    const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(smem));  // shared addresses from here on
+    const uint32_t tab = base + 4u * kCanonTabWord;
+    if (tab & 16383u) return;  // (the launchers have checked it: every CTA of the grid agrees)
+    const uint32_t rec_addr = base + 4u * static_cast<uint32_t>(cs.rec);
+    const uint32_t pw_addr = base + 4u * static_cast<uint32_t>(cs.pw);
+    const uint32_t w_addr = base + 4u * static_cast<uint32_t>(cs.w);
+    const uint32_t rows_addr = base + 4u * static_cast<uint32_t>(cs.rows);
+    const uint32_t exp_addr = base + 4u * static_cast<uint32_t>(cs.expand);
+    const uint32_t lane4 = 4u * static_cast<uint32_t>(lane);
+    const uint32_t lane_w = kPacked ? 2u * static_cast<uint32_t>(lane) : lane4;
+    const uint32_t seg_magic = nseg > 1 ? (0xFFFFFFFFu / static_cast<uint32_t>(nseg)) + 1u : 0u;
+    // Segment u: cells j0 .. j0 + n - 1 of row i; the segment below it, and the one to its left
+    struct Segment {
+        int i, j0, n, below, left;
+    };
+    auto segment = [&](int u) {
+        Segment r;
+        r.i = nseg > 1 ? static_cast<int>(__umulhi(static_cast<uint32_t>(u), seg_magic)) : u;
+        const int s = u - r.i * nseg;
+        r.j0 = s * uc;
+        r.n = min(uc, Wc - r.j0);
+        r.below = r.i + 1 == W ? s : u + nseg;
+        r.left = s > 0 ? u - 1 : u + nseg - 1;
+        return r;
+    };
+    auto row_addr = [&](int u) { return rows_addr + 128u * static_cast<uint32_t>(u) + lane4; };
+    // a segment's new nibbles, and its first column for the segment to its left
+    auto store_row = [&](int u, const Segment& sg, uint32_t o) {
+        sts16<2>(row_addr(u), o);
+        sts8<1>(row_addr(sg.left), (o >> (4u * static_cast<uint32_t>(sg.n) - 2u)) << 6);
+    };
+    auto w_of = [&](int cell) { return w_addr + kWCell * static_cast<uint32_t>(cell) + lane_w; };
+    auto load_w = [&](uint32_t addr) -> uint32_t { return kPacked ? lds32(exp_addr + 4u * lds16(addr)) : lds32(addr); };
     // cluster neighbours (unused without a split)
     char* sm_next = sm;
     char* sm_prev = sm;
@@ -113,21 +169,48 @@ __device__ __forceinline__ void sweep_canon_body(const SweepArgs& a, int word, u
         bos0 = cl.map_shared_rank(s_bos, static_cast<unsigned int>(rank0));
     }
 
-    const uint4* recs = a.crec;
     const uint32_t chain = static_cast<uint32_t>(word) * 32u + lane;
-    LaneConst lc = lane_const(lane, lane);
     const Round0Lane r0l = round0_lane(chain);
     const bool measuring = a.measure_every > 0;
     if (active) {
-        if (kSmemRec) {  // [n_cells][kCellRec] records, 16-byte aligned
-            uint4* s_rec = reinterpret_cast<uint4*>(smem + canon_smem_rec_offset(g));
-            for (int x = threadIdx.x; x < g.n_cells * kCellRec; x += blockDim.x) s_rec[x] = __ldg(a.crec + x);
-            recs = s_rec;
-        }
-        const uint4* gt = reinterpret_cast<const uint4*>(a.ctab + static_cast<size_t>(word) * kCanonTab);
-        for (int x = threadIdx.x; x < kCanonTab / 4; x += blockDim.x) reinterpret_cast<uint4*>(s_th)[x] = gt[x];
+        // (every load of the staging is in flight before the first is waited for: a one-sweep launch
+        // is mostly this)
+        const uint32_t* gt = a.ctab + static_cast<size_t>(word) * kCanonTab;
+        auto stage = [&](uint32_t dst, const uint4* src, int n) {
+            for (int x = threadIdx.x; x < n; x += blockDim.x)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16u * static_cast<uint32_t>(x)), "l"(src + x)
+                             : "memory");
+        };
+        stage(tab + kRowVis, reinterpret_cast<const uint4*>(gt + kCanonTh), 4 * 32 * 32 / 4);
+        if (kMode == kCanonRec && first) stage(rec_addr, a.crec, g.n_cells * kCellRec);
+        // spins to row form: the site words of a segment's word (lane = bit), bit-transposed (lane = chain)
         const uint32_t* gv = a.v + static_cast<size_t>(word) * g.N;
-        for (int x = threadIdx.x; x < g.N; x += blockDim.x) s_v[x] = __ldcg(gv + x);
+        for (int u0 = warp; u0 < W * nseg; u0 += 4 * nwarp) {
+            uint32_t v[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int u = u0 + k * nwarp;
+                v[k] = 0u;
+                if (u < W * nseg) {
+                    const Segment sg = segment(u);
+                    const int j = sg.j0 + sg.n == Wc ? 0 : sg.j0 + sg.n;  // the next segment's first cell: bits 15, 14
+                    const int p = lane - 16;
+                    const int site = p >= 0 ? row_site(p, sg.i, sg.j0, sg.n, g.Lc) : (2 * sg.i - 1 - p) * g.Lc + 2 * j;
+                    if (p >= -2 && p < 4 * sg.n) v[k] = __ldcg(gv + site);
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (u0 + k * nwarp < W * nseg) sts32(row_addr(u0 + k * nwarp), transpose32(v[k], lane));
+        }
+        build_threshold_tables(s_tab, gt, threadIdx.x, blockDim.x);
+        if (kPacked && first)
+            for (int x = threadIdx.x; x < 1024; x += blockDim.x) smem[cs.expand + x] = expand_word(static_cast<uint32_t>(x));
+        if (band == 0 && warp == post_warp && measuring) {
+#pragma unroll
+            for (int x = 0; x < kNSum; ++x)
+                s_acc[x * 32 + lane] = __ldcg(a.sums + static_cast<size_t>(chain) * kNSum + x);
+        }
         for (int x = threadIdx.x; x < 96; x += blockDim.x) s_cnt[x] = 0;
         if (a.sq_every > 0) {
             for (int x = threadIdx.x; x < 33; x += blockDim.x) s_seg[x] = a.seg[word * 33 + x];
@@ -138,146 +221,195 @@ __device__ __forceinline__ void sweep_canon_body(const SweepArgs& a, int word, u
             s_sob[lane] = sob;
             s_bos[sob] = lane;
         }
+        asm volatile("cp.async.wait_all;" ::: "memory");
     }
     __syncthreads();
-    lc.lb = 4u * static_cast<uint32_t>(s_bos[lane]);  // lane reads the column of its rung
-    if (active && band == 0 && warp == post_warp && measuring) {
-        for (int x = 0; x < kNSum; ++x)
-            s_acc[x * 32 + lane] = __ldcg(a.sums + static_cast<size_t>(chain) * kNSum + x);
-    }
+    uint32_t tab4 = tab + 4u * static_cast<uint32_t>(s_bos[lane]);  // lane reads the column of its rung
     if (kCluster) body_sync<true>();  // every rank started before any shared memory crosses CTAs
 
-    // sweep and measurement counters: kernel arguments, or the batch's device clock
     int64_t meas = meas0;
-    // Cells of this warp: c_begin + warp, + nwarp, ...; each described by its
-    // kCellRec records (shared-memory byte offsets and round-0 Philox words).
-    const uint32_t lane4 = 4u * static_cast<uint32_t>(lane);
-    const uint4* rec0 = recs + static_cast<size_t>(c_begin + warp) * kCellRec;
-    const int rstep = nwarp * kCellRec;
-    const int last_row = c_end - Wc, first_row_end = c_begin + Wc;
-
     EveryCounter every_meas(t0, a.measure_every), every_swap(t0, a.swap_every), every_sq(t0, kCluster ? 0 : a.sq_every);
     for (int it = 0; it < n_sweeps; ++it) {
         const uint32_t t = t0 + static_cast<uint32_t>(it);
         const Round1Sweep rs = round1_sweep(r0l.hi ^ t ^ a.rk[0], a.rk);
-        const uint4* rec = rec0;
-        if (kPaper && !kCluster) {
-            for (int cell = c_begin + warp; cell < c_end; cell += nwarp, rec += rstep) {
-                const uint4 h0 = ld_rec<kSmemRec>(rec), h1 = ld_rec<kSmemRec>(rec + 1),
-                            h2 = ld_rec<kSmemRec>(rec + 2);
-                sts_off(sm, h1.y + lane4, hidden_cell_rec_paper(sm, h0, h1, h2, s_th, rs, r0l.lo, a.rk, lc,
-                                                                2u * lane4));
-            }
-            __syncthreads();
-            rec = rec0;
-            for (int cell = c_begin + warp; cell < c_end; cell += nwarp, rec += rstep)
-                visible_cell_rec_paper(sm, ld_rec<kSmemRec>(rec + 3), ld_rec<kSmemRec>(rec + 4), lane4, s_tv, lc);
-            __syncthreads();
-        } else if (kCluster && nb > 1) {  // a band of a split word, or a padding rank of one
-            // the last cell row first (the next band waits for its hidden words), arrive, the rest,
-            // then wait: the cluster barrier's latency overlaps the interior rows
-            if (active) {
-                for (int cell = last_row + warp; cell < c_end; cell += nwarp) {
-                    const uint4* r = recs + static_cast<size_t>(cell) * kCellRec;
-                    const uint4 h0 = ld_rec<kSmemRec>(r), h1 = ld_rec<kSmemRec>(r + 1), h2 = ld_rec<kSmemRec>(r + 2);
-                    const uint32_t w = hidden_cell_rec(sm, h0, h1, h2, ld_rec5<kSmemRec>(r), s_th, rs, r0l.lo, a.rk, lc);
-                    sts_off(sm, h1.y + lane4, w);
-                    sts_off(sm_next, h1.y + lane4, w);
+        if (every_swap.now() && band == 0 && warp == post_warp) s_u[lane] = swap_uniform(a, lane, word, t);
+        // hidden half-step; a band's last cell row first (the next band waits for its hidden words),
+        // arrive, the rest, then wait: the cluster barrier's latency overlaps the interior rows
+        const int split = kCluster && nb > 1 ? u_end - nseg : u_begin;
+        for (int ph = kCluster && nb > 1 ? 0 : 1; ph < 2; ++ph) {
+            const int ub = ph == 0 ? split : u_begin, ue = ph == 0 || !(kCluster && nb > 1) ? u_end : split;
+            if (!kCluster || active)
+                for (int u = ub + warp; u < ue; u += nwarp) {
+                    const Segment sg = segment(u);
+                    Windows win(lds32(row_addr(u)), lds32(row_addr(sg.below)), sg.n);
+                    const int cell = sg.i * Wc + sg.j0;
+                    CellRecs<kMode> rec(rec_addr, a.crec, cell);
+                    const uint32_t wo = w_of(cell), po = pw_addr + 256u * static_cast<uint32_t>(cell) + 2u * lane4;
+                    const uint32_t tab8 = 2u * tab4 - tab;
+                    auto one = [&](auto jc) {
+                        constexpr int j = decltype(jc)::value;
+                        const HiddenThresholds th(win, tab8, tab4);
+                        const uint4 q0 = rec.template get<kCellRec * j>(), q1 = rec.template get<kCellRec * j + 1>();
+                        uint32_t w;
+                        if (kPaper) {
+                            uint2 vis;
+                            w = hidden_row_cell_paper(th, q0, q1, rs, r0l.lo, a.rk, vis);
+                            if (!kRedraw) sts64<256 * j>(po, vis);
+                        } else {
+                            w = hidden_row_cell<kPacked>(th, q0, q1, rs, r0l.lo, a.rk);
+                        }
+                        if (kPacked)
+                            sts16<static_cast<int>(kWCell) * j>(wo, w);
+                        else
+                            sts32<static_cast<int>(kWCell) * j>(wo, w);
+                        if (kCluster && ph == 0) {  // what the cells below read
+                            char* o = sm_next + (wo + kWCell * j - base);
+                            if (kPacked)
+                                *reinterpret_cast<uint16_t*>(o) = static_cast<uint16_t>(w);
+                            else
+                                *reinterpret_cast<uint32_t*>(o) = w;
+                        }
+                        win.next();
+                    };
+                    one(Cell<0>());
+                    if (sg.n > 1) {
+                        one(Cell<1>());
+                        if (sg.n > 2) one(Cell<2>());
+                    }
                 }
-            }
-            cluster_arrive();
-            if (active) {
-                for (int cell = c_begin + warp; cell < last_row; cell += nwarp) {
-                    const uint4* r = recs + static_cast<size_t>(cell) * kCellRec;
-                    const uint4 h0 = ld_rec<kSmemRec>(r), h1 = ld_rec<kSmemRec>(r + 1), h2 = ld_rec<kSmemRec>(r + 2);
-                    sts_off(sm, h1.y + lane4,
-                            hidden_cell_rec(sm, h0, h1, h2, ld_rec5<kSmemRec>(r), s_th, rs, r0l.lo, a.rk, lc));
-                }
-            }
-            __syncthreads();
-            cluster_wait();
-            // the first cell row first (the previous band waits for its spins)
-            if (active) {
-                for (int cell = c_begin + warp; cell < first_row_end; cell += nwarp) {
-                    const uint4* r = recs + static_cast<size_t>(cell) * kCellRec;
-                    const uint4 v0 = ld_rec<kSmemRec>(r + 3);
-                    const U4 o = visible_cell_rec(sm, v0, ld_rec<kSmemRec>(r + 4), lane4, s_tv, rs, r0l.lo, a.rk, lc);
-                    sts_off(sm_prev, v0.x, o.x);
-                    sts_off(sm_prev, v0.x + 4u, o.y);
-                }
-            }
-            cluster_arrive();
-            if (active) {
-                for (int cell = first_row_end + warp; cell < c_end; cell += nwarp) {
-                    const uint4* r = recs + static_cast<size_t>(cell) * kCellRec;
-                    visible_cell_rec(sm, ld_rec<kSmemRec>(r + 3), ld_rec<kSmemRec>(r + 4), lane4, s_tv, rs, r0l.lo,
-                                     a.rk, lc);
-                }
-            }
-            __syncthreads();
-            cluster_wait();
-        } else {  // the whole word in one CTA
-        for (int cell = c_begin + warp; cell < c_end; cell += nwarp, rec += rstep) {
-            const uint4 h0 = ld_rec<kSmemRec>(rec), h1 = ld_rec<kSmemRec>(rec + 1), h2 = ld_rec<kSmemRec>(rec + 2);
-            const uint32_t h5 = kSmemRec ? reinterpret_cast<const uint32_t*>(rec + 5)[0]
-                                         : __ldg(reinterpret_cast<const uint32_t*>(rec + 5));
-            const uint32_t w = hidden_cell_rec(sm, h0, h1, h2, h5, s_th, rs, r0l.lo, a.rk, lc);
-            sts_off(sm, h1.y + lane4, w);
-            if (kCluster && nb > 1 && cell >= last_row) sts_off(sm_next, h1.y + lane4, w);
+            if (kCluster && ph == 0) cluster_arrive();
         }
-        body_sync<kCluster>();
-        rec = rec0;
-        for (int cell = c_begin + warp; cell < c_end; cell += nwarp, rec += rstep) {
-            const uint4 v0 = ld_rec<kSmemRec>(rec + 3), v1 = ld_rec<kSmemRec>(rec + 4);
-            const U4 o = visible_cell_rec(sm, v0, v1, lane4, s_tv, rs, r0l.lo, a.rk, lc);
-            if (kCluster && nb > 1 && cell < first_row_end) {
-                sts_off(sm_prev, v0.x, o.x);
-                sts_off(sm_prev, v0.x + 4u, o.y);
-            }
+        __syncthreads();
+        if (kCluster && nb > 1) cluster_wait();
+        // visible half-step; a band's first cell row first (the previous band waits for its spins)
+        const int vsplit = kCluster && nb > 1 ? u_begin + nseg : u_begin;
+        for (int ph = kCluster && nb > 1 ? 0 : 1; ph < 2; ++ph) {
+            const int ub = ph == 0 ? u_begin : vsplit, ue = ph == 0 ? vsplit : u_end;
+            if (!kCluster || active)
+                for (int u = ub + warp; u < ue; u += nwarp) {
+                    const Segment sg = segment(u);
+                    const int cell = sg.i * Wc + sg.j0;
+                    CellRecs<kMode> rec(rec_addr, a.crec, cell);
+                    const uint32_t po = pw_addr + 256u * static_cast<uint32_t>(cell) + 2u * lane4;
+                    const uint32_t wo = w_of(cell), wu = w_of(sg.i > 0 ? cell - Wc : cell + (W - 1) * Wc);
+                    uint32_t left = load_w(w_of(sg.j0 > 0 ? cell - 1 : cell + Wc - 1)), o = 0u;
+                    auto draw = [&](auto jc) {
+                        constexpr int j = decltype(jc)::value;
+                        if (kPaper) {
+                            uint2 vis;
+                            if (kRedraw) {
+                                const U4 q = visible_draw(rec.template get<kCellRec * j + 2>(), rs, r0l.lo, a.rk);
+                                vis = make_uint2(q.y, q.z);
+                            } else {
+                                vis = lds64<256 * j>(po);
+                            }
+                            return U4{vis.x << 16, vis.x, vis.y << 16, vis.y};
+                        }
+                        return visible_draw(rec.template get<kCellRec * j + 2>(), rs, r0l.lo, a.rk);
+                    };
+                    auto decide = [&](auto jc, const U4& q) {
+                        constexpr uint32_t off = kWCell * decltype(jc)::value;
+                        const uint32_t own = load_w(wo + off);
+                        o = visible_row_cell(merge_words(own, load_w(wu + off), left), q, tab4, o);
+                        left = own;
+                    };
+                    if (sg.n == 3) {  // the three calls side by side
+                        const U4 a0 = draw(Cell<0>()), a1 = draw(Cell<1>()), a2 = draw(Cell<2>());
+                        decide(Cell<0>(), a0);
+                        decide(Cell<1>(), a1);
+                        decide(Cell<2>(), a2);
+                    } else {
+                        const U4 a0 = draw(Cell<0>());
+                        decide(Cell<0>(), a0);
+                        if (sg.n > 1) decide(Cell<1>(), draw(Cell<1>()));
+                    }
+                    store_row(u, sg, o);
+                    if (kCluster && ph == 0) {  // the previous band reads this row as its row below
+                        *reinterpret_cast<uint16_t*>(sm_prev + (row_addr(u) + 2u - base)) = static_cast<uint16_t>(o);
+                        *reinterpret_cast<uint8_t*>(sm_prev + (row_addr(sg.left) + 1u - base)) =
+                            static_cast<uint8_t>((o >> (4u * static_cast<uint32_t>(sg.n) - 2u)) << 6);
+                    }
+                }
+            if (kCluster && ph == 0) cluster_arrive();
         }
-        body_sync<kCluster>();
-        }
+        __syncthreads();
+        if (kCluster && nb > 1) cluster_wait();
         const bool do_meas = every_meas.step();
         const bool do_swap = every_swap.step();
         if (do_meas || do_swap) {
             if (active) {
                 int anti0 = 0, anti1 = 0, pos = 0;
-                rec = rec0;
-                for (int cell = c_begin + warp; cell < c_end; cell += nwarp, rec += rstep)
-                    count_cell_rec(sm, ld_rec<kSmemRec>(rec), ld_rec<kSmemRec>(rec + 1), lane, anti0, anti1, pos);
+                for (int u = u_begin + warp; u < u_end; u += nwarp) {
+                    const Segment sg = segment(u);
+                    count_segment(lds32(row_addr(u)), lds32(row_addr(sg.below)), sg.n, anti0, anti1, pos);
+                }
                 atomicAdd(&cnt0[lane], anti0);
                 atomicAdd(&cnt0[32 + lane], anti1);
                 atomicAdd(&cnt0[64 + lane], pos);
             }
             body_sync<kCluster>();
-            if (band == 0 && warp == post_warp)
-                post_sweep_warp(a, s_cnt, s_sob, s_bos, lane, word, t, do_meas, do_swap, meas, s_acc);
-            if (do_meas) ++meas;
+            const bool post = band == 0 && warp == post_warp;
+            RungCounts rc{0, 0, 0};
+            if (post) {
+                rc = rung_counts(a, s_cnt, s_sob, lane);
+                if (do_swap) swap_rungs(a, rc, s_sob, s_bos, lane, word, t, s_u[lane]);
+            }
             // A swap round changes the permutation every warp reads next; a
             // measurement alone touches only warp post_warp's sums and the counts, which
             // the next measurement reaches after the next sweep's barriers.
             if (do_swap) {
                 body_sync<kCluster>();
-                if (active) lc.lb = 4u * static_cast<uint32_t>(bos0[lane]);
+                if (active) tab4 = tab + 4u * static_cast<uint32_t>(bos0[lane]);
+            }
+            if (do_meas) {
+                if (post) add_measurement(a, rc, lane, word, t, meas, s_acc);
+                ++meas;
             }
         }
-        if (every_sq.step()) {
-            accumulate_correlations_any(a, s_v, s_w, s_seg, s_segmask, warp, nwarp, lane);  // s_w: dead here
+        if (every_sq.step()) {  // the hidden words are dead here: their space holds the lattice
+            uint32_t* scratch = smem + cs.w;
+            const int L = g.L;
+            if (L <= 32) {  // one word per row and chain
+                for (int R = warp; R < L; R += nwarp) {
+                    uint32_t m = 0u;
+                    for (int j0 = 0, s = 0; j0 < Wc; j0 += uc, ++s) {
+                        const int n = min(uc, Wc - j0);
+                        // bits 0, 2 of a nibble: columns 1, 0 of row R
+                        const uint32_t x = lds32(row_addr((R >> 1) * nseg + s)) >> (17 - (R & 1));
+                        for (int j = 0; j < n; ++j) {
+                            const uint32_t c = x >> (4 * (n - 1 - j));
+                            m |= (((c >> 2) & 1u) | ((c & 1u) << 1)) << (2 * (j0 + j));
+                        }
+                    }
+                    scratch[R * 32 + lane] = m;
+                }
+                __syncthreads();
+                accumulate_correlations_rows(a, scratch, s_seg, s_segmask, warp, nwarp, lane);
+            } else {  // one word per site
+                for (int u = warp; u < W * nseg; u += nwarp) {
+                    const Segment sg = segment(u);
+                    const uint32_t v = transpose32(lds32(row_addr(u)) >> 16, lane);
+                    if (lane < 4 * sg.n) scratch[row_site(lane, sg.i, sg.j0, sg.n, g.Lc)] = v;
+                }
+                __syncthreads();
+                accumulate_correlations_sites(a, scratch, s_seg, s_segmask, warp, nwarp, lane);
+            }
             __syncthreads();
         }
     }
     if (kCluster) body_sync<true>();  // no rank reads another's shared memory after this
     if (!active) return;
     uint32_t* gv = a.v + static_cast<size_t>(word) * g.N;
-    const int s_begin = kCluster ? 2 * row0 * g.Lc : 0;  // own spin rows
-    const int s_end = kCluster ? min(2 * row1, g.L) * g.Lc : g.N;
-    for (int x = s_begin + static_cast<int>(threadIdx.x); x < s_end; x += blockDim.x) gv[x] = s_v[x];
+    for (int u = u_begin + warp; u < u_end; u += nwarp) {  // own rows
+        const Segment sg = segment(u);
+        const uint32_t v = transpose32(lds32(row_addr(u)) >> 16, lane);
+        if (lane < 4 * sg.n) gv[row_site(lane, sg.i, sg.j0, sg.n, g.Lc)] = v;
+    }
     if (band == 0 && warp == post_warp && a.swap_every > 0) a.sob[word * 32 + lane] = s_sob[lane];
     if (band == 0 && warp == post_warp && measuring) {
         for (int x = 0; x < kNSum; ++x) a.sums[static_cast<size_t>(chain) * kNSum + x] = s_acc[x * 32 + lane];
     }
 }
-
 
 }  // namespace canon
 }  // namespace crbm

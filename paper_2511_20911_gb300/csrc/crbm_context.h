@@ -28,6 +28,7 @@ struct crbm_ctx {
     std::vector<double> beta;
     std::vector<uint32_t> tables;  // [n_params][nTab]
     crbm::DeviceState d;
+    crbm::CanonLaunch plan;        // canonical SMEM sweep: launch choices for `warps`
     std::string err;
 };
 

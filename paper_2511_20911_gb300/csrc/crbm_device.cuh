@@ -137,6 +137,20 @@ __device__ __forceinline__ uint32_t bit_of(uint32_t word, int lane) { return (wo
 
 __device__ __forceinline__ uint32_t rotr(uint32_t x, uint32_t s) { return __funnelshift_r(x, x, s); }
 
+// 32 x 32 bit transpose across a warp: lane c returns the word whose bit l is
+// bit c of lane l's x (block swaps of 16, 8, 4, 2 and 1 rows and columns).
+__device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
+    constexpr uint32_t kLow[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        const int j = 16 >> i;
+        const uint32_t m = kLow[i];
+        const uint32_t y = __shfl_xor_sync(0xffffffffu, x, j);
+        x = (lane & j) ? ((x & ~m) | ((y >> j) & m)) : ((x & m) | ((y << j) & ~m));
+    }
+    return x;
+}
+
 // Release store of a progress counter in global memory.
 __device__ __forceinline__ void st_release(int* p, int v) {
     asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
@@ -200,12 +214,13 @@ __device__ __forceinline__ void claim_word(int* state, int nw, int n_chunks, uns
 // measurement, a swap round or a correlation sample is taken), started at
 // sweep t0, so that the sweep loop needs no integer division per sweep.
 // k <= 0: never.  step() answers for the current sweep and moves on to the
-// next; every thread calls it once per sweep.
+// next; every thread calls it once per sweep.  now() only answers.
 struct EveryCounter {
     int left, k;  // sweeps after the current one before the next hit (k <= 0: negative, never 0)
     __device__ __forceinline__ EveryCounter(uint32_t t0, int k_)
         : left(k_ > 0 ? static_cast<int>(static_cast<uint32_t>(k_) - 1u - t0 % static_cast<uint32_t>(k_)) : -1),
           k(k_) {}
+    __device__ __forceinline__ bool now() const { return left == 0; }
     __device__ __forceinline__ bool step() {
         const bool hit = left == 0;
         left = hit ? k - 1 : left - 1;
@@ -230,86 +245,92 @@ static __device__ __noinline__ void record_first_hit(int64_t* hit, const int32_t
     if (ht[1] < 0 && E <= ht[0]) ht[1] = static_cast<int64_t>(t) + 1;
 }
 
-// Post-sweep step of the SMEM kernels, run by one warp (the one that keeps
-// the running sums) after every warp has added its per-lane counts to s_cnt ([0..31] anti-aligned J filters, [32..63]
-// anti-aligned J' filters, [64..95] +1 spins; lane = replica slot).  Lane k
-// then stands for temperature rung k, held by slot s_sob[k] (the identity
-// without tempering):
-//  - measurement: rung k's (NJ, NJ', M) go to series row 32 word + k and are
-//    added to the running sums s_acc[x][k] (shared memory, so that they hold
-//    no registers through the sweep loop);
-//  - replica exchange (round m): pairs (k, k+1) with k = m (mod 2) swap rungs
-//    when E_k <= E_{k+1}, else when a Philox word (k, m, word, swap tag) is
-//    below the host-built threshold of nearbyint(2^32 exp((b_k - b_{k+1}) dE / 16)).
-__device__ __forceinline__ void post_sweep_warp(const SweepArgs& a, int* s_cnt, int* s_sob,
-                                                 int* s_bos, int lane, int word, uint32_t t,
-                                                 bool do_meas, bool do_swap, int64_t meas,
-                                                 int64_t* s_acc) {
+// Post-sweep step, run by one warp (the one that keeps the running sums) after
+// every warp has added its per-lane counts to s_cnt ([0..31] anti-aligned J
+// filters, [32..63] anti-aligned J' filters, [64..95] +1 spins; lane = replica
+// slot).  Lane k then stands for temperature rung k, held by slot s_sob[k] (the
+// identity without tempering): rung_counts, then swap_rungs (replica exchange),
+// whose new permutation the other warps wait for, then add_measurement.
+struct RungCounts {
+    int nJ, nP, M;
+};
+// Rung k's (NJ, NJ', M); clears the counts.
+__device__ __forceinline__ RungCounts rung_counts(const SweepArgs& a, int* s_cnt, const int* s_sob, int lane) {
     const Geometry& g = a.g;
-    const int nJr = g.n_real_bonds[0] - 2 * s_cnt[lane];
-    const int nPr = g.n_real_bonds[1] - 2 * s_cnt[32 + lane];
-    const int Mr = 2 * s_cnt[64 + lane] - g.N;
+    const int nJ = g.n_real_bonds[0] - 2 * s_cnt[lane];
+    const int nP = g.n_real_bonds[1] - 2 * s_cnt[32 + lane];
+    const int M = 2 * s_cnt[64 + lane] - g.N;
     s_cnt[lane] = 0;
     s_cnt[32 + lane] = 0;
     s_cnt[64 + lane] = 0;
+    const int slot = s_sob[lane];
+    return {__shfl_sync(0xffffffffu, nJ, slot), __shfl_sync(0xffffffffu, nP, slot), __shfl_sync(0xffffffffu, M, slot)};
+}
+
+// Measurement `meas`, after sweep t: rung k's counts go to series row 32 word + k
+// and are added to the running sums s_acc[x][k] (shared memory, so that they hold
+// no registers through the sweep loop).
+__device__ __forceinline__ void add_measurement(const SweepArgs& a, const RungCounts& c, int lane, int word, uint32_t t,
+                                                int64_t meas, int64_t* s_acc) {
+    const uint32_t row = static_cast<uint32_t>(word) * 32u + static_cast<uint32_t>(lane);
+    const int64_t nJ = c.nJ, nP = c.nP, M = c.M;
+    if (meas < a.series_len) {
+        int32_t* e = a.series + (static_cast<size_t>(meas) * a.n_chains_padded + row) * 3;
+        e[0] = c.nJ;
+        e[1] = c.nP;
+        e[2] = c.M;
+    }
+    int64_t* acc = s_acc + lane;
+    acc[0 * 32] += 1;
+    acc[1 * 32] += nJ;
+    acc[2 * 32] += nP;
+    acc[3 * 32] += M;
+    acc[4 * 32] += M < 0 ? -M : M;
+    acc[5 * 32] += nJ * nJ;
+    acc[6 * 32] += nP * nP;
+    acc[7 * 32] += M * M;
+    acc[8 * 32] += nJ * nP;
+    acc[9 * 32] += nJ * M;
+    acc[10 * 32] += nP * M;
+    if (a.hit) record_first_hit(a.hit, a.hit_q, row, nJ, nP, M, t);
+}
+
+// The uniform of rung k = lane in the exchange round after sweep t: a Philox
+// word (k, m, word, swap tag) of round m.  It depends on no state, so a caller
+// may draw it ahead of the counts.
+__device__ __forceinline__ uint32_t swap_uniform(const SweepArgs& a, int lane, int word, uint32_t t) {
+    const uint32_t m = (t + 1u) / static_cast<uint32_t>(a.swap_every) - 1u;
+    return philox(static_cast<uint32_t>(lane), m, static_cast<uint32_t>(word), kTagSwap, a.key0, a.key1).x;
+}
+
+// Replica exchange (round m): pairs (k, k+1) with k = m (mod 2) swap rungs when
+// E_k <= E_{k+1}, else when u is below the host-built threshold of nearbyint(2^32
+// exp((b_k - b_{k+1}) dE / 16)).
+__device__ __forceinline__ void swap_rungs(const SweepArgs& a, const RungCounts& c, int* s_sob, int* s_bos, int lane,
+                                           int word, uint32_t t, uint32_t u) {
     const int k = lane;
     const int slot = s_sob[k];
-    const int64_t nJ = __shfl_sync(0xffffffffu, nJr, slot);
-    const int64_t nP = __shfl_sync(0xffffffffu, nPr, slot);
-    const int64_t M = __shfl_sync(0xffffffffu, Mr, slot);
-    if (do_meas) {
-        const uint32_t row = static_cast<uint32_t>(word) * 32u + k;
-        if (meas < a.series_len) {
-            int32_t* e = a.series + (static_cast<size_t>(meas) * a.n_chains_padded + row) * 3;
-            e[0] = static_cast<int32_t>(nJ);
-            e[1] = static_cast<int32_t>(nP);
-            e[2] = static_cast<int32_t>(M);
-        }
-        int64_t* acc = s_acc + k;
-        acc[0 * 32] += 1;
-        acc[1 * 32] += nJ;
-        acc[2 * 32] += nP;
-        acc[3 * 32] += M;
-        acc[4 * 32] += M < 0 ? -M : M;
-        acc[5 * 32] += nJ * nJ;
-        acc[6 * 32] += nP * nP;
-        acc[7 * 32] += M * M;
-        acc[8 * 32] += nJ * nP;
-        acc[9 * 32] += nJ * M;
-        acc[10 * 32] += nP * M;
-        if (a.hit) record_first_hit(a.hit, a.hit_q, row, nJ, nP, M, t);
+    const int32_t* q = a.wq + 3 * word;
+    const long long E = static_cast<long long>(__ldg(q)) * c.nJ + static_cast<long long>(__ldg(q + 1)) * c.nP -
+                        static_cast<long long>(__ldg(q + 2)) * c.M;
+    const long long E1 = __shfl_down_sync(0xffffffffu, E, 1);
+    const uint32_t m = (t + 1u) / static_cast<uint32_t>(a.swap_every) - 1u;
+    bool accept = false;
+    if (k < 31 && (static_cast<uint32_t>(k) & 1u) == (m & 1u)) {
+        const long long D = E - E1;
+        const int idx = word * 32 + k;
+        accept = D <= 0 || (D < __ldg(a.swap_len + idx) && u < __ldg(a.swap_tab + __ldg(a.swap_off + idx) + D));
     }
-    if (do_swap) {
-        const int32_t* q = a.wq + 3 * word;
-        const long long E = static_cast<long long>(q[0]) * nJ + static_cast<long long>(q[1]) * nP -
-                            static_cast<long long>(q[2]) * M;
-        const long long E1 = __shfl_down_sync(0xffffffffu, E, 1);
-        const uint32_t m = (t + 1u) / static_cast<uint32_t>(a.swap_every) - 1u;
-        bool accept = false;
-        if (k < 31 && (static_cast<uint32_t>(k) & 1u) == (m & 1u)) {
-            const long long D = E - E1;
-            if (D <= 0) {
-                accept = true;
-            } else {
-                const int idx = word * 32 + k;
-                if (D < a.swap_len[idx]) {
-                    const U4 u = philox(static_cast<uint32_t>(k), m, static_cast<uint32_t>(word), kTagSwap,
-                                        a.key0, a.key1);
-                    accept = u.x < a.swap_tab[a.swap_off[idx] + D];
-                }
-            }
-        }
-        const uint32_t am = __ballot_sync(0xffffffffu, accept);
-        const int up = __shfl_down_sync(0xffffffffu, slot, 1);
-        const int dn = __shfl_up_sync(0xffffffffu, slot, 1);
-        int ns = slot;
-        if ((am >> k) & 1u)
-            ns = up;
-        else if (k > 0 && ((am >> (k - 1)) & 1u))
-            ns = dn;
-        s_sob[k] = ns;
-        s_bos[ns] = k;
-    }
+    const uint32_t am = __ballot_sync(0xffffffffu, accept);
+    const int up = __shfl_down_sync(0xffffffffu, slot, 1);
+    const int dn = __shfl_up_sync(0xffffffffu, slot, 1);
+    int ns = slot;
+    if ((am >> k) & 1u)
+        ns = up;
+    else if (k > 0 && ((am >> (k - 1)) & 1u))
+        ns = dn;
+    s_sob[k] = ns;
+    s_bos[ns] = k;
 }
 
 // Spin correlations of Sec. IV.B for the chains of each parameter-point
@@ -413,29 +434,20 @@ static __device__ __forceinline__ void accumulate_correlations_word(const SweepA
 }
 
 // The same correlations for a square lattice of even side kL <= 32, in
-// bit-transposed form: the lattice is first transposed so that lane l holds,
-// for every row R, the kL spins of chain l as a kL-bit mask (rows in
-// `scratch`, [kL][32] words of the caller's dead shared memory).  Work items
+// bit-transposed form: lane l holds, for every row R, the kL spins of chain l
+// as a kL-bit mask (rows in `scratch`, [kL][32] words).  Work items
 // are (dR, slice of rows R); in an item lane l counts, for every column offset
 // dC, the sites at which row R of chain l and row R + dR rotated by dC differ
 // (the rotation is one funnel shift of the row written twice side by side),
 // and the counts of a parameter point's chains are summed by one warp
-// reduction over the point's lane mask.  Every thread of the CTA calls it.
+// reduction over the point's lane mask.  The caller has filled `scratch`.
 template <int kL>
-static __device__ __forceinline__ void accumulate_correlations_bits(const SweepArgs& a, const uint32_t* s_v,
-                                                             uint32_t* scratch, const int* s_seg,
-                                                             const uint32_t* s_segmask, int warp, int nwarp,
-                                                             int lane) {
+static __device__ __forceinline__ void accumulate_correlations_bits(const SweepArgs& a, const uint32_t* scratch,
+                                                             const int* s_seg, const uint32_t* s_segmask, int warp,
+                                                             int nwarp, int lane) {
     static_assert(kL % 2 == 0 && kL >= 4 && kL <= 32, "even side up to 32");
     constexpr int N = kL * kL, n_dr = kL / 2 + 1;
     constexpr uint32_t kFull = kL == 32 ? 0xffffffffu : (1u << (kL % 32)) - 1u;
-    for (int R = warp; R < kL; R += nwarp) {
-        const uint32_t* row = s_v + R * kL;
-        uint32_t m = 0u;
-#pragma unroll
-        for (int C = 0; C < kL; ++C) m |= ((row[C] >> lane) & 1u) << C;
-        scratch[R * 32 + lane] = m;
-    }
     // this lane's parameter point: its lane mask, index and whether it reports
     const int nseg = s_seg[0];
     uint32_t smask = 1u << lane;
@@ -448,7 +460,6 @@ static __device__ __forceinline__ void accumulate_correlations_bits(const SweepA
     const bool leader = p >= 0 && (smask & ((1u << lane) - 1u)) == 0u;  // the point's lowest lane
     const long long n_pt = __popc(smask);
     unsigned long long* cp = reinterpret_cast<unsigned long long*>(a.corr) + static_cast<size_t>(p < 0 ? 0 : p) * N;
-    __syncthreads();
     const int slices = max(1, min(kL, (nwarp + n_dr - 1) / n_dr));
     const int n_items = n_dr * slices;
     for (int item = warp; item < n_items; item += nwarp) {
@@ -478,22 +489,25 @@ static __device__ __forceinline__ void accumulate_correlations_bits(const SweepA
     }
 }
 
-// Correlations of one word: the bit-transposed form for even square sides up
-// to 32 when the caller has scratch space, else the word-parallel one (one
-// call site in the sweep kernels, out of line: it runs every sq_every sweeps).
-static __device__ __noinline__ void accumulate_correlations_any(const SweepArgs& a, const uint32_t* s_v,
-                                                                   uint32_t* scratch, const int* s_seg,
-                                                                   const uint32_t* s_segmask, int warp, int nwarp,
-                                                                   int lane) {
-    switch (scratch ? a.g.L : 0) {
+// The bit-transposed form by side (out of line: it runs every sq_every sweeps).
+static __device__ __noinline__ void accumulate_correlations_rows(const SweepArgs& a, const uint32_t* scratch,
+                                                                 const int* s_seg, const uint32_t* s_segmask, int warp,
+                                                                 int nwarp, int lane) {
+    switch (a.g.L) {
 #define CRBM_CORR_BITS(k) \
-    case k: accumulate_correlations_bits<k>(a, s_v, scratch, s_seg, s_segmask, warp, nwarp, lane); return;
+    case k: accumulate_correlations_bits<k>(a, scratch, s_seg, s_segmask, warp, nwarp, lane); return;
         CRBM_CORR_BITS(4) CRBM_CORR_BITS(6) CRBM_CORR_BITS(8) CRBM_CORR_BITS(10) CRBM_CORR_BITS(12)
         CRBM_CORR_BITS(14) CRBM_CORR_BITS(16) CRBM_CORR_BITS(18) CRBM_CORR_BITS(20) CRBM_CORR_BITS(22)
         CRBM_CORR_BITS(24) CRBM_CORR_BITS(26) CRBM_CORR_BITS(28) CRBM_CORR_BITS(30) CRBM_CORR_BITS(32)
 #undef CRBM_CORR_BITS
-        default: accumulate_correlations_word(a, s_v, s_seg, s_segmask, warp, nwarp, lane);
     }
+}
+
+// The word-parallel form from one word per site, out of line too.
+static __device__ __noinline__ void accumulate_correlations_sites(const SweepArgs& a, const uint32_t* s_v,
+                                                                  const int* s_seg, const uint32_t* s_segmask,
+                                                                  int warp, int nwarp, int lane) {
+    accumulate_correlations_word(a, s_v, s_seg, s_segmask, warp, nwarp, lane);
 }
 
 }  // namespace dev

@@ -145,7 +145,7 @@ __device__ __forceinline__ void count_cell(const Geometry& g, const uint32_t* s_
 // writes v).  kPaper: CRBM_PRECISION_PAPER draws (see the cores).
 template <bool kPaper>
 __device__ __forceinline__ void sweep_generic_body(const SweepArgs& a, int word) {
-    extern __shared__ __align__(16) uint32_t smem[];
+    extern __shared__ __align__(128) uint32_t smem[];
     const Geometry& g = a.g;
     const GenericSmem gs = generic_smem(g);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
@@ -217,13 +217,24 @@ __device__ __forceinline__ void sweep_generic_body(const SweepArgs& a, int word)
             atomicAdd(&s_cnt[32 + lane], anti1);
             atomicAdd(&s_cnt[64 + lane], pos);
             __syncthreads();
-            if (warp == 0) post_sweep_warp(a, s_cnt, s_sob, s_bos, lane, word, t, do_meas, do_swap, meas, s_acc);
-            if (do_meas) ++meas;
-            __syncthreads();
-            if (do_swap) lb = 4u * static_cast<uint32_t>(s_bos[lane]);
+            RungCounts rc{0, 0, 0};
+            if (warp == 0) {
+                rc = rung_counts(a, s_cnt, s_sob, lane);
+                if (do_swap) swap_rungs(a, rc, s_sob, s_bos, lane, word, t, swap_uniform(a, lane, word, t));
+            }
+            // A swap round changes the permutation every warp reads next; a measurement alone touches only
+            // warp 0's sums and the counts, which the next one reaches after the next sweep's barriers.
+            if (do_swap) {
+                __syncthreads();
+                lb = 4u * static_cast<uint32_t>(s_bos[lane]);
+            }
+            if (do_meas) {
+                if (warp == 0) add_measurement(a, rc, lane, word, t, meas, s_acc);
+                ++meas;
+            }
         }
         if (every_sq.step()) {
-            accumulate_correlations_any(a, s_v, nullptr, s_seg, s_segmask, warp, nwarp, lane);
+            accumulate_correlations_sites(a, s_v, s_seg, s_segmask, warp, nwarp, lane);
             __syncthreads();
         }
     }

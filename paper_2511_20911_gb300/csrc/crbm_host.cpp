@@ -237,13 +237,26 @@ void free_device(DeviceState& d) {
     d = DeviceState{};
 }
 
-int default_warps(const Geometry& g) {
+// Warps per CTA of the SMEM sweeps.  Bit-plane and generic sweeps: about six
+// cells per warp, up to 16.  The canonical sweep, by whether every SM has two
+// words or more (us per sweep of 384 words with 4, 8, 12, 16 warps: L = 6 2.65
+// 2.81, L = 12 6.07 6.07 5.42 5.50, L = 18 11.5 10.6 11.0 11.4, L = 24 21.1 18.7 -
+// 18.5, L = 30 32.6 29.1 28.8 28.4; of 152 words with 8, 16, 32: L = 18 5.1 4.6
+// 4.7, L = 48 30.1 26.6 26.4, L = 64 74.4 50.2 47.6; L = 6, every sweep measured:
+// 1.29 with 9 warps, 1.20 with 12, one of them free to finish the measurements).
+int default_warps(const Geometry& g, int n_words) {
     if (const char* env = std::getenv("CRBM_WARPS")) {
         const int w = std::atoi(env);
         if (w >= 1 && w <= kMaxSweepWarps) return w;
     }
-    // about six cells per warp, up to 16 warps per CTA
-    return std::max(1, std::min(std::min(16, kMaxSweepWarps), (g.n_cells + 5) / 6));
+    if (!g.canonical || g.bitplane) return std::max(1, std::min(std::min(16, kMaxSweepWarps), (g.n_cells + 5) / 6));
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+        sms = 152;
+    if (n_words >= 2 * sms && g.n_cells <= 400)  // (larger ones hold one CTA per SM)
+        return std::min(kMaxSweepWarps, g.n_cells < 16 ? 4 : g.n_cells < 30 || (g.n_cells >= 50 && g.n_cells <= 144) ? 8 : 12);
+    return std::min(kMaxSweepWarps, g.n_cells < 8 ? 8 : g.n_cells <= 16 ? 12 : g.n_cells <= 600 ? 16 : 32);
 }
 
 }  // namespace
@@ -392,7 +405,7 @@ int crbm_create(crbm_ctx** out, const crbm_params* p) {
     ctx->series_len = p->series_len;
     ctx->sq_every = p->sq_every;
     ctx->stream = static_cast<cudaStream_t>(p->stream);
-    ctx->warps = default_warps(g);
+    ctx->warps = default_warps(g, ctx->n_words);
     for (int k = 0; k < 3; ++k) ctx->q[k].resize(p->n_params);
     ctx->q_odd.resize(p->n_params);
     ctx->beta.assign(p->beta, p->beta + p->n_params);
@@ -617,41 +630,23 @@ int crbm_create(crbm_ctx** out, const crbm_params* p) {
             o[2] = b[0] | (cell << 16) | (x << 28);
         }
     } else if (g.canonical && ctx->layout == CRBM_LAYOUT_SMEM) {
-        const int L = g.L, W = g.W, Lc = g.Lc, Wc = g.Wc;
         const uint32_t key0 = static_cast<uint32_t>(ctx->seed), key1 = static_cast<uint32_t>(ctx->seed >> 32);
         const uint32_t rk2 = key0 + 0x9E3779B9u, rk4 = key0 + 2u * 0x9E3779B9u;  // round keys 1, 2 (word 0)
-        const uint32_t vb = 4u * kCanonSmemV, wb = 4u * static_cast<uint32_t>(kCanonSmemV + g.N);
-        auto site = [&](int R, int C) { return vb + 4u * static_cast<uint32_t>((R % L) * Lc + C % Lc); };
-        auto hrow = [&](int i, int j) { return wb + 128u * static_cast<uint32_t>(i * Wc + j); };
         crec.assign(static_cast<size_t>(g.n_cells) * kCellRec * 4, 0u);
-        for (int i = 0; i < W; ++i)
-            for (int j = 0; j < Wc; ++j) {
-                uint32_t* o = &crec[static_cast<size_t>(i * Wc + j) * kCellRec * 4];
-                const uint64_t m = 0xD2511F53ull * static_cast<uint32_t>(i * Wc + j);
-                const uint32_t lo = static_cast<uint32_t>(m), hi = static_cast<uint32_t>(m >> 32) ^ key1;
-                uint32_t qh[4], ql[4];  // round-1 products of the calls with tags 0, 1, 2, visible
-                const uint32_t tags[4] = {0u, 1u, 2u, kTagVis};
-                for (int t = 0; t < 4; ++t) {
-                    const uint64_t p = 0xCD9E8D57ull * (hi ^ tags[t]);
-                    qh[t] = static_cast<uint32_t>(p >> 32) ^ rk2;
-                    ql[t] = static_cast<uint32_t>(p) ^ rk4;
-                }
-                const int R = 2 * i, C = 2 * j;
-                const uint32_t rec[kCellRec * 4] = {
-                    site(R, C),     site(R + 1, C), site(R + 2, C),        site(R, C + 2),
-                    site(R + 1, C + 2), hrow(i, j), lo,                    qh[2],
-                    qh[0],          ql[0],          qh[1],                 ql[1],
-                    site(R, C),     site(R + 1, C), hrow(i, j),            hrow((i + W - 1) % W, j),
-                    hrow(i, (j + Wc - 1) % Wc), lo, qh[3],                 ql[3],
-                    ql[2],          0u,             0u,                    0u};
-                std::copy(rec, rec + kCellRec * 4, o);
-                if (g.paper) {  // the cell's row of visible draws replaces Q2.hi and Qv.hi
-                    const uint32_t pw = 4u * static_cast<uint32_t>(canon_smem_pw_offset(g)) +
-                                        256u * static_cast<uint32_t>(i * Wc + j);
-                    o[7] = pw;
-                    o[18] = pw;
-                }
+        for (int c = 0; c < g.n_cells; ++c) {
+            const uint64_t m = 0xD2511F53ull * static_cast<uint32_t>(c);
+            const uint32_t lo = static_cast<uint32_t>(m), hi = static_cast<uint32_t>(m >> 32) ^ key1;
+            uint32_t qh[4], ql[4];  // round-1 products of the calls with tags 0, 1, 2, visible
+            const uint32_t tags[4] = {0u, 1u, 2u, g.paper ? 1u : kTagVis};
+            for (int t = 0; t < 4; ++t) {
+                const uint64_t p = 0xCD9E8D57ull * (hi ^ tags[t]);
+                qh[t] = static_cast<uint32_t>(p >> 32) ^ rk2;
+                ql[t] = static_cast<uint32_t>(p) ^ rk4;
             }
+            const uint32_t rec[kCellRec * 4] = {lo,    qh[0], ql[0], qh[1], ql[1], qh[2],
+                                                ql[2], 0u,    lo,    qh[3], ql[3], 0u};
+            std::copy(rec, rec + kCellRec * 4, &crec[static_cast<size_t>(c) * kCellRec * 4]);
+        }
     }
     // Per-cell records of the generic SMEM sweep (layout in crbm_internal.h).
     if (!g.canonical && ctx->layout == CRBM_LAYOUT_SMEM) {
@@ -809,13 +804,10 @@ int crbm_sweep(crbm_ctx* ctx, int64_t n_sweeps) {
         if (ctx->layout == CRBM_LAYOUT_STREAM) {
             e = launch_sweep_stream(a, ctx->stream, &ctx->launches);
         } else {
-            // canonical: persistent grid over (word, chunk) items, chunks of about
-            // 1/CRBM_CHUNKS_PER_WORD of the launch (at least 8 sweeps): short
-            // enough that the last round leaves few SMs idle, long enough that
-            // reloading a word's tables and state stays cheap
+            // canonical: persistent grid over (word, chunk of sweeps) items, the launcher picks the chunk
             const int chunk = std::max(8, (a.n_sweeps + CRBM_CHUNKS_PER_WORD - 1) / CRBM_CHUNKS_PER_WORD);
             e = ctx->g.bitplane    ? launch_sweep_bitplane(a, ctx->warps, chunk, ctx->d.sched, ctx->stream)
-                : ctx->g.canonical ? launch_sweep_canon_persistent(a, ctx->warps, chunk, ctx->d.sched, ctx->stream)
+                : ctx->g.canonical ? launch_sweep_canon_persistent(a, ctx->warps, ctx->d.sched, ctx->plan, ctx->stream)
                                    : launch_sweep_generic(a, ctx->warps, ctx->stream);
             ++ctx->launches;
         }

@@ -37,32 +37,20 @@ constexpr int kBpHidPlanes = 0, kBpVisPlanes = 192, kBpFlip = 512, kBpTab = 516;
 static_assert(kBpHidPlanes % 4 == 0 && kBpVisPlanes % 4 == 0 && kBpTab % 4 == 0 && (kNSum * 64) % 4 == 0,
               "the sweeps read four threshold planes with one 16-byte load");
 
-// Canonical fast-path tables per packed word: hidden [2 cls][4 idx][32 lanes]
-// then visible [4 spin positions][32 idx][32 lanes] (see crbm_canon.cu).
+// Canonical fast-path tables per packed word in HBM: hidden [2 cls][4 idx][32
+// lanes] then visible [4 spin positions][32 idx][32 lanes] (crbm_canon_core.cuh).
 constexpr int kCanonTh = 2 * 4 * 32;
 constexpr int kCanonTab = kCanonTh + 4 * 32 * 32;
-// Canonical SMEM-resident sweep: dynamic shared memory holds, in 32-bit
-// words, [kAccWords running sums][kCanonTab tables][N spins]
-// [n_cells x 32 per-lane hidden words][counters ...]; kCanonSmemV is the
-// offset of the spins.
-constexpr int kCanonSmemV = kAccWords + kCanonTab;
-// Per-cell records of that sweep, kCellRec uint4 per cell, built on the host
-// so that the cell loops do no index arithmetic.  Byte offsets are from the
-// start of dynamic shared memory; rc.lo = lo(M0 cell) is a round-0 Philox
-// word of the cell (M0, M1 the Philox multipliers).  Round 1 multiplies the
-// warp-uniform word rc.hi ^ tag = hi(M0 cell) ^ key1 ^ tag by M1, so that
-// product is built here too, per call tag t: Qt = (hi(M1 (rc.hi ^ t)) ^ rk2,
-// lo(M1 (rc.hi ^ t)) ^ rk4), with the round keys it is XORed with
-// (tags 0, 1, 2: hidden calls; v: the visible call):
-//   [0] spins (0,0) (1,0) (2,0) (0,2) of the 3x3 window (site (r,1) is (r,0) + 4)
-//   [1] spin (1,2), the cell's hidden row, rc.lo, Q2.hi
-//   [2] Q0.hi, Q0.lo, Q1.hi, Q1.lo
-//   [3] spins (0,0) (1,0) of the cell, hidden rows of the cell and of the cell above
-//   [4] hidden row of the cell to the left, rc.lo, Qv.hi, Qv.lo
-//   [5] Q2.lo, 0, 0, 0
-// In paper precision (two calls per cell) Q2 and Qv are not used: [1].w and
-// [4].z hold the byte offset of the cell's row of visible draws instead.
-constexpr int kCellRec = 6;
+// Per-cell records of the canonical SMEM sweep, kCellRec uint4 per cell, built
+// on the host: the warp-uniform Philox words of the cell's calls.  lo = lo(M0
+// cell) is a round-0 word (M0, M1 the Philox multipliers).  Round 1 multiplies
+// hi(M0 cell) ^ key1 ^ tag by M1, the same for every lane, so that product is
+// built here too, per call tag t, XORed with the round keys it meets:
+// Qt = (hi ^ rk2, lo ^ rk4)
+//   [0] lo, Q0.h, Q0.l, Q1.h   [1] Q1.l, Q2.h, Q2.l, 0   [2] lo, Qv.h, Qv.l, 0
+// (tags 0, 1, 2: hidden calls; v: the visible call -- in paper precision the
+// tag-1 call, whose words 1 and 2 carry the visible uniforms).
+constexpr int kCellRec = 3;
 // (class, second-endpoint flag) of the five filter slots of each spin
 // position (0,0), (0,1), (1,0), (1,1) in the canonical visible tables.
 constexpr int kCanonSlot[4][5][2] = {{{0, 0}, {0, 0}, {1, 0}, {0, 1}, {0, 1}},
@@ -94,20 +82,65 @@ struct Geometry {
     int bitplane;  // CRBM_RNG_BITPLANE: uniforms from bit-plane words shared by the 32 chains of a word
     int8_t r1[kMaxBonds], c1[kMaxBonds], r2[kMaxBonds], c2[kMaxBonds];
     uint8_t cls[kMaxBonds];
+    // canonical SMEM sweep: a row of cells is cut into n_seg segments of seg_cells cells (the last
+    // may be shorter), the unit of work of a warp; set per launch (canon_segments)
+    int seg_cells, n_seg;
 };
 
-// Word offset, after [kCanonSmemV][N][n_cells x 32][3 x 32 counters]
-// [33 segments][32 masks][32][32] replica tables rounded up to 16 bytes, of
-// the paper-precision visible draws: [n_cells][32 lanes] pairs of words, the
-// two Philox words of tag 1 that carry a cell's four 16-bit visible uniforms
-// (drawn in the hidden half-step, read in the visible one).  The records
-// follow them when the sweep copies the records into shared memory.
-__host__ __device__ inline size_t canon_smem_pw_offset(const Geometry& g) {
-    return (static_cast<size_t>(kCanonSmemV) + g.N + static_cast<size_t>(g.n_cells) * 32 + 96 + 33 + 32 + 64 + 3) &
-           ~static_cast<size_t>(3);
-}
-__host__ __device__ inline size_t canon_smem_rec_offset(const Geometry& g) {
-    return canon_smem_pw_offset(g) + (g.paper ? static_cast<size_t>(g.n_cells) * 64 : 0);
+// How a canonical SMEM sweep keeps a word's state (crbm_canon_body.cuh).
+//   kCanonRec     a 32-bit hidden word per cell and lane, the per-cell records in
+//                 shared memory
+//   kCanonPlain   the same, the records read through the read-only cache
+//   kCanonPacked  as kCanonPlain with 16-bit hidden words, expanded by a table, or,
+//                 in paper precision, the visible half-step drawing its call again
+//                 instead of keeping the words: lattices that fit no other way
+constexpr int kCanonRec = 0, kCanonPlain = 1, kCanonPacked = 2;
+constexpr int kMaxSegCells = 3;  // cells of a row segment, the unit of work of a warp (crbm_row_core.cuh)
+// Dynamic shared memory of that sweep, offsets in 32-bit words.  The tables lie
+// at shared address 16384 (the table loads merge their index into the address
+// by OR), dynamic shared memory starts at kReservedSmem in kernels without
+// static shared memory (checked by the launchers); the space below the tables
+// takes what fits of the other arrays, the rest follows the tables.
+constexpr int kReservedSmem = 1024;
+constexpr int kCanonTabWord = (16384 - kReservedSmem) / 4;
+constexpr int kCanonTabBytes = 40960;   // a word's tables (crbm_row_core.cuh) ...
+constexpr int kCanonAccByte = 21760;    // ... with room for the running sums inside
+struct CanonSmem {
+    int acc;      // [kNSum][32] running sums (int64)
+    int cnt;      // [3][32] measurement counters
+    int sob;      // [32] slot of each rung, then [32] rung of each slot
+    int segmask;  // [32]
+    int seg;      // [33]; [33], [34]: the persistent scheduler's word and chunk
+    int u;        // [32] uniforms of a swap round
+    int w;        // [n_cells][32] hidden words (kCanonPacked, exact precision: 16-bit)
+    int pw;       // [n_cells][32] pairs (paper precision unless kCanonPacked): visible draws
+    int rec;      // [n_cells][kCellRec * 4] (kCanonRec)
+    int rows;     // [W][n_seg][32] spins of a row segment of cells
+    int expand;   // [1024] 32-bit form of a 16-bit hidden word (kCanonPacked, exact precision)
+    int total;
+};
+__host__ __device__ inline CanonSmem canon_smem(const Geometry& g, int mode) {
+    CanonSmem s;
+    int low = 260, high = kCanonTabWord + kCanonTabBytes / 4;
+    auto place = [&](int words) {
+        int& at = low + words <= kCanonTabWord ? low : high;
+        const int r = at;
+        at += words;
+        return r;
+    };
+    s.acc = kCanonTabWord + kCanonAccByte / 4;
+    s.cnt = 0;
+    s.sob = 96;
+    s.segmask = 160;
+    s.seg = 192;
+    s.u = 228;
+    s.w = place(g.n_cells * (mode == kCanonPacked && !g.paper ? 16 : 32));
+    s.pw = place(g.paper && mode != kCanonPacked ? g.n_cells * 64 : 0);
+    s.rec = place(mode == kCanonRec ? g.n_cells * kCellRec * 4 : 0);
+    s.rows = place(g.W * g.n_seg * 32);
+    s.expand = place(mode == kCanonPacked && !g.paper ? 1024 : 0);
+    s.total = high;
+    return s;
 }
 
 // Generic SMEM-resident sweep (any filter list, odd L, open boundaries).
@@ -239,22 +272,30 @@ constexpr int kMaxBatch = 16;
 struct BatchArgs {
     const int4* items;    // per CTA: (descriptor or -1, word, band, bands)
     int n_desc;
-    int smem_rec;         // 1: canonical members stage their per-cell records in shared memory
+    int canon_mode;       // kCanonRec or, when a canonical member does not fit that way, kCanonPacked
     SweepArgs d[kMaxBatch];
 };
 
 // Kernel launchers (crbm_kernels.cu).  All return cudaGetLastError().
 size_t smem_bytes_generic(const Geometry& g);
+// Shared memory that decides which canonical lattices the SMEM layout takes
+// (with the spins one word per site): at most 227 KB.
 size_t smem_bytes_canon(const Geometry& g);
-// Whether the canonical persistent sweep keeps the per-cell records in shared
-// memory (when that does not lower the CTAs per SM), and its dynamic shared
-// memory with that choice.
-bool canon_smem_records(const Geometry& g);
-size_t smem_bytes_canon_launch(const Geometry& g);
+// Canonical SMEM sweep: cuts g's rows of cells into segments for CTAs of
+// `warps` warps, and picks the mode (kCanon*) with the least work per cell
+// that fits a CTA.  Returns the launch's dynamic shared memory.
+// bands > 1: for a band of cell rows of a word split over a cluster.
+size_t canon_plan(Geometry& g, int warps, int* mode, int bands = 1);
+// A launch's choices, kept by the context between calls of the same shape.
+struct CanonLaunch {
+    int warps = 0, device = -1;  // what they were made for
+    int mode = 0, seg_cells = 0, n_seg = 0, cta = 0, per_sm = 0, sms = 0;
+    size_t smem = 0;
+};
 cudaError_t launch_init(const Geometry& g, uint32_t* v, int n_words, uint32_t key0,
                         uint32_t key1, cudaStream_t st);
 cudaError_t launch_sweep_generic(const SweepArgs& a, int warps_per_cta, cudaStream_t st);
-cudaError_t launch_sweep_canon_persistent(const SweepArgs& a, int warps_per_cta, int chunk, int* sched,
+cudaError_t launch_sweep_canon_persistent(const SweepArgs& a, int warps_per_cta, int* sched, CanonLaunch& plan,
                                           cudaStream_t st);
 cudaError_t launch_sweep_stream(const SweepArgs& a, cudaStream_t st, int64_t* launches);
 // Bit-plane sweep (crbm_bitplane.cu): a persistent grid that claims (word,

@@ -45,20 +45,24 @@ std::string shape_key(const crbm_ctx* ctx) {
     return s;
 }
 
-// Shared memory of a batch member's body (bit-plane records from global memory).
-size_t member_smem(const crbm_ctx* ctx) {
-    return ctx->g.bitplane ? smem_bytes_bitplane(ctx->g, false)
-           : ctx->g.canonical ? smem_bytes_canon(ctx->g)
-                              : smem_bytes_generic(ctx->g);
+// Shared memory of a batch member's body on CTAs of `warps` warps (bit-plane
+// records from global memory; canonical members in mode `canon_mode`, a word
+// split into `bands`).
+size_t member_smem(const crbm_ctx* ctx, int warps, int canon_mode, int bands) {
+    if (ctx->g.bitplane) return smem_bytes_bitplane(ctx->g, false);
+    if (!ctx->g.canonical) return smem_bytes_generic(ctx->g);
+    Geometry g = ctx->g;
+    int mode = 0;
+    canon_plan(g, warps, &mode, bands);
+    return sizeof(uint32_t) * static_cast<size_t>(canon_smem(g, canon_mode).total);
 }
-
-int smem_ok(const crbm_ctx* ctx) { return member_smem(ctx) <= 227 * 1024; }
 
 cudaError_t launch_one(const SweepArgs& a, const crbm_ctx* ctx, int warps) {
     if (!ctx->g.canonical) return launch_sweep_generic(a, warps, ctx->stream);
     const int chunk = std::max(8, (a.n_sweeps + CRBM_CHUNKS_PER_WORD - 1) / CRBM_CHUNKS_PER_WORD);  // as crbm_sweep does
     if (ctx->g.bitplane) return launch_sweep_bitplane(a, warps, chunk, ctx->d.sched, ctx->stream);
-    return launch_sweep_canon_persistent(a, warps, chunk, ctx->d.sched, ctx->stream);
+    CanonLaunch plan;
+    return launch_sweep_canon_persistent(a, warps, ctx->d.sched, plan, ctx->stream);
 }
 
 }  // namespace
@@ -175,7 +179,7 @@ struct crbm_batch {
     std::vector<int64_t> staged;       // pinned-free staging for clock uploads
     int threads = 0;
     size_t smem = 0;
-    int smem_rec = 0;                  // canonical members stage their records in shared memory
+    int canon_mode = 0;                // canonical members' shared-memory form (kCanonRec or kCanonPacked)
     int modes = 0;                     // kBatchPaper | kBatchBitplane: member kinds present
     int cluster = 1;                   // CTAs per item (thread-block cluster)
     std::vector<int> bands;            // per member: CTAs its words are split over
@@ -187,6 +191,19 @@ struct crbm_batch {
 
 namespace {
 thread_local std::string g_batch_create_error;
+
+// CTAs of `threads` threads: the canonical members' records in shared memory
+// where every member then fits a CTA, else their packed form.
+void set_threads(crbm_batch* b, int threads) {
+    b->threads = threads;
+    for (const int mode : {kCanonRec, kCanonPacked}) {
+        b->canon_mode = mode;
+        b->smem = 0;
+        for (size_t c = 0; c < b->ctx.size(); ++c)
+            b->smem = std::max(b->smem, member_smem(b->ctx[c], threads / 32, mode, b->bands[c]));
+        if (b->smem <= 227 * 1024) return;
+    }
+}
 
 void batch_free(crbm_batch* b) {
     if (b->exec) cudaGraphExecDestroy(b->exec);
@@ -211,7 +228,7 @@ int crbm_batch_create(crbm_batch** out, crbm_ctx* const* ctxs, int32_t n_ctx) {
     int warps = 1;
     for (int c = 0; c < n_ctx; ++c) {
         crbm_ctx* x = ctxs[c];
-        if (!x || x->layout != CRBM_LAYOUT_SMEM || !smem_ok(x) || x->stream != ctxs[0]->stream ||
+        if (!x || x->layout != CRBM_LAYOUT_SMEM || x->stream != ctxs[0]->stream ||
             x->device != ctxs[0]->device || std::count(ctxs, ctxs + c, x)) {
             g_batch_create_error = "batch members must be distinct SMEM-layout contexts on one device and stream";
             delete b;
@@ -219,21 +236,11 @@ int crbm_batch_create(crbm_batch** out, crbm_ctx* const* ctxs, int32_t n_ctx) {
         }
         b->ctx.push_back(x);
         warps = std::max(warps, x->warps);
-        b->smem = std::max(b->smem, member_smem(x));
         if (x->g.paper) b->modes |= kBatchPaper;
         if (x->g.bitplane) b->modes |= kBatchBitplane;
     }
-    // stage the canonical members' per-cell records in shared memory when all of them fit
-    size_t with_rec = b->smem;
-    for (auto* x : b->ctx)
-        if (x->g.canonical && !x->g.bitplane)
-            with_rec = std::max(with_rec, sizeof(uint32_t) * canon_smem_rec_offset(x->g) +
-                                              sizeof(uint4) * static_cast<size_t>(x->g.n_cells) * kCellRec);
-    if (with_rec <= 227 * 1024) {
-        b->smem = with_rec;
-        b->smem_rec = 1;
-    }
-    b->threads = 32 * warps;
+    b->bands.assign(n_ctx, 1);
+    set_threads(b, 32 * warps);
     // Thread-block clusters of `cluster` CTAs (CRBM_BATCH_CLUSTER, default 8,
     // a power of two; 1 = none).  A canonical exact-precision, lane-uniform
     // member without correlations is
@@ -253,12 +260,13 @@ int crbm_batch_create(crbm_batch** out, crbm_ctx* const* ctxs, int32_t n_ctx) {
     int target = 16;
     for (auto* x : b->ctx)
         if (splittable(x)) target = std::max(target, x->g.n_cells / std::min(cluster, x->g.W));
-    for (auto* x : b->ctx) {
-        int nb = 1;
-        if (splittable(x))
-            while (nb < cluster && 2 * nb <= x->g.W && x->g.n_cells / nb > target) nb *= 2;
-        b->bands.push_back(nb);
-    }
+    for (int c = 0; c < n_ctx; ++c)
+        if (splittable(b->ctx[c])) {
+            const Geometry& g = b->ctx[c]->g;
+            int& nb = b->bands[c];
+            while (nb < cluster && 2 * nb <= g.W && g.n_cells / nb > target) nb *= 2;
+        }
+    set_threads(b, 32 * warps);  // (the bands cut their rows into other segments)
     if (*std::max_element(b->bands.begin(), b->bands.end()) == 1) cluster = 1;  // nothing to split
     // tasks: split words cluster by cluster (heaviest member first), then
     // whole words one per CTA (heaviest first), padded to whole clusters
@@ -350,11 +358,13 @@ int crbm_batch_sweep(crbm_batch* b, int64_t n_sweeps) {
         BatchArgs args{};
         args.items = b->items;
         args.n_desc = n;
-        args.smem_rec = b->smem_rec;
+        args.canon_mode = b->canon_mode;
         for (int c = 0; c < n; ++c) {
             args.d[c] = fill_sweep_args(b->ctx[c], static_cast<int>(n_sweeps));
             args.d[c].clock = b->clock + 2 * c;
             args.d[c].n_bands = b->bands[c];
+            int mode = 0;
+            if (args.d[c].g.canonical && !args.d[c].g.bitplane) canon_plan(args.d[c].g, b->threads / 32, &mode, b->bands[c]);
             b->hit_seen[c] = b->ctx[c]->d.hit;
         }
         cudaGraph_t graph = nullptr;
@@ -453,8 +463,8 @@ int crbm_batch_autotune(crbm_batch* b, int64_t probe_sweeps, int32_t* best_threa
     for (int w : cand) {
         if (e != cudaSuccess || rc != CRBM_OK) break;
         if (w > kMaxSweepWarps) continue;
-        if (b->cluster > 1 && batch_max_active_clusters(b->cluster, 32 * w, b->smem, b->modes) < 1) continue;
-        b->threads = 32 * w;
+        set_threads(b, 32 * w);
+        if (b->cluster > 1 && batch_max_active_clusters(b->cluster, b->threads, b->smem, b->modes) < 1) continue;
         drop_graph();
         rc = crbm_batch_sweep(b, std::max<int64_t>(1, probe_sweeps / 4));  // warm-up (and the graph)
         drop_graph();
@@ -473,7 +483,7 @@ int crbm_batch_autotune(crbm_batch* b, int64_t probe_sweeps, int32_t* best_threa
     }
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
-    b->threads = (rc == CRBM_OK && e == cudaSuccess) ? best : threads0;
+    set_threads(b, (rc == CRBM_OK && e == cudaSuccess) ? best : threads0);
     drop_graph();
     if (rc != CRBM_OK || e != cudaSuccess) {
         const int rr = restore();  // best effort: the members as they were

@@ -1,0 +1,53 @@
+"""The canonical SMEM sweep's row form (segments of one to three cells of a row
+of cells per word, crbm_row_core.cuh) against the oracle, bit for bit: rows cut
+into segments of every length, one segment per row (its own right neighbour), and
+the lattices whose hidden words or visible draws are kept in their smaller forms."""
+import numpy as np
+import pytest
+
+import paper_2511_20911_gb300 as crbm
+from paper_2511_20911_gb300 import workloads
+
+pytestmark = pytest.mark.gpu
+EXACT, PAPER = crbm.CRBM_PRECISION_EXACT, crbm.CRBM_PRECISION_PAPER
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    crbm.load_library()
+
+
+def check(orc, L, Lc, precision, n, splits, warps, monkeypatch):
+    monkeypatch.setenv("CRBM_WARPS", str(warps))
+    params = workloads.random_params(np.random.default_rng(L * 97 + Lc), 3)
+    cp = (np.arange(n) % 3).astype(np.int32)
+    s = crbm.Sampler(L, params, n, chain_param=cp, seed=L + Lc, L_cols=Lc, measure_every=1, precision=precision,
+                     layout=crbm.CRBM_LAYOUT_SMEM)
+    ids = np.arange(n, dtype=np.uint32)
+    spins = orc.init_spins((L, Lc), ids, L + Lc)
+    sums, t = None, 0
+    for k in splits:
+        s.sweep(k)
+        sums, _, _ = orc.run((L, Lc), params, cp, spins, L + Lc, t, k, 1, chain_ids=ids, periodic=(True, True), sums=sums,
+                             precision=precision)
+        t += k
+        assert np.array_equal(s.get_spins(), spins), f"spins after {t} sweeps"
+    assert np.array_equal(s.observables(), sums)
+
+
+# one segment per row (4, 6 columns), segments of 2 + 2, 3 + 2, 3 + 3 + 1 cells and of single cells (many warps)
+@pytest.mark.parametrize("precision", [EXACT, PAPER])
+@pytest.mark.parametrize("L,Lc,warps", [(4, 4, 1), (4, 6, 3), (6, 4, 9), (8, 8, 2), (8, 10, 4), (10, 14, 5), (14, 10, 32),
+                                        (30, 22, 8)])
+def test_segment_lengths(orc, L, Lc, warps, precision, monkeypatch):
+    check(orc, L, Lc, precision, 37, [1, 6], warps, monkeypatch)
+
+
+# records from global memory (64 x 64, 18 x 96: long rows), 16-bit hidden words (68, 76), visible draws made twice (38 x 52)
+@pytest.mark.parametrize("L,Lc,precision", [(64, 64, EXACT), (18, 96, EXACT), (68, 68, EXACT), (76, 76, EXACT),
+                                            (56, 96, EXACT), (38, 52, PAPER), (18, 96, PAPER)])
+def test_large_lattices(orc, L, Lc, precision, monkeypatch):
+    check(orc, L, Lc, precision, 33, [3], 16, monkeypatch)
