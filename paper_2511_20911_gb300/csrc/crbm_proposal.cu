@@ -41,8 +41,8 @@
 // with the exact beta, and accepted blocks flipped in place with atomic XOR
 // (the two halves of a word are separate items).
 //
-// Training runs one example per thread in fp32 (bf16-rounded weights and
-// activations), back-propagates the binary cross-entropy and updates with
+// Training (k_prop_train) runs on the CUDA cores in fp32 (bf16-rounded weights
+// and activations), back-propagates the binary cross-entropy and updates with
 // Adam.
 #include <algorithm>
 #include <cstring>
@@ -547,171 +547,411 @@ struct Example {
     float beta, h;            // bf16-rounded
 };
 
-// Draw examples from a context's chains: chain and block origin from Philox.
-__global__ void k_prop_extract(Geometry g, const uint32_t* v, const float* chain_bh, int n_chains,
-                               Example* ex, int n, uint32_t step, uint32_t k0, uint32_t k1) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n) return;
-    const int L = g.L;
-    const U4 r = philox(static_cast<uint32_t>(e), step, 0u, kTagExample, k0, k1);
-    const int c = static_cast<int>(r.x % static_cast<uint32_t>(n_chains));
-    const int bR = static_cast<int>(r.y % static_cast<uint32_t>(L)), bC = static_cast<int>(r.z % static_cast<uint32_t>(L));
-    Example& x = ex[e];
-    for (int pos = 0; pos < kP * kP; ++pos) {
+// One example from a spin lookup, by one warp.
+template <typename Spin>
+__device__ __forceinline__ void fill_example(Example& x, int L, int bR, int bC, float beta, float h, int lane, Spin spin_at) {
+    for (int pos = lane; pos < kP * kP; pos += 32) {
         const int R = (bR - 3 + pos / kP + 2 * L) % L, C = (bC - 3 + pos % kP + 2 * L) % L;
         const bool in = ((R - bR + L) % L) < kK && ((C - bC + L) % L) < kK;
-        const int sp = ((v[static_cast<size_t>(c >> 5) * g.N + R * L + C] >> (c & 31)) & 1u) ? 1 : -1;
-        x.spin[pos] = in ? 0 : static_cast<int8_t>(sp);
+        x.spin[pos] = in ? static_cast<int8_t>(0) : spin_at(R, C);
         x.inside[pos] = in ? 1 : 0;
     }
-    for (int s = 0; s < kK * kK; ++s) {
-        const int R = (bR + s / kK) % L, C = (bC + s % kK) % L;
-        x.target[s] = ((v[static_cast<size_t>(c >> 5) * g.N + R * L + C] >> (c & 31)) & 1u) ? 1 : -1;
+    if (lane < kK * kK) x.target[lane] = spin_at((bR + lane / kK) % L, (bC + lane % kK) % L);
+    if (lane == 0) {
+        x.pr = static_cast<uint8_t>((bR + 1) & 1);  // parity of row bR - 3 (L even)
+        x.pc = static_cast<uint8_t>((bC + 1) & 1);
+        x.beta = beta;
+        x.h = h;
     }
-    x.pr = static_cast<uint8_t>((bR + 1) & 1);  // parity of row bR - 3 (L even)
-    x.pc = static_cast<uint8_t>((bC + 1) & 1);
-    x.beta = chain_bh[4 * c];
-    x.h = chain_bh[4 * c + 1];
+}
+
+// Draw examples from a context's chains: chain and block origin from Philox;
+// one warp per example (38 us for 4096 examples with one thread each, 4 now).
+__global__ void k_prop_extract(Geometry g, const uint32_t* v, const float* chain_bh, int n_chains,
+                               Example* ex, int n, uint32_t step, uint32_t k0, uint32_t k1) {
+    const int e = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (e >= n) return;
+    const U4 r = philox(static_cast<uint32_t>(e), step, 0u, kTagExample, k0, k1);
+    const int c = static_cast<int>(r.x % static_cast<uint32_t>(n_chains));
+    const uint32_t* vw = v + static_cast<size_t>(c >> 5) * g.N;
+    fill_example(ex[e], g.L, static_cast<int>(r.y % static_cast<uint32_t>(g.L)),
+                 static_cast<int>(r.z % static_cast<uint32_t>(g.L)), chain_bh[4 * c], chain_bh[4 * c + 1], lane,
+                 [&](int R, int C) { return static_cast<int8_t>(((vw[R * g.L + C] >> (c & 31)) & 1u) ? 1 : -1); });
+}
+
+// The same for given configurations [n][L*L], block origins [n][2] and (beta, h) [n][2].
+__global__ void k_prop_gather(const int8_t* spins, int L, const int32_t* origins, const float* beta_h, Example* ex, int n) {
+    const int e = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (e >= n) return;
+    const int8_t* v = spins + static_cast<size_t>(e) * L * L;
+    fill_example(ex[e], L, ((origins[2 * e] % L) + L) % L, ((origins[2 * e + 1] % L) + L) % L, beta_h[2 * e],
+                 beta_h[2 * e + 1], lane, [&](int R, int C) { return v[R * L + C]; });
 }
 
 __device__ __forceinline__ float bf16r(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 
 // Forward + backward of the mean binary cross-entropy in fp32 on
 // bf16-rounded weights and activations (the roundings pass gradients straight
-// through).  A CTA takes kTrainEx examples in turn, with the weights, its
-// gradient sums and one example's activations and deltas in shared memory;
-// within an example a thread takes output positions (forward, deltas) or
-// parameters (weight gradients), so every gradient sum has one owner thread
-// and the CTA adds its sums to grad with one atomic per parameter.  grad and
-// loss accumulate.
-constexpr int kTrainEx = 16, kTrainThreads = 128;
-__global__ void __launch_bounds__(kTrainThreads) k_prop_train(const float* __restrict__ w, const Example* ex, int n,
-                                                              float* grad, float* loss) {
-    __shared__ float sW[kNP], sG[kNP];
-    __shared__ float s_in[6][kP * kP], s_a1[16][kS1 * kS1], s_a2[16][kS2 * kS2];
-    __shared__ float s_d1[16][kS1 * kS1], s_d2[16][kS2 * kS2], s_dl[kK * kK];
-    __shared__ float s_loss;
-    const int tid = threadIdx.x;
-    for (int i = tid; i < kNP; i += kTrainThreads) {
-        sW[i] = w[i];
-        sG[i] = 0.f;
+// through).  A persistent CTA per SM of kTrainSlots slots of 64 threads, which
+// share the weights; a slot takes examples in turn, one at a time, its
+// activations and deltas in shared memory and its gradient sums in registers
+// over all its examples (added up per CTA at the end, then one atomic per
+// parameter and CTA).  grad and loss accumulate (the loss in 64 bits: 1216 slots
+// add to it).
+// What bounds it: 0.37 M multiply-adds per example on the FP32 pipe (38 us for
+// 4096 examples at its peak).  With a thread per output or per parameter every
+// multiply-add took two shared-memory loads (773 us); here a thread holds a tile
+// of 12 to 36 outputs, so that a 16-byte load of weights and one of activations
+// feed 4 to 12 of them.  The forward sums keep their order (channel, then tap),
+// so that the bf16 roundings are the same.
+constexpr int kTrainSlots = 8, kTrainThreads = 64 * kTrainSlots;
+// Shared memory, floats.  Weights: W1 and W2 as [channel, tap][16 outputs], W2
+// as [output, tap][16 channels], W3.  Slot: inputs [6][100]; a1 [16][68] (68: rows
+// of eight channels on distinct banks); a2 [16][37], later d1 [16][68]; d2 with a
+// border of two zeros [10 rows][11][20] (channels last, strides so that eight
+// rows' 16-byte loads are on distinct banks); the logits' deltas with the same
+// border [8][8]; two partial logits [2][16].
+constexpr int tW1 = 0, tB1 = tW1 + 54 * 16, tW2 = tB1 + 16, tB2 = tW2 + 144 * 16, tW2b = tB2 + 16, tW3 = tW2b + 144 * 16,
+              tSlot = tW3 + 148;
+constexpr int kA1S = 68, kA2S = 37, kD2P = 20, kD2R = 11 * kD2P;
+constexpr int uIn = 0, uA1 = uIn + 600, uD1 = uA1 + 16 * kA1S, uD2 = uD1 + 16 * kA1S, uDl = uD2 + 10 * kD2R, uLg = uDl + 64,
+              kSlotFloats = uLg + 32;
+constexpr int kTrainSmem = 4 * (tSlot + kTrainSlots * kSlotFloats);
+static_assert(tSlot % 4 == 0 && kSlotFloats % 4 == 0 && uA1 % 4 == 0 && uD1 % 4 == 0 && uD2 % 4 == 0 && tW2 % 4 == 0 &&
+                  tW2b % 4 == 0 && kTrainSmem <= 227 * 1024 && kNP <= kTrainSlots * kSlotFloats,
+              "16-byte loads; the gradient sums of a CTA reuse the slots");
+
+__device__ __forceinline__ void slot_sync(int slot) { asm volatile("bar.sync %0, 64;" ::"r"(1 + slot) : "memory"); }
+
+__global__ void __launch_bounds__(kTrainThreads, 1) k_prop_train(const float* __restrict__ w, const Example* ex, int n,
+                                                                 float* grad, double* loss) {
+    extern __shared__ __align__(16) float sm[];
+    const int slot = threadIdx.x >> 6, tid = threadIdx.x & 63, wid = tid >> 5, lane = tid & 31;
+    float* S = sm + tSlot + slot * kSlotFloats;
+    float* sIn = S + uIn;
+    float* sA1 = S + uA1;
+    float* sA2 = S + uD1;
+    float* sD1 = S + uD1;
+    float* sD2 = S + uD2;
+    float* sDl = S + uDl;
+    float* sLg = S + uLg;
+    for (int i = threadIdx.x; i < 54 * 16; i += kTrainThreads) sm[tW1 + i] = w[oW1 + (i & 15) * 54 + (i >> 4)];
+    for (int i = threadIdx.x; i < 144 * 16; i += kTrainThreads) {
+        sm[tW2 + i] = w[oW2 + (i & 15) * 144 + (i >> 4)];
+        const int o = i / 144, t = (i >> 4) % 9, c = i & 15;  // [o][t][c]
+        sm[tW2b + i] = w[oW2 + (o * 16 + c) * 9 + t];
     }
-    if (tid == 0) s_loss = 0.f;
+    for (int i = threadIdx.x; i < 16; i += kTrainThreads) {
+        sm[tB1 + i] = w[oB1 + i];
+        sm[tB2 + i] = w[oB2 + i];
+    }
+    for (int i = threadIdx.x; i < 145; i += kTrainThreads) sm[tW3 + i] = w[oW3 + i];
+    for (int i = tid; i < kSlotFloats - uD2; i += 64) S[uD2 + i] = 0.f;  // the borders stay zero
+    __syncthreads();
     const float inv = 1.f / (static_cast<float>(n) * kK * kK);
-    const int e_end = min(n, (blockIdx.x + 1) * kTrainEx);
-    for (int e = blockIdx.x * kTrainEx; e < e_end; ++e) {
-        const Example& x = ex[e];
-        __syncthreads();  // the previous example's buffers are free
-        for (int pos = tid; pos < kP * kP; pos += kTrainThreads) {
-            s_in[0][pos] = x.spin[pos];
-            s_in[1][pos] = x.inside[pos];
-            s_in[2][pos] = static_cast<float>((x.pr + pos / kP) & 1);
-            s_in[3][pos] = static_cast<float>((x.pc + pos % kP) & 1);
-            s_in[4][pos] = x.beta;
-            s_in[5][pos] = x.h;
+    const int cg = lane >> 3, r8 = lane & 7;     // tiles of layer 1 and d1: channels 4 cg .. + 3, row r8, columns 4 wid .. + 3
+    const int c16 = tid & 15, q4 = tid >> 4;     // the small layers: channel, quarter
+    const int cW2 = 8 * wid + r8, ogW2 = cg;     // tile of W2's gradient: outputs 4 ogW2 .. + 3, channel cW2, nine taps
+    float g2[4][9], g1s[9], g1m[9], g1r[3], g1c[3], g3[3];
+#pragma unroll
+    for (int t = 0; t < 9; ++t) {
+        g1s[t] = g1m[t] = 0.f;
+#pragma unroll
+        for (int o = 0; o < 4; ++o) g2[o][t] = 0.f;
+    }
+#pragma unroll
+    for (int t = 0; t < 3; ++t) g1r[t] = g1c[t] = g3[t] = 0.f;
+    float g1beta = 0.f, g1h = 0.f, gb1 = 0.f, gb2 = 0.f, gb3 = 0.f, lsum = 0.f;
+
+    // the next example's bytes are fetched while this one is worked on
+    const int step = kTrainSlots * gridDim.x;
+    int e = slot * gridDim.x + blockIdx.x;
+    int8_t n_spin[2] = {0, 0}, n_target = 0;
+    uint8_t n_in[2] = {0, 0}, n_pr = 0, n_pc = 0;
+    float n_beta = 0.f, n_h = 0.f;
+    auto fetch = [&](int k) {
+        const Example& x = ex[k];
+        n_spin[0] = x.spin[tid];
+        n_in[0] = x.inside[tid];
+        if (tid < kP * kP - 64) {
+            n_spin[1] = x.spin[64 + tid];
+            n_in[1] = x.inside[64 + tid];
         }
-        __syncthreads();
-        for (int i = tid; i < 16 * kS1 * kS1; i += kTrainThreads) {  // layer 1
-            const int o = i / (kS1 * kS1), p = i % (kS1 * kS1), y = p / kS1, xx = p % kS1;
-            float acc = sW[oB1 + o];
+        n_target = x.target[c16];
+        n_pr = x.pr;
+        n_pc = x.pc;
+        n_beta = x.beta;
+        n_h = x.h;
+    };
+    if (e < n) fetch(e);
+    for (; e < n; e += step) {
+        const int pr = n_pr, pc = n_pc, target = n_target;
+        const float beta = n_beta, h = n_h;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int pos = tid + 64 * k;
+            if (pos < kP * kP) {
+                sIn[pos] = n_spin[k];
+                sIn[100 + pos] = n_in[k];
+                sIn[200 + pos] = static_cast<float>((pr + pos / kP) & 1);
+                sIn[300 + pos] = static_cast<float>((pc + pos % kP) & 1);
+                sIn[400 + pos] = beta;
+                sIn[500 + pos] = h;
+            }
+        }
+        slot_sync(slot);
+        if (e + step < n) fetch(e + step);
+        {  // layer 1: 4 channels x 4 columns
+            float acc[4][4];
+            const float4 b = *reinterpret_cast<const float4*>(sm + tB1 + 4 * cg);
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                acc[0][x] = b.x;
+                acc[1][x] = b.y;
+                acc[2][x] = b.z;
+                acc[3][x] = b.w;
+            }
+#pragma unroll 1
             for (int c = 0; c < 6; ++c)
 #pragma unroll
-                for (int t = 0; t < 9; ++t) acc += sW[oW1 + (o * 6 + c) * 9 + t] * s_in[c][(y + t / 3) * kP + xx + t % 3];
-            s_a1[o][p] = bf16r(fmaxf(acc, 0.f));
+                for (int ty = 0; ty < 3; ++ty) {
+                    const float2* in = reinterpret_cast<const float2*>(sIn + c * 100 + (r8 + ty) * kP + 4 * wid);
+                    const float2 i0 = in[0], i1 = in[1], i2 = in[2];
+                    const float v[6] = {i0.x, i0.y, i1.x, i1.y, i2.x, i2.y};
+#pragma unroll
+                    for (int tx = 0; tx < 3; ++tx) {
+                        const float4 k = *reinterpret_cast<const float4*>(sm + tW1 + (c * 9 + ty * 3 + tx) * 16 + 4 * cg);
+#pragma unroll
+                        for (int x = 0; x < 4; ++x) {
+                            acc[0][x] += k.x * v[x + tx];
+                            acc[1][x] += k.y * v[x + tx];
+                            acc[2][x] += k.z * v[x + tx];
+                            acc[3][x] += k.w * v[x + tx];
+                        }
+                    }
+                }
+#pragma unroll
+            for (int o = 0; o < 4; ++o)
+                *reinterpret_cast<float4*>(sA1 + (4 * cg + o) * kA1S + r8 * kS1 + 4 * wid) =
+                    make_float4(bf16r(fmaxf(acc[o][0], 0.f)), bf16r(fmaxf(acc[o][1], 0.f)), bf16r(fmaxf(acc[o][2], 0.f)),
+                                bf16r(fmaxf(acc[o][3], 0.f)));
         }
-        __syncthreads();
-        for (int i = tid; i < 16 * kS2 * kS2; i += kTrainThreads) {  // layer 2
-            const int o = i / (kS2 * kS2), p = i % (kS2 * kS2), y = p / kS2, xx = p % kS2;
-            float acc = sW[oB2 + o];
+        slot_sync(slot);
+        if (tid < 48) {  // layer 2: 2 channels x a row of 6
+            const int og = tid & 7, y = tid >> 3;
+            const float2 b = *reinterpret_cast<const float2*>(sm + tB2 + 2 * og);
+            float acc[2][6];
+#pragma unroll
+            for (int x = 0; x < 6; ++x) {
+                acc[0][x] = b.x;
+                acc[1][x] = b.y;
+            }
+#pragma unroll 2
             for (int c = 0; c < 16; ++c)
 #pragma unroll
-                for (int t = 0; t < 9; ++t) acc += sW[oW2 + (o * 16 + c) * 9 + t] * s_a1[c][(y + t / 3) * kS1 + xx + t % 3];
-            s_a2[o][p] = bf16r(fmaxf(acc, 0.f));
-        }
-        __syncthreads();
-        if (tid < 32) {  // layer 3 and the loss: lanes 0 .. 15 take the block sites
-            float l = 0.f;
-            if (tid < kK * kK) {
-                const int y = tid / kK, xx = tid % kK;
-                float acc = sW[oB3];
-                for (int c = 0; c < 16; ++c)
+                for (int ty = 0; ty < 3; ++ty) {
+                    const float4* in = reinterpret_cast<const float4*>(sA1 + c * kA1S + (y + ty) * kS1);
+                    const float4 i0 = in[0], i1 = in[1];
+                    const float v[8] = {i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, i1.z, i1.w};
 #pragma unroll
-                    for (int t = 0; t < 9; ++t) acc += sW[oW3 + c * 9 + t] * s_a2[c][(y + t / 3) * kS2 + xx + t % 3];
-                const float yv = x.target[tid] > 0 ? 1.f : 0.f;
-                l = (acc > 0.f ? acc + log1pf(__expf(-acc)) : log1pf(__expf(acc))) - yv * acc;
-                s_dl[tid] = (1.f / (1.f + __expf(-acc)) - yv) * inv;
+                    for (int tx = 0; tx < 3; ++tx) {
+                        const float2 k = *reinterpret_cast<const float2*>(sm + tW2 + (c * 9 + ty * 3 + tx) * 16 + 2 * og);
+#pragma unroll
+                        for (int x = 0; x < 6; ++x) {
+                            acc[0][x] += k.x * v[x + tx];
+                            acc[1][x] += k.y * v[x + tx];
+                        }
+                    }
+                }
+#pragma unroll
+            for (int o = 0; o < 2; ++o)
+#pragma unroll
+                for (int x = 0; x < 6; ++x) sA2[(2 * og + o) * kA2S + y * kS2 + x] = bf16r(fmaxf(acc[o][x], 0.f));
+        }
+        slot_sync(slot);
+        {  // layer 3: block site c16, channels 4 q4 .. + 3; then the loss and the logits' deltas
+            float acc = 0.f;
+            const int y = c16 / kK, x = c16 % kK;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int t = 0; t < 9; ++t)
+                    acc += sm[tW3 + (4 * q4 + k) * 9 + t] * sA2[(4 * q4 + k) * kA2S + (y + t / 3) * kS2 + x + t % 3];
+            acc += __shfl_xor_sync(0xffffffffu, acc, 16);
+            if (lane < 16) sLg[16 * wid + lane] = acc;
+        }
+        slot_sync(slot);
+        if (tid < kK * kK) {
+            const float z = sm[tW3 + 144] + (sLg[tid] + sLg[16 + tid]);
+            const float yv = target > 0 ? 1.f : 0.f;
+            lsum += (z > 0.f ? z + log1pf(__expf(-z)) : log1pf(__expf(z))) - yv * z;
+            const float d = (1.f / (1.f + __expf(-z)) - yv) * inv;
+            sDl[(tid / kK + 2) * 8 + tid % kK + 2] = d;
+            gb3 += d;
+        }
+        slot_sync(slot);
+        {  // layer 3's weight gradients, the deltas of layer 2's outputs (zero where ReLU was off)
+            const float* a2 = sA2 + c16 * kA2S;
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const int t = q4 + 4 * j;
+                if (t < 9) {
+                    const int ty = t / 3, tx = t % 3;
+                    float g = 0.f;
+#pragma unroll
+                    for (int p = 0; p < kK * kK; ++p)
+                        g += sDl[(p / kK + 2) * 8 + p % kK + 2] * a2[(p / kK + ty) * kS2 + p % kK + tx];
+                    g3[j] += g;
+                }
             }
+            float w3[9];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-            if (tid == 0) s_loss += l;
-        }
-        __syncthreads();
-        // layer 3: weight gradients and the deltas of layer 2's outputs (zero where ReLU was off)
-        for (int i = tid; i < 16 * 9; i += kTrainThreads) {
-            const int c = i / 9, t = i % 9;
-            float g = 0.f;
+            for (int t = 0; t < 9; ++t) w3[t] = sm[tW3 + c16 * 9 + t];
 #pragma unroll
-            for (int p = 0; p < kK * kK; ++p) g += s_dl[p] * s_a2[c][(p / kK + t / 3) * kS2 + p % kK + t % 3];
-            sG[oW3 + i] += g;
-        }
-        if (tid == 0) {
-            float g = 0.f;
-            for (int p = 0; p < kK * kK; ++p) g += s_dl[p];
-            sG[oB3] += g;
-        }
-        for (int i = tid; i < 16 * kS2 * kS2; i += kTrainThreads) {
-            const int c = i / (kS2 * kS2), q = i % (kS2 * kS2), qy = q / kS2, qx = q % kS2;
-            float d = 0.f;
+            for (int k = 0; k < 9; ++k) {
+                const int q = 9 * q4 + k, qy = q / kS2, qx = q % kS2;
+                float d = 0.f;
 #pragma unroll
-            for (int t = 0; t < 9; ++t) {
-                const int py = qy - t / 3, px = qx - t % 3;
-                if (py >= 0 && py < kK && px >= 0 && px < kK) d += s_dl[py * kK + px] * sW[oW3 + c * 9 + t];
+                for (int t = 0; t < 9; ++t) d += sDl[(qy - t / 3 + 2) * 8 + qx - t % 3 + 2] * w3[t];
+                d = a2[q] > 0.f ? d : 0.f;
+                sD2[(qy + 2) * kD2R + (qx + 2) * kD2P + c16] = d;
+                gb2 += d;
             }
-            s_d2[c][q] = s_a2[c][q] > 0.f ? d : 0.f;
         }
-        __syncthreads();
-        // layer 2: weight and bias gradients, the deltas of layer 1's outputs
-        for (int i = tid; i < 16 * 16 * 9; i += kTrainThreads) {
-            const int o = i / 144, c = (i / 9) % 16, t = i % 9;
-            float g = 0.f;
-#pragma unroll 4
-            for (int p = 0; p < kS2 * kS2; ++p) g += s_d2[o][p] * s_a1[c][(p / kS2 + t / 3) * kS1 + p % kS2 + t % 3];
-            sG[oW2 + i] += g;
-        }
-        if (tid < 16) {
-            float g = 0.f;
-            for (int p = 0; p < kS2 * kS2; ++p) g += s_d2[tid][p];
-            sG[oB2 + tid] += g;
-        }
-        for (int i = tid; i < 16 * kS1 * kS1; i += kTrainThreads) {
-            const int c = i / (kS1 * kS1), q = i % (kS1 * kS1), qy = q / kS1, qx = q % kS1;
-            float d = 0.f;
+        slot_sync(slot);
+        {  // layer 2's weight gradients: 4 outputs x 9 taps of channel cW2
+            const float* a1 = sA1 + cW2 * kA1S;
+#pragma unroll 1
+            for (int y = 0; y < kS2; ++y) {
+                float v[3][kS1];
 #pragma unroll
-            for (int t = 0; t < 9; ++t) {
-                const int py = qy - t / 3, px = qx - t % 3;
-                if (py >= 0 && py < kS2 && px >= 0 && px < kS2)
-                    for (int o = 0; o < 16; ++o) d += s_d2[o][py * kS2 + px] * sW[oW2 + (o * 16 + c) * 9 + t];
+                for (int ty = 0; ty < 3; ++ty) {
+                    const float4 v0 = *reinterpret_cast<const float4*>(a1 + (y + ty) * kS1),
+                                 v1 = *reinterpret_cast<const float4*>(a1 + (y + ty) * kS1 + 4);
+                    v[ty][0] = v0.x, v[ty][1] = v0.y, v[ty][2] = v0.z, v[ty][3] = v0.w;
+                    v[ty][4] = v1.x, v[ty][5] = v1.y, v[ty][6] = v1.z, v[ty][7] = v1.w;
+                }
+#pragma unroll
+                for (int x = 0; x < kS2; ++x) {
+                    const float4 d = *reinterpret_cast<const float4*>(sD2 + (y + 2) * kD2R + (x + 2) * kD2P + 4 * ogW2);
+#pragma unroll
+                    for (int t = 0; t < 9; ++t) {
+                        const float a = v[t / 3][x + t % 3];
+                        g2[0][t] += d.x * a;
+                        g2[1][t] += d.y * a;
+                        g2[2][t] += d.z * a;
+                        g2[3][t] += d.w * a;
+                    }
+                }
             }
-            s_d1[c][q] = s_a1[c][q] > 0.f ? d : 0.f;
         }
-        __syncthreads();
-        // layer 1: weight and bias gradients
-        for (int i = tid; i < 16 * 6 * 9; i += kTrainThreads) {
-            const int o = i / 54, c = (i / 9) % 6, t = i % 9;
-            float g = 0.f;
-#pragma unroll 4
-            for (int p = 0; p < kS1 * kS1; ++p) g += s_d1[o][p] * s_in[c][(p / kS1 + t / 3) * kP + p % kS1 + t % 3];
-            sG[oW1 + i] += g;
+        {  // the deltas of layer 1's outputs: 4 channels x 4 columns of row r8 (over a2, dead since the last barrier)
+            float acc[4][4];
+#pragma unroll
+            for (int o = 0; o < 4; ++o)
+#pragma unroll
+                for (int x = 0; x < 4; ++x) acc[o][x] = 0.f;
+#pragma unroll 1
+            for (int og = 0; og < 4; ++og)
+#pragma unroll 1
+                for (int ty = 0; ty < 3; ++ty) {
+                    const float* d2 = sD2 + (r8 - ty + 2) * kD2R + 4 * wid * kD2P + 4 * og;
+                    float v[6][4];
+#pragma unroll
+                    for (int k = 0; k < 6; ++k) {
+                        const float4 d = *reinterpret_cast<const float4*>(d2 + k * kD2P);
+                        v[k][0] = d.x, v[k][1] = d.y, v[k][2] = d.z, v[k][3] = d.w;
+                    }
+#pragma unroll
+                    for (int o = 0; o < 4; ++o)
+#pragma unroll
+                        for (int tx = 0; tx < 3; ++tx) {
+                            const float4 k = *reinterpret_cast<const float4*>(sm + tW2b + ((4 * og + o) * 9 + ty * 3 + tx) * 16 + 4 * cg);
+#pragma unroll
+                            for (int x = 0; x < 4; ++x) {
+                                acc[0][x] += k.x * v[x - tx + 2][o];
+                                acc[1][x] += k.y * v[x - tx + 2][o];
+                                acc[2][x] += k.z * v[x - tx + 2][o];
+                                acc[3][x] += k.w * v[x - tx + 2][o];
+                            }
+                        }
+                }
+#pragma unroll
+            for (int o = 0; o < 4; ++o) {
+                const int i = (4 * cg + o) * kA1S + r8 * kS1 + 4 * wid;
+                const float4 a = *reinterpret_cast<const float4*>(sA1 + i);
+                *reinterpret_cast<float4*>(sD1 + i) =
+                    make_float4(a.x > 0.f ? acc[o][0] : 0.f, a.y > 0.f ? acc[o][1] : 0.f, a.z > 0.f ? acc[o][2] : 0.f,
+                                a.w > 0.f ? acc[o][3] : 0.f);
+            }
         }
-        if (tid < 16) {
-            float g = 0.f;
-            for (int p = 0; p < kS1 * kS1; ++p) g += s_d1[tid][p];
-            sG[oB1 + tid] += g;
+        slot_sync(slot);
+        // layer 1's weight gradients: output c16, rows 2 q4 and 2 q4 + 1.  The parity planes are constant
+        // along a row or column and the beta and h planes everywhere: sums of the deltas.
+#pragma unroll 1
+        for (int row = 2 * q4; row < 2 * q4 + 2; ++row) {
+            const float4 d0 = *reinterpret_cast<const float4*>(sD1 + c16 * kA1S + row * kS1),
+                         d1 = *reinterpret_cast<const float4*>(sD1 + c16 * kA1S + row * kS1 + 4);
+            const float d[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
+#pragma unroll
+            for (int ty = 0; ty < 3; ++ty) {
+                const float2* in = reinterpret_cast<const float2*>(sIn + (row + ty) * kP);
+                float v[kP], m[kP];
+#pragma unroll
+                for (int k = 0; k < kP / 2; ++k) {
+                    const float2 i = in[k], j = in[50 + k];
+                    v[2 * k] = i.x, v[2 * k + 1] = i.y;
+                    m[2 * k] = j.x, m[2 * k + 1] = j.y;
+                }
+#pragma unroll
+                for (int tx = 0; tx < 3; ++tx)
+#pragma unroll
+                    for (int x = 0; x < kS1; ++x) {
+                        g1s[ty * 3 + tx] += d[x] * v[x + tx];
+                        g1m[ty * 3 + tx] += d[x] * m[x + tx];
+                    }
+            }
+            const float even = (d[0] + d[2]) + (d[4] + d[6]), odd = (d[1] + d[3]) + (d[5] + d[7]), all = even + odd;
+#pragma unroll
+            for (int t = 0; t < 3; ++t) {
+                g1r[t] += ((pr + row + t) & 1) ? all : 0.f;
+                g1c[t] += ((pc + t) & 1) ? even : odd;
+            }
+            g1beta += beta * all;
+            g1h += h * all;
+            gb1 += all;
         }
+        slot_sync(slot);  // the slot's buffers are free
+    }
+    // the CTA's sums, in the slots' space, then one atomic per parameter
+    __syncthreads();
+    float* G = sm + tSlot;
+    for (int i = threadIdx.x; i < kNP; i += kTrainThreads) G[i] = 0.f;
+    __syncthreads();
+#pragma unroll
+    for (int t = 0; t < 9; ++t) {
+#pragma unroll
+        for (int o = 0; o < 4; ++o) atomicAdd(&G[oW2 + ((4 * ogW2 + o) * 16 + cW2) * 9 + t], g2[o][t]);
+        atomicAdd(&G[oW1 + (c16 * 6 + 0) * 9 + t], g1s[t]);
+        atomicAdd(&G[oW1 + (c16 * 6 + 1) * 9 + t], g1m[t]);
+        atomicAdd(&G[oW1 + (c16 * 6 + 2) * 9 + t], g1r[t / 3]);
+        atomicAdd(&G[oW1 + (c16 * 6 + 3) * 9 + t], g1c[t % 3]);
+        atomicAdd(&G[oW1 + (c16 * 6 + 4) * 9 + t], g1beta);
+        atomicAdd(&G[oW1 + (c16 * 6 + 5) * 9 + t], g1h);
+    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+        if (q4 + 4 * j < 9) atomicAdd(&G[oW3 + c16 * 9 + q4 + 4 * j], g3[j]);
+    atomicAdd(&G[oB1 + c16], gb1);
+    atomicAdd(&G[oB2 + c16], gb2);
+    if (tid < kK * kK) {
+        atomicAdd(&G[oB3], gb3);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xFFFFu, lsum, o);
+        if (tid == 0 && lsum != 0.f) atomicAdd(loss, static_cast<double>(lsum) / (static_cast<double>(n) * kK * kK));
     }
     __syncthreads();
-    for (int i = tid; i < kNP; i += kTrainThreads) atomicAdd(&grad[i], sG[i]);
-    if (tid == 0) atomicAdd(loss, s_loss * inv);
+    for (int i = threadIdx.x; i < kNP; i += kTrainThreads) atomicAdd(&grad[i], G[i]);
 }
 
 // Adam (Kingma & Ba) on the fp32 master weights; also refreshes the
@@ -809,13 +1049,16 @@ struct crbm_proposal {
     float* m = nullptr;      // Adam moments
     float* v2 = nullptr;
     float* grad = nullptr;
-    float* loss = nullptr;
+    double* loss = nullptr;  // [kLossCap], a training step each
     uint16_t* bmat = nullptr;  // tensor-core B operands (bf16)
     float* bias = nullptr;     // b2, b3
     float* c1 = nullptr;     // folded layer-1 constants
     unsigned long long* stats = nullptr;
     crbm::Example* ex = nullptr;
     int ex_cap = 0;
+    char* raw = nullptr;     // crbm_proposal_loss_grad: the given spins, origins, beta and h
+    size_t raw_cap = 0;
+    int train_sms = 0, train_dev = -1;  // SM count of the device the training kernel was set up on
     int64_t adam_t = 0;
     uint64_t seed = 0;
     int pass_sms = 0, pass_dev = -1;  // SM count of the device the pass kernel was set up on
@@ -919,6 +1162,41 @@ int ensure_examples(crbm_proposal* p, int n) {
     return CRBM_OK;
 }
 
+constexpr int kLossCap = 1024;  // steps whose losses stay on the device before they are read back
+
+int ensure_raw(crbm_proposal* p, size_t bytes) {
+    if (bytes <= p->raw_cap) return CRBM_OK;
+    cudaFree(p->raw);
+    p->raw = nullptr;
+    p->raw_cap = 0;
+    if (cudaMalloc(reinterpret_cast<void**>(&p->raw), bytes) != cudaSuccess) {
+        p->raw = nullptr;
+        cudaGetLastError();  // not sticky: clear it for later launch checks
+        return prop_fail(CRBM_ENOMEM, "examples");
+    }
+    p->raw_cap = bytes;
+    return CRBM_OK;
+}
+
+// Loss and gradient of the n examples in p->ex, added to *loss and p->grad.
+cudaError_t launch_train(crbm_proposal* p, int n, double* loss, cudaStream_t st) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess && (p->train_sms == 0 || p->train_dev != dev)) {
+        int sms = 0;
+        e = cudaFuncSetAttribute(crbm::k_prop_train, cudaFuncAttributeMaxDynamicSharedMemorySize, crbm::kTrainSmem);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e == cudaSuccess) {
+            p->train_sms = sms;
+            p->train_dev = dev;
+        }
+    }
+    if (e != cudaSuccess) return e;
+    crbm::k_prop_train<<<std::min(n, p->train_sms), crbm::kTrainThreads, crbm::kTrainSmem, st>>>(p->wb, p->ex, n, p->grad,
+                                                                                              loss);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_pass(crbm_ctx* ctx, crbm_proposal* p, crbm::PassRecord* rec) {
     const int L = ctx->g.L;
     const int nb1 = std::max(1, L / 8);
@@ -972,7 +1250,7 @@ int crbm_proposal_create(crbm_proposal** out, int32_t block, uint64_t seed) {
     float** bufs[] = {&p->w, &p->wb, &p->m, &p->v2, &p->grad};
     for (float** b : bufs)
         if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(b), kNP * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&p->loss), sizeof(float));
+    if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&p->loss), kLossCap * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&p->bmat), crbm::kBElems * sizeof(uint16_t));
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&p->bias), 33 * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&p->c1), crbm::kC1 * sizeof(float));
@@ -1003,7 +1281,7 @@ int crbm_proposal_create(crbm_proposal** out, int32_t block, uint64_t seed) {
 
 void crbm_proposal_destroy(crbm_proposal* p) {
     if (!p) return;
-    void* b[] = {p->w, p->wb, p->m, p->v2, p->grad, p->loss, p->bmat, p->bias, p->c1, p->stats, p->ex};
+    void* b[] = {p->w, p->wb, p->m, p->v2, p->grad, p->loss, p->bmat, p->bias, p->c1, p->stats, p->ex, p->raw};
     for (void* x : b)
         if (x) cudaFree(x);
     delete p;
@@ -1033,35 +1311,25 @@ int crbm_proposal_loss_grad(crbm_proposal* p, const int8_t* spins, int32_t L, co
         return prop_fail(CRBM_EINVAL, "bad arguments");
     int rc = ensure_examples(p, n);
     if (rc) return rc;
-    std::vector<Example> ex(n);
-    for (int e = 0; e < n; ++e) {
-        const int8_t* v = spins + static_cast<size_t>(e) * L * L;
-        const int bR = ((origins[2 * e] % L) + L) % L, bC = ((origins[2 * e + 1] % L) + L) % L;
-        Example& x = ex[e];
-        std::memset(&x, 0, sizeof(x));
-        for (int pos = 0; pos < crbm::kP * crbm::kP; ++pos) {
-            const int R = (bR - 3 + pos / crbm::kP + 2 * L) % L, C = (bC - 3 + pos % crbm::kP + 2 * L) % L;
-            const bool in = ((R - bR + L) % L) < crbm::kK && ((C - bC + L) % L) < crbm::kK;
-            x.spin[pos] = in ? 0 : v[R * L + C];
-            x.inside[pos] = in ? 1 : 0;
-        }
-        for (int s = 0; s < crbm::kK * crbm::kK; ++s)
-            x.target[s] = v[((bR + s / crbm::kK) % L) * L + (bC + s % crbm::kK) % L];
-        x.pr = static_cast<uint8_t>((bR + 1) & 1);
-        x.pc = static_cast<uint8_t>((bC + 1) & 1);
-        x.beta = beta_h[2 * e];
-        x.h = beta_h[2 * e + 1];
-    }
-    cudaError_t e = cudaMemcpy(p->ex, ex.data(), n * sizeof(Example), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(p->grad, 0, kNP * 4);
-    if (e == cudaSuccess) e = cudaMemset(p->loss, 0, 4);
+    const size_t b_spins = static_cast<size_t>(n) * L * L, off_o = (b_spins + 15) & ~static_cast<size_t>(15);
+    rc = ensure_raw(p, off_o + 16 * static_cast<size_t>(n));
+    if (rc) return rc;
+    int32_t* d_origins = reinterpret_cast<int32_t*>(p->raw + off_o);
+    float* d_bh = reinterpret_cast<float*>(d_origins + 2 * static_cast<size_t>(n));
+    cudaError_t e = cudaMemcpy(p->raw, spins, b_spins, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(d_origins, origins, 8 * static_cast<size_t>(n), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(d_bh, beta_h, 8 * static_cast<size_t>(n), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemsetAsync(p->grad, 0, kNP * 4, nullptr);
+    if (e == cudaSuccess) e = cudaMemsetAsync(p->loss, 0, sizeof(double), nullptr);
     if (e == cudaSuccess) {
-        crbm::k_prop_train<<<(n + crbm::kTrainEx - 1) / crbm::kTrainEx, crbm::kTrainThreads>>>(p->wb, p->ex, n,
-                                                                                              p->grad, p->loss);
+        crbm::k_prop_gather<<<(n + 3) / 4, 128>>>(reinterpret_cast<const int8_t*>(p->raw), L, d_origins, d_bh, p->ex, n);
         e = cudaGetLastError();
     }
+    if (e == cudaSuccess) e = launch_train(p, n, p->loss, nullptr);
     if (e == cudaSuccess) e = cudaMemcpy(grad, p->grad, kNP * 4, cudaMemcpyDeviceToHost);
-    if (e == cudaSuccess) e = cudaMemcpy(loss, p->loss, 4, cudaMemcpyDeviceToHost);
+    double sum = 0.0;
+    if (e == cudaSuccess) e = cudaMemcpy(&sum, p->loss, sizeof(sum), cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess) *loss = static_cast<float>(sum);
     return e == cudaSuccess ? CRBM_OK : prop_fail(CRBM_ECUDA, cudaGetErrorString(e));
 }
 
@@ -1076,18 +1344,14 @@ int crbm_proposal_train(crbm_proposal* p, crbm_ctx* ctx, int32_t steps, int32_t 
     cudaStream_t st = ctx->stream;
     for (int s = 0; s < steps; ++s) {
         if (sweeps_between > 0 && (rc = crbm_sweep(ctx, sweeps_between))) return prop_fail(rc, crbm_last_error(ctx));
-        cudaError_t e = cudaSuccess;
-        crbm::k_prop_extract<<<(batch + 127) / 128, 128, 0, st>>>(
+        double* step_loss = p->loss + s % kLossCap;  // read back kLossCap steps at a time
+        crbm::k_prop_extract<<<(batch + 3) / 4, 128, 0, st>>>(
             ctx->g, ctx->d.v, ctx->d.chain_bh, ctx->n_chains, p->ex, batch,
             static_cast<uint32_t>(p->adam_t), static_cast<uint32_t>(p->seed), static_cast<uint32_t>(p->seed >> 32));
-        e = cudaGetLastError();
+        cudaError_t e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaMemsetAsync(p->grad, 0, kNP * 4, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(p->loss, 0, 4, st);
-        if (e == cudaSuccess) {
-            crbm::k_prop_train<<<(batch + crbm::kTrainEx - 1) / crbm::kTrainEx, crbm::kTrainThreads, 0, st>>>(
-                p->wb, p->ex, batch, p->grad, p->loss);
-            e = cudaGetLastError();
-        }
+        if (e == cudaSuccess && s % kLossCap == 0) e = cudaMemsetAsync(p->loss, 0, kLossCap * sizeof(double), st);
+        if (e == cudaSuccess) e = launch_train(p, batch, step_loss, st);
         ++p->adam_t;
         const float b1 = 0.9f, b2 = 0.999f;
         const float c1 = 1.f - std::pow(b1, static_cast<float>(p->adam_t));
@@ -1097,9 +1361,12 @@ int crbm_proposal_train(crbm_proposal* p, crbm_ctx* ctx, int32_t steps, int32_t 
                                                                   b1, b2, 1e-8f, c1, c2);
             e = cudaGetLastError();
         }
-        if (e == cudaSuccess && losses) {
-            e = cudaMemcpyAsync(&losses[s], p->loss, 4, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess && losses && (s % kLossCap == kLossCap - 1 || s == steps - 1)) {
+            const int s0 = s - s % kLossCap;
+            double sums[kLossCap];
+            e = cudaMemcpyAsync(sums, p->loss, sizeof(double) * static_cast<size_t>(s - s0 + 1), cudaMemcpyDeviceToHost, st);
             if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+            for (int k = s0; e == cudaSuccess && k <= s; ++k) losses[k] = static_cast<float>(sums[k - s0]);
         }
         if (e != cudaSuccess) return prop_fail(CRBM_ECUDA, std::string("train: ") + cudaGetErrorString(e));
     }
