@@ -34,9 +34,11 @@ __global__ void __launch_bounds__(kMaxThreads, 1) k_sweep_batch(const __grid_con
     const uint32_t t0 = static_cast<uint32_t>(a.clock[0]);
     if (!a.g.canonical) {
         if ((kModes & kBatchPaper) && a.g.paper)
-            generic::sweep_generic_body<true>(a, task.y);
+            generic::sweep_generic_body<true, 0>(a, task.y);
+        else if (a.g.nb == 10)
+            generic::sweep_generic_body<false, 10>(a, task.y);
         else
-            generic::sweep_generic_body<false>(a, task.y);
+            generic::sweep_generic_body<false, 0>(a, task.y);
     } else if ((kModes & kBatchBitplane) && a.g.bitplane) {  // whole words; node records from global memory
         const uint32_t* hrec = reinterpret_cast<const uint32_t*>(a.crec);
         const uint32_t* vrec = hrec + static_cast<size_t>(a.g.n_cells) * bp::kBpNodes;

@@ -147,8 +147,8 @@ int pick_chunk(int n_sweeps, int n_words, int grid) {
 
 // The segments' length.  Warp w takes segments w, w + warps, ... of a half-step
 // and runs on SM sub-partition w % 4, so the half-step takes about what the
-// fullest sub-partition has to issue (its segments, each a fifth of a cell on top
-// of its cells), and a CTA alone on its SM also what its fullest warp has.
+// fullest sub-partition has to issue (its segments, each half a cell on top of its
+// cells), and a CTA alone on its SM also what its fullest warp has.
 size_t canon_plan(Geometry& g, int warps, int* mode, int bands) {
     constexpr size_t kCtaMax = 227 * 1024;
     auto bytes = [&](int m) { return sizeof(uint32_t) * static_cast<size_t>(canon_smem(g, m).total); };
@@ -174,7 +174,7 @@ size_t canon_plan(Geometry& g, int warps, int* mode, int bands) {
             most = std::max(most, c);
         }
         fullest += most;
-        const double cost = (fullest + rounds) * (g.seg_cells + 0.2);
+        const double cost = (fullest + rounds) * (g.seg_cells + 0.5);
         if (nseg == min_seg || (cost < best_cost && bytes(*mode) <= kCtaMax)) {
             best = nseg;
             best_cost = cost;

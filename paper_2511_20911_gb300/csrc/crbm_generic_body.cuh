@@ -28,6 +28,16 @@ __device__ __forceinline__ uint32_t or_if_less(uint32_t w, uint32_t q, uint32_t 
     return w;
 }
 
+// The threshold of filter record e: the lane's bits of its two endpoint words
+// rotated to address bits 7 and 8 and selected bitwise (four ALU instructions:
+// these, with the wide products, bound the sweep).
+__device__ __forceinline__ uint32_t filter_threshold(const char* sm, const uint4& e, uint32_t rot0, uint32_t rot1,
+                                                     uint32_t lb) {
+    const uint32_t a = rotr(lds32(sm, e.x), rot0), b = rotr(lds32(sm, e.y), rot1);
+    const uint32_t i = (a & 0x80u) | (b & ~0x80u);
+    return lds32(sm, e.z + ((i & 0x180u) | lb));
+}
+
 // Generic hidden half-step of one cell (Eq. 9): filter k of the cell reads
 // its two endpoint words (the zero word for a zero-padded endpoint, whose
 // pad pattern selects table rows that give it no weight), moves the lane's
@@ -41,39 +51,39 @@ __device__ __forceinline__ uint32_t or_if_less(uint32_t w, uint32_t q, uint32_t 
 // ten filters): filter k < 8 takes half k & 1 of word k >> 1 of tag 0, filters
 // 8 and 9 the halves of word 0 of tag 1, each compared as the upper half of a
 // 32-bit word against the 16-bit threshold in the table entry's upper half.
-template <bool kPaper>
+// kNb: the number of filters, or 0 (g.nb).  With ten known filters their records
+// are loaded at fixed offsets and no filter is tested for (a third of the ALU
+// instructions of a cell were these tests and addresses).
+template <bool kPaper, int kNb>
 __device__ __forceinline__ void hidden_cell_generic(const Geometry& g, char* sm, const uint4* __restrict__ rh,
                                                     uint32_t hw_byte, int cell, const Round1Sweep& rs, uint32_t Y,
-                                                    const uint32_t (&rk)[20], uint32_t lm, uint32_t rot0,
-                                                    uint32_t rot1, uint32_t lb, int lane) {
+                                                    const uint32_t (&rk)[20], uint32_t rot0, uint32_t rot1,
+                                                    uint32_t lb, int lane) {
     const Round0Cell rc = round0_cell(static_cast<uint32_t>(cell), rk[1]);
     const Round2Cell r2 = round2_cell(rs.hik ^ rc.b);
-    const uint4* r = rh + static_cast<size_t>(cell) * g.nb;
+    const int nb = kNb ? kNb : g.nb, n_calls = kNb ? (kNb + 3) / 4 : g.n_calls;
+    const uint4* r = rh + static_cast<size_t>(cell) * nb;
     uint32_t h = 0u;
     if (kPaper) {
         const U4 q0 = philox_from_round2(Y, rs, r2, rc.a, rk);
-        const U4 q1 = g.nb > 8 ? philox_from_round2(Y, rs, r2, rc.a ^ 1u, rk) : U4{0u, 0u, 0u, 0u};
+        const U4 q1 = nb > 8 ? philox_from_round2(Y, rs, r2, rc.a ^ 1u, rk) : U4{0u, 0u, 0u, 0u};
 #pragma unroll
         for (int k = 0; k < 10; ++k) {
-            if (k < g.nb) {
+            if (k < nb) {
                 const uint32_t word = k < 8 ? pick(q0, k >> 1) : q1.x;
-                const uint4 e = __ldg(r + k);
-                const uint32_t a = rotr(lds32(sm, e.x) & lm, rot0), b = rotr(lds32(sm, e.y) & lm, rot1);
-                h = or_if_less(h, (k & 1) ? word : word << 16, lds32(sm, e.z + (a | b | lb)), 1u << k);
+                h = or_if_less(h, (k & 1) ? word : word << 16, filter_threshold(sm, __ldg(r + k), rot0, rot1, lb), 1u << k);
             }
         }
     }
 #pragma unroll
     for (int c = 0; c < 4; ++c) {  // call c draws for filters 4c .. 4c + 3
-        if (!kPaper && c < g.n_calls) {
+        if (!kPaper && c < n_calls) {
             const U4 q = philox_from_round2(Y, rs, r2, rc.a ^ static_cast<uint32_t>(c), rk);
 #pragma unroll
             for (int x = 0; x < 4; ++x) {
                 const int k = 4 * c + x;
-                if (k < g.nb) {
-                    const uint4 e = __ldg(r + k);
-                    const uint32_t a = rotr(lds32(sm, e.x) & lm, rot0), b = rotr(lds32(sm, e.y) & lm, rot1);
-                    h = or_if_less(h, pick(q, x), lds32(sm, e.z + (a | b | lb)), 1u << k);
+                if (k < nb) {
+                    h = or_if_less(h, pick(q, x), filter_threshold(sm, __ldg(r + k), rot0, rot1, lb), 1u << k);
                 }
             }
         }
@@ -89,16 +99,23 @@ __device__ __forceinline__ void hidden_cell_generic(const Geometry& g, char* sm,
 // lane), so that bit k is the term of filter k at its first endpoint and bit
 // 16 + k at its second; a spin's n_J, n_J' are then 2 popc(masked) - degree,
 // and its table row is the record's row of n = -degree plus
-// 2 (2 DJp + 1) popc_J + 2 popc_J'.  kPaper: the spin at window offset x =
-// 2r + c takes half x & 1 of word 1 + (x >> 1) of tag 1.
+// 2 (2 DJp + 1) popc_J + 2 popc_J'.  In cells where no spin meets the same
+// (filter, endpoint) in two of the rows (all but those that an odd periodic side
+// wraps onto itself; bit 31 of the first source offset) the masked rows are
+// merged first, two counts per spin instead of eight (a POPC takes 8.4 cycles):
+// jmask, the bits of the J filters, splits the merged word.  kPaper: the spin at window offset x = 2r + c
+// takes half x & 1 of word 1 + (x >> 1) of tag 1.
 template <bool kPaper>
 __device__ __forceinline__ void visible_cell_generic(char* sm, const uint4* __restrict__ rv, int cell,
                                                      const Round1Sweep& rs, uint32_t Y, const uint32_t (&rk)[20],
-                                                     uint32_t sflip, uint32_t stepJ, uint32_t lb, int lane) {
+                                                     uint32_t sflip, uint32_t stepJ, uint32_t lb, int lane,
+                                                     uint32_t jmask) {
     const uint4* r = rv + static_cast<size_t>(cell) * kGenVisRec;
     const Round0Cell rc = round0_cell(static_cast<uint32_t>(cell), rk[1]);
     const U4 q = philox_from_round2(Y, rs, round2_cell(rs.hik ^ rc.b), rc.a ^ (kPaper ? 1u : kTagVis), rk);
-    const uint4 src = __ldg(r);
+    uint4 src = __ldg(r);
+    const bool merged = (src.x & 0x80000000u) != 0u;
+    src.x &= 0x7FFFFFFFu;
     const uint32_t l2 = 2u * static_cast<uint32_t>(lane);
     uint32_t w[4];
     w[0] = lds16(sm, src.x + l2);
@@ -110,9 +127,17 @@ __device__ __forceinline__ void visible_cell_generic(char* sm, const uint4* __re
     const uint4 tb = __ldg(r + 9), so = __ldg(r + 10);
 #pragma unroll
     for (int x = 0; x < 4; ++x) {
-        const uint4 mj = __ldg(r + 1 + 2 * x), mp = __ldg(r + 2 + 2 * x);
-        const uint32_t cj = __popc(w[0] & mj.x) + __popc(w[1] & mj.y) + __popc(w[2] & mj.z) + __popc(w[3] & mj.w);
-        const uint32_t cp = __popc(w[0] & mp.x) + __popc(w[1] & mp.y) + __popc(w[2] & mp.z) + __popc(w[3] & mp.w);
+        uint32_t cj, cp;
+        if (merged) {  // (the J' masks are in the J masks' place too)
+            const uint4 m = __ldg(r + 1 + 2 * x);
+            const uint32_t b = (w[0] & m.x) | (w[1] & m.y) | (w[2] & m.z) | (w[3] & m.w);
+            cj = __popc(b & jmask);
+            cp = __popc(b & ~jmask);
+        } else {
+            const uint4 mj = __ldg(r + 1 + 2 * x), mp = __ldg(r + 2 + 2 * x);
+            cj = __popc(w[0] & mj.x) + __popc(w[1] & mj.y) + __popc(w[2] & mj.z) + __popc(w[3] & mj.w);
+            cp = __popc(w[0] & mp.x) + __popc(w[1] & mp.y) + __popc(w[2] & mp.z) + __popc(w[3] & mp.w);
+        }
         const uint32_t row = (x == 0 ? tb.x : x == 1 ? tb.y : x == 2 ? tb.z : tb.w) + cj * stepJ + (cp << 8);
         const uint32_t u = kPaper ? ((x & 1) ? pick(q, 1 + (x >> 1)) : pick(q, 1 + (x >> 1)) << 16) : pick(q, x);
         const uint32_t vw = __ballot_sync(0xffffffffu, u < lds32(sm, row + lb));
@@ -143,12 +168,16 @@ __device__ __forceinline__ void count_cell(const Geometry& g, const uint32_t* s_
 // sweeps on device.  Warps split the cells of each half-step; __syncthreads
 // separates the half-steps (hidden reads v / writes h; visible reads h /
 // writes v).  kPaper: CRBM_PRECISION_PAPER draws (see the cores).
-template <bool kPaper>
+// kNb: 10 when the context has ten filters (the SS list on any lattice), else 0.
+template <bool kPaper, int kNb>
 __device__ __forceinline__ void sweep_generic_body(const SweepArgs& a, int word) {
     extern __shared__ __align__(128) uint32_t smem[];
     const Geometry& g = a.g;
     const GenericSmem gs = generic_smem(g);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+    // (the shuffle tells the compiler that the warp index is warp-uniform: the cells' Philox words and record
+    // addresses then run on the uniform pipe)
+    const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);
+    const int nwarp = blockDim.x >> 5;
     char* sm = reinterpret_cast<char*>(smem);
     int64_t* s_acc = reinterpret_cast<int64_t*>(smem);  // [kNSum][32] running sums
     uint32_t* s_tab = smem + gs.tab;
@@ -176,8 +205,11 @@ __device__ __forceinline__ void sweep_generic_body(const SweepArgs& a, int word)
     }
     const uint32_t sn[2] = {bit_of(a.sneg[2 * word], lane), bit_of(a.sneg[2 * word + 1], lane)};
     uint32_t sflip = 0u;  // filters whose class coefficient is -1 for this lane
-    for (int k = 0; k < g.nb; ++k) sflip |= (g.cls[k] ? sn[1] : sn[0]) << k;
-    const uint32_t lm = 1u << lane;
+    uint32_t jmask = 0u;  // bits of the J filters in an expanded row
+    for (int k = 0; k < g.nb; ++k) {
+        sflip |= (g.cls[k] ? sn[1] : sn[0]) << k;
+        if (g.cls[k] == 0) jmask |= 0x10001u << k;
+    }
     const uint32_t rot0 = static_cast<uint32_t>(lane - 7) & 31u, rot1 = static_cast<uint32_t>(lane - 8) & 31u;
     const uint32_t stepJ = 256u * static_cast<uint32_t>(2 * g.DJp + 1);
     const uint32_t chain = static_cast<uint32_t>(word) * 32u + lane;
@@ -202,10 +234,10 @@ __device__ __forceinline__ void sweep_generic_body(const SweepArgs& a, int word)
         const uint32_t t = t0 + static_cast<uint32_t>(it);
         const Round1Sweep rs = round1_sweep(r0l.hi ^ t ^ a.rk[0], a.rk);
         for (int cell = warp; cell < g.n_cells; cell += nwarp)
-            hidden_cell_generic<kPaper>(g, sm, rh, hw_byte, cell, rs, r0l.lo, a.rk, lm, rot0, rot1, lb, lane);
+            hidden_cell_generic<kPaper, kNb>(g, sm, rh, hw_byte, cell, rs, r0l.lo, a.rk, rot0, rot1, lb, lane);
         __syncthreads();
         for (int cell = warp; cell < g.n_cells; cell += nwarp)
-            visible_cell_generic<kPaper>(sm, rv, cell, rs, r0l.lo, a.rk, sflip, stepJ, lb, lane);
+            visible_cell_generic<kPaper>(sm, rv, cell, rs, r0l.lo, a.rk, sflip, stepJ, lb, lane, jmask);
         __syncthreads();
         const bool do_meas = every_meas.step();
         const bool do_swap = every_swap.step();

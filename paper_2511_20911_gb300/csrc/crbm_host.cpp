@@ -237,8 +237,10 @@ void free_device(DeviceState& d) {
     d = DeviceState{};
 }
 
-// Warps per CTA of the SMEM sweeps.  Bit-plane and generic sweeps: about six
-// cells per warp, up to 16.  The canonical sweep, by whether every SM has two
+// Warps per CTA of the SMEM sweeps.  Bit-plane sweep: about six cells per warp,
+// up to 16.  Generic sweep (us per sweep with 4, 8, 16 warps, 48 words of 18 x 12
+// spins: 8.8 6.2 5.4, 304 words: 11.7 9.8 10.7, 600 words: 18.7 19.1 21.1, of 9 x 9
+// spins 9.1 10.0 11.5): fewer warps the more words an SM has.  The canonical sweep, by whether every SM has two
 // words or more (us per sweep of 384 words with 4, 8, 12, 16 warps: L = 6 2.65
 // 2.81, L = 12 6.07 6.07 5.42 5.50, L = 18 11.5 10.6 11.0 11.4, L = 24 21.1 18.7 -
 // 18.5, L = 30 32.6 29.1 28.8 28.4; of 152 words with 8, 16, 32: L = 18 5.1 4.6
@@ -249,11 +251,14 @@ int default_warps(const Geometry& g, int n_words) {
         const int w = std::atoi(env);
         if (w >= 1 && w <= kMaxSweepWarps) return w;
     }
-    if (!g.canonical || g.bitplane) return std::max(1, std::min(std::min(16, kMaxSweepWarps), (g.n_cells + 5) / 6));
+    if (g.bitplane) return std::max(1, std::min(std::min(16, kMaxSweepWarps), (g.n_cells + 5) / 6));
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
         sms = 152;
+    if (!g.canonical)
+        return std::max(1, std::min(std::min(n_words <= sms ? 16 : n_words < 3 * sms || g.n_cells >= 64 ? 8 : 4, kMaxSweepWarps),
+                                    g.n_cells));
     if (n_words >= 2 * sms && g.n_cells <= 400)  // (larger ones hold one CTA per SM)
         return std::min(kMaxSweepWarps, g.n_cells < 16 ? 4 : g.n_cells < 30 || (g.n_cells >= 50 && g.n_cells <= 144) ? 8 : 12);
     return std::min(kMaxSweepWarps, g.n_cells < 8 ? 8 : g.n_cells <= 16 ? 12 : g.n_cells <= 600 ? 16 : 32);
@@ -683,6 +688,7 @@ int crbm_create(crbm_ctx** out, const crbm_params* p) {
             uint32_t* o = &crec[(nh + static_cast<size_t>(c) * kGenVisRec) * 4];
             for (int q = 0; q < 4; ++q)
                 o[q] = 4u * static_cast<uint32_t>(src[q] >= 0 ? gs.hw + static_cast<size_t>(src[q]) * 16 : gs.zrow);
+            bool merged = true;  // no (filter, endpoint) of a spin in two of the four rows
             for (int x = 0; x < 4; ++x) {
                 const int R = 2 * i + (x >> 1), C = 2 * j + (x & 1);
                 uint32_t* mj = o + 4 * (1 + 2 * x);
@@ -690,6 +696,7 @@ int crbm_create(crbm_ctx** out, const crbm_params* p) {
                 int deg[2] = {0, 0};
                 if (R < g.L && C < g.Lc) {
                     const int s = R * g.Lc + C;
+                    uint32_t seen = 0u;
                     for (const int e : incid[s]) {
                         const int cc = e / (2 * kMaxBonds), k = (e / 2) % kMaxBonds, second = e & 1;
                         int q = 0;
@@ -699,7 +706,10 @@ int crbm_create(crbm_ctx** out, const crbm_params* p) {
                             return fail(nullptr, CRBM_EINVAL, "internal: incidence outside the cell's windows");
                         }
                         const int cls = g.cls[k];
-                        (cls ? mp : mj)[q] |= 1u << (k + 16 * second);
+                        const uint32_t bit = 1u << (k + 16 * second);
+                        (cls ? mp : mj)[q] |= bit;
+                        if (seen & bit) merged = false;
+                        seen |= bit;
                         ++deg[cls];
                     }
                     o[4 * 10 + x] = site_off(s);
@@ -709,6 +719,11 @@ int crbm_create(crbm_ctx** out, const crbm_params* p) {
                 const int odd_table = (g.n_vis_tab == 2 && (C & 1)) ? g.nTv : 0;  // odd column: second table
                 o[4 * 9 + x] = 4u * static_cast<uint32_t>(
                     gs.tab + static_cast<size_t>(kGenHid + odd_table + (g.DJ - deg[0]) * nP + (g.DJp - deg[1])) * 32);
+            }
+            if (merged) {
+                for (int x = 0; x < 4; ++x)
+                    for (int q = 0; q < 4; ++q) o[4 * (1 + 2 * x) + q] |= o[4 * (2 + 2 * x) + q];
+                o[0] |= 0x80000000u;
             }
         }
     }

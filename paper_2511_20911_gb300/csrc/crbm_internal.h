@@ -38,7 +38,7 @@ static_assert(kBpHidPlanes % 4 == 0 && kBpVisPlanes % 4 == 0 && kBpTab % 4 == 0 
               "the sweeps read four threshold planes with one 16-byte load");
 
 // Canonical fast-path tables per packed word in HBM: hidden [2 cls][4 idx][32
-// lanes] then visible [4 spin positions][32 idx][32 lanes] (crbm_canon_core.cuh).
+// lanes] then visible [4 spin positions][32 idx][32 lanes] (crbm_row_core.cuh).
 constexpr int kCanonTh = 2 * 4 * 32;
 constexpr int kCanonTab = kCanonTh + 4 * 32 * 32;
 // Per-cell records of the canonical SMEM sweep, kCellRec uint4 per cell, built
@@ -158,7 +158,9 @@ constexpr int kGenHid = 2 * 4 * 4;
 //     above-left; a zero row where there is none); then per owned spin
 //     x = 2 r + c: [1 + 2x] J masks, [2 + 2x] J' masks over the four rows'
 //     expanded words (bit k: filter k with the spin as first endpoint, bit
-//     16 + k: as second endpoint); [9] the table row of n_J = n_J' = -deg
+//     16 + k: as second endpoint); in a cell whose first source offset
+//     has bit 31 set no spin meets the same (filter, endpoint) in two of the rows,
+//     and [1 + 2x] has the J and the J' masks; [9] the table row of n_J = n_J' = -deg
 //     of each spin; [10] each spin's word (a scratch word for a position past
 //     the lattice edge).
 constexpr int kGenVisRec = 11;

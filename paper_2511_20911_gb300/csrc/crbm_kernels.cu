@@ -16,9 +16,9 @@ namespace {
 
 using namespace dev;
 
-template <bool kPaper>
+template <bool kPaper, int kNb>
 __global__ void __launch_bounds__(512, 1) k_sweep_generic(const SweepArgs a) {
-    generic::sweep_generic_body<kPaper>(a, blockIdx.x);
+    generic::sweep_generic_body<kPaper, kNb>(a, blockIdx.x);
 }
 
 // Initial spins: site (R, C) of chain c is +1 iff word 2(R&1)+(C&1) of
@@ -133,7 +133,8 @@ cudaError_t launch_init(const Geometry& g, uint32_t* v, int n_words, uint32_t ke
 
 cudaError_t launch_sweep_generic(const SweepArgs& a, int warps_per_cta, cudaStream_t st) {
     const size_t smem = smem_bytes_generic(a.g);
-    auto kernel = a.g.paper ? k_sweep_generic<true> : k_sweep_generic<false>;
+    auto kernel = a.g.nb == 10 ? (a.g.paper ? k_sweep_generic<true, 10> : k_sweep_generic<false, 10>)
+                               : (a.g.paper ? k_sweep_generic<true, 0> : k_sweep_generic<false, 0>);
     if (smem > 48 * 1024) {
         const cudaError_t e =
             cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
