@@ -4,8 +4,6 @@
 // The spins are kept in row form (crbm_row_core.cuh).
 #pragma once
 
-#include <type_traits>
-
 #include <cooperative_groups.h>
 
 #include "crbm_row_core.cuh"
@@ -35,9 +33,6 @@ struct CellRecs<kCanonRec> {
         return lds128<16 * k>(p);
     }
 };
-
-template <int j>
-using Cell = std::integral_constant<int, j>;  // the j-th cell of a segment
 
 // The two halves of a cluster barrier, so that work no other CTA waits for
 // can run between them: arrive (release: this thread's earlier shared-memory
@@ -185,6 +180,8 @@ __device__ __forceinline__ void sweep_canon_body(const SweepArgs& a, int word, u
         if (kMode == kCanonRec && first) stage(rec_addr, a.crec, g.n_cells * kCellRec);
         // spins to row form: the site words of a segment's word (lane = bit), bit-transposed (lane = chain)
         const uint32_t* gv = a.v + static_cast<size_t>(word) * g.N;
+        const Transpose32 transpose(lane);
+        const SegmentSites site(g.Lc, lane);
         for (int u0 = warp; u0 < W * nseg; u0 += 4 * nwarp) {
             uint32_t v[4];
 #pragma unroll
@@ -193,15 +190,13 @@ __device__ __forceinline__ void sweep_canon_body(const SweepArgs& a, int word, u
                 v[k] = 0u;
                 if (u < W * nseg) {
                     const Segment sg = segment(u);
-                    const int j = sg.j0 + sg.n == Wc ? 0 : sg.j0 + sg.n;  // the next segment's first cell: bits 15, 14
-                    const int p = lane - 16;
-                    const int site = p >= 0 ? row_site(p, sg.i, sg.j0, sg.n, g.Lc) : (2 * sg.i - 1 - p) * g.Lc + 2 * j;
-                    if (p >= -2 && p < 4 * sg.n) v[k] = __ldcg(gv + site);
+                    const int sx = site(lane, sg.i, sg.j0, sg.n, sg.j0 + sg.n == Wc ? 0 : sg.j0 + sg.n);
+                    if (lane >= 14 && lane < 16 + 4 * sg.n) v[k] = __ldcg(gv + sx);
                 }
             }
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                if (u0 + k * nwarp < W * nseg) sts32(row_addr(u0 + k * nwarp), transpose32(v[k], lane));
+                if (u0 + k * nwarp < W * nseg) sts32(row_addr(u0 + k * nwarp), transpose(v[k]));
         }
         build_threshold_tables(s_tab, gt, threadIdx.x, blockDim.x);
         if (kPacked && first)
@@ -310,7 +305,7 @@ __device__ __forceinline__ void sweep_canon_body(const SweepArgs& a, int word, u
                     auto decide = [&](auto jc, const U4& q) {
                         constexpr uint32_t off = kWCell * decltype(jc)::value;
                         const uint32_t own = load_w(wo + off);
-                        o = visible_row_cell(merge_words(own, load_w(wu + off), left), q, tab4, o);
+                        o = visible_row_cell<kRowVis>(merge_words(own, load_w(wu + off), left), q, tab4, o);
                         left = own;
                     };
                     if (sg.n == 3) {  // the three calls side by side
@@ -386,10 +381,11 @@ __device__ __forceinline__ void sweep_canon_body(const SweepArgs& a, int word, u
                 __syncthreads();
                 accumulate_correlations_rows(a, scratch, s_seg, s_segmask, warp, nwarp, lane);
             } else {  // one word per site
+                const SegmentSites site(g.Lc, lane);
                 for (int u = warp; u < W * nseg; u += nwarp) {
                     const Segment sg = segment(u);
-                    const uint32_t v = transpose32(lds32(row_addr(u)) >> 16, lane);
-                    if (lane < 4 * sg.n) scratch[row_site(lane, sg.i, sg.j0, sg.n, g.Lc)] = v;
+                    const uint32_t v = transpose32(lds32(row_addr(u)), lane);
+                    if (lane >= 16 && lane < 16 + 4 * sg.n) scratch[site(lane, sg.i, sg.j0, sg.n, sg.j0 + sg.n)] = v;
                 }
                 __syncthreads();
                 accumulate_correlations_sites(a, scratch, s_seg, s_segmask, warp, nwarp, lane);
@@ -400,10 +396,12 @@ __device__ __forceinline__ void sweep_canon_body(const SweepArgs& a, int word, u
     if (kCluster) body_sync<true>();  // no rank reads another's shared memory after this
     if (!active) return;
     uint32_t* gv = a.v + static_cast<size_t>(word) * g.N;
+    const Transpose32 transpose(lane);
+    const SegmentSites site(g.Lc, lane);
     for (int u = u_begin + warp; u < u_end; u += nwarp) {  // own rows
         const Segment sg = segment(u);
-        const uint32_t v = transpose32(lds32(row_addr(u)) >> 16, lane);
-        if (lane < 4 * sg.n) gv[row_site(lane, sg.i, sg.j0, sg.n, g.Lc)] = v;
+        const uint32_t v = transpose(lds32(row_addr(u)));
+        if (lane >= 16 && lane < 16 + 4 * sg.n) gv[site(lane, sg.i, sg.j0, sg.n, sg.j0 + sg.n)] = v;
     }
     if (band == 0 && warp == post_warp && a.swap_every > 0) a.sob[word * 32 + lane] = s_sob[lane];
     if (band == 0 && warp == post_warp && measuring) {

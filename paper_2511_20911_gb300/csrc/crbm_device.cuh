@@ -138,18 +138,31 @@ __device__ __forceinline__ uint32_t bit_of(uint32_t word, int lane) { return (wo
 __device__ __forceinline__ uint32_t rotr(uint32_t x, uint32_t s) { return __funnelshift_r(x, x, s); }
 
 // 32 x 32 bit transpose across a warp: lane c returns the word whose bit l is
-// bit c of lane l's x (block swaps of 16, 8, 4, 2 and 1 rows and columns).
-__device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
-    constexpr uint32_t kLow[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
+// bit c of lane l's x (block swaps of 16, 8, 4, 2 and 1 rows and columns).  A lane
+// keeps half of its bits in each swap and takes the others from its partner's
+// word, rotated: with the masks and amounts of its lane at hand that is a
+// shuffle, a rotation and a bitwise select.
+struct Transpose32 {
+    uint32_t keep[5], rot[5];
+    __device__ __forceinline__ explicit Transpose32(int lane) {
+        constexpr uint32_t kLow[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
 #pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        const int j = 16 >> i;
-        const uint32_t m = kLow[i];
-        const uint32_t y = __shfl_xor_sync(0xffffffffu, x, j);
-        x = (lane & j) ? ((x & ~m) | ((y >> j) & m)) : ((x & m) | ((y << j) & ~m));
+        for (int i = 0; i < 5; ++i) {
+            const uint32_t j = 16u >> i;
+            keep[i] = (lane & j) ? ~kLow[i] : kLow[i];
+            rot[i] = (lane & j) ? 32u - j : j;
+        }
     }
-    return x;
-}
+    __device__ __forceinline__ uint32_t operator()(uint32_t x) const {
+#pragma unroll
+        for (int i = 0; i < 5; ++i) {
+            const uint32_t y = __shfl_xor_sync(0xffffffffu, x, 16 >> i);
+            x = (x & keep[i]) | (__funnelshift_l(y, y, rot[i]) & ~keep[i]);
+        }
+        return x;
+    }
+};
+__device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) { return Transpose32(lane)(x); }
 
 // Release store of a progress counter in global memory.
 __device__ __forceinline__ void st_release(int* p, int v) {

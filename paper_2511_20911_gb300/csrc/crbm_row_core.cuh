@@ -25,6 +25,8 @@
 //    balloted or stored per cell.
 #pragma once
 
+#include <type_traits>
+
 #include "crbm_device.cuh"
 
 namespace crbm {
@@ -157,6 +159,9 @@ __device__ __forceinline__ void sts64(uint32_t addr, uint2 x) {
     asm volatile("st.shared.v2.u32 [%0+%3], {%1, %2};" ::"r"(addr), "r"(x.x), "r"(x.y), "n"(kOff) : "memory");
 }
 
+template <int j>
+using Cell = std::integral_constant<int, j>;  // the j-th cell of a segment
+
 // The windows of a segment of n cells from its word and the word of the segment
 // below, the current cell's (the first's) at bits 13 .. 8; next() moves on.
 struct Windows {
@@ -269,18 +274,34 @@ __device__ __forceinline__ uint32_t expand_word(uint32_t h) {
 
 // Visible half-step of one cell: its uniforms against the thresholds at the
 // merged bits c; the four decisions are the next nibble of the new word o.
+// kVis: the visible tables' offset from tab4's address.
+template <int kVis>
 __device__ __forceinline__ uint32_t visible_row_cell(uint32_t c, const U4& u, uint32_t tab4, uint32_t o) {
     constexpr uint32_t f = 31u << 7;
-    const uint32_t t00 = tab32<kRowVis>((c & f) | tab4);
-    const uint32_t t01 = tab32<kRowVis + 4096>(((c >> 5) & f) | tab4);
-    const uint32_t t10 = tab32<kRowVis + 8192>(((c >> 10) & f) | tab4);
-    const uint32_t t11 = tab32<kRowVis + 12288>(((c >> 15) & f) | tab4);
+    const uint32_t t00 = tab32<kVis>((c & f) | tab4);
+    const uint32_t t01 = tab32<kVis + 4096>(((c >> 5) & f) | tab4);
+    const uint32_t t10 = tab32<kVis + 8192>(((c >> 10) & f) | tab4);
+    const uint32_t t11 = tab32<kVis + 12288>(((c >> 15) & f) | tab4);
     o *= 16u;
     o = or_if_less<8u>(o, u.x, t00);
     o = or_if_less<2u>(o, u.y, t01);
     o = or_if_less<4u>(o, u.z, t10);
     o = or_if_less<1u>(o, u.w, t11);
     return o;
+}
+
+// Record words of cell `cell` (see kCellRec), formed on the device: the hidden
+// calls', and the visible call's (in paper precision the tag-1 call).
+__device__ __forceinline__ void hidden_call_words(uint32_t cell, const uint32_t (&rk)[20], uint4& q0, uint4& q1) {
+    const Round0Cell rc = round0_cell(cell, rk[1]);
+    const Round1Call c0 = round1_call(rc.a, rk), c1 = round1_call(rc.a ^ 1u, rk), c2 = round1_call(rc.a ^ 2u, rk);
+    q0 = make_uint4(rc.b, c0.h, c0.l, c1.h);
+    q1 = make_uint4(c1.l, c2.h, c2.l, 0u);
+}
+__device__ __forceinline__ uint4 visible_call_words(uint32_t cell, uint32_t tag, const uint32_t (&rk)[20]) {
+    const Round0Cell rc = round0_cell(cell, rk[1]);
+    const Round1Call cv = round1_call(rc.a ^ tag, rk);
+    return make_uint4(rc.b, cv.h, cv.l, 0u);
 }
 
 // Measurement counts of a segment of n cells (words as for Windows): anti-aligned
@@ -294,10 +315,23 @@ __device__ __forceinline__ void count_segment(uint32_t own, uint32_t below, int 
     pos += __popc(s);
 }
 
-// Site of bit p (0 .. 4 n - 1) of the word of cells j0 .. j0 + n - 1 of cell row i.
-__device__ __forceinline__ int row_site(int p, int i, int j0, int n, int Lc) {
-    return (2 * i + 1 - (p & 1)) * Lc + 2 * (j0 + n - 1 - (p >> 2)) + 1 - ((p >> 1) & 1);
-}
+// The site of each bit 14 .. 16 + 4 n - 1 of a segment's word, lane = bit: cells
+// j .. j + n - 1 of cell row i, jn the next segment's first cell (bits 15, 14).
+// Full segments away from the right edge share their offsets from the first
+// cell's site.
+struct SegmentSites {
+    int Lc, full;
+    __device__ __forceinline__ SegmentSites(int Lc_, int lane) : Lc(Lc_) { full = offset(lane - 16, 3, 6); }
+    // site of bit 16 + p less the first cell's; next = column of jn less the first cell's
+    __device__ __forceinline__ int offset(int p, int n, int next) const {
+        return p >= 0 ? (1 - (p & 1)) * Lc + 2 * (n - 1 - (p >> 2)) + 1 - ((p >> 1) & 1) : (-1 - p) * Lc + next;
+    }
+    // lanes < 14 and >= 16 + 4 n have no site
+    __device__ __forceinline__ int operator()(int lane, int i, int j, int n, int jn) const {
+        const int first = 2 * i * Lc + 2 * j;
+        return first + (n == 3 && jn > j ? full : offset(lane - 16, n, 2 * (jn - j)));
+    }
+};
 
 }  // namespace canon
 }  // namespace crbm

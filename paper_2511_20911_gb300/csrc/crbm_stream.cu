@@ -2,14 +2,15 @@
 // filters, even periodic L x Lc): spins and hidden units live in HBM and one sweep
 // is two launches, the hidden half-step (Eq. 9) then the visible half-step
 // (Eq. 10).  Spins are stored as 64-chain words, two 32-bit halves per site
-// ([group][site][2]); a CTA works on one 32-chain half and one tile of cells,
-// staging its tile (plus a one-site / one-cell halo) in shared memory with
-// plain coalesced loads, and reuses the per-cell cores of the SMEM path.  In
-// paper precision (kPaper) the hidden half-step makes the tag-0 and tag-1
-// calls and the visible half-step draws the tag-1 call again for its four
-// 16-bit uniforms: three calls per cell instead of four.
+// ([group][site][2]); a CTA works on one 32-chain half and one tile of cells.
+// The hidden half-step stages its tile's spins in row form (a bit transpose per
+// segment of three cells) and the visible one its tile's hidden words with one
+// cell of halo; both reuse the per-cell cores of the SMEM path
+// (crbm_row_core.cuh).  In paper precision (kPaper) the hidden half-step makes
+// the tag-0 and tag-1 calls and the visible half-step draws the tag-1 call again
+// for its four 16-bit uniforms: three calls per cell instead of four.
 #include "crbm_bitplane_core.cuh"
-#include "crbm_canon_core.cuh"
+#include "crbm_row_core.cuh"
 
 namespace crbm {
 namespace {
@@ -17,16 +18,35 @@ namespace {
 using namespace dev;
 using namespace canon;
 
-constexpr int kTI = 16;  // tile rows of cells
+// Tiles of the lane-uniform sweep and of the count: 4, 8 or 16 rows of cells by 4,
+// 5 or 6 segments of three (RowCut).
+constexpr int kTI = 16;  // tile rows of cells (at most)
+constexpr int kMaxTileSeg = 6, kMaxTileCols = 3 * kMaxTileSeg;
+// Tiles of the bit-plane sweep.
 constexpr int kTJ = 16;  // tile columns of cells
-#ifndef CRBM_STREAM_THREADS
-#define CRBM_STREAM_THREADS 256
-#endif
-#ifndef CRBM_STREAM_VIS_THREADS
-#define CRBM_STREAM_VIS_THREADS 256
-#endif
-constexpr int kStreamThreads = CRBM_STREAM_THREADS;      // hidden and count kernels
-constexpr int kStreamVisThreads = CRBM_STREAM_VIS_THREADS;
+constexpr int kStreamThreads = 256;  // every kernel
+constexpr int kStreamVisThreads = kStreamThreads;
+
+// Cut of the lattice into row tiles: the width that pads it least, 16 rows where
+// these make four CTAs per SM and else fewer, down to 4 (100 x 100 spins, 64
+// chains: 27 us per sweep in tiles of 16 rows, 16 in tiles of 4).
+struct RowCut {
+    int seg, rows;
+};
+inline RowCut row_cut(const Geometry& g, int n_words, int sms) {
+    RowCut c{5, kTI};
+    int waste = 1 << 30;
+    for (int s = 4; s <= kMaxTileSeg; ++s) {
+        const int pad = (g.Wc + 3 * s - 1) / (3 * s) * (3 * s) - g.Wc;
+        if (pad < waste || (pad == waste && s == 5)) {
+            c.seg = s;
+            waste = pad;
+        }
+    }
+    const int64_t columns = static_cast<int64_t>((g.Wc + 3 * c.seg - 1) / (3 * c.seg)) * n_words;
+    while (c.rows > 4 && columns * ((g.W + c.rows - 1) / c.rows) < 4 * sms) c.rows /= 2;
+    return c;
+}
 
 __device__ __forceinline__ size_t vidx(int w, int N, int s) {
     return (static_cast<size_t>(w >> 1) * N + s) * 2 + (w & 1);
@@ -41,12 +61,7 @@ __device__ __forceinline__ void stage_rungs(const SweepArgs& a, int w, int* s_bo
         s_bos[a.swap_every > 0 ? __ldg(a.sob + static_cast<size_t>(w) * 32 + lane) : lane] = lane;
     }
 }
-#ifndef CRBM_STREAM_MIN_BLOCKS
-#define CRBM_STREAM_MIN_BLOCKS 4
-#endif
-#ifndef CRBM_STREAM_VIS_MIN_BLOCKS
-#define CRBM_STREAM_VIS_MIN_BLOCKS 4
-#endif
+constexpr int kStreamMinBlocks = 4;
 
 // Stage spin rows 2 i0 .. 2 i0 + 2 TI and columns 2 j0 .. 2 j0 + 2 TJ
 // (wrapped) of half-word w into s_v[(2 TI + 1)][(2 TJ + 1)].  Every load of a
@@ -106,157 +121,200 @@ __device__ __forceinline__ void stage_spin_tile(const SweepArgs& a, int w, int i
         stage_spin_tile<false>(a, w, i0, j0, s_v);
 }
 
-// Stage the hidden words of cells i0 - 1 .. i0 + TI - 1 x j0 - 1 .. j0 + TJ - 1
-// (wrapped) of half-word w into s_h[(TI + 1)][(TJ + 1)][32], 16 bytes per
-// load, in batches whose loads are all issued before their stores.
-// kOneWrap: W > TI and Wc > TJ, so i0 - 1 + li in [-1, W + TI - 2] (and the
-// same for columns) wraps with one add or subtraction of W (Wc).
-template <bool kOneWrap>
-__device__ __forceinline__ void stage_hidden_halo(const SweepArgs& a, int w, int i0, int j0, uint32_t* s_h) {
-    constexpr int HS = kTJ + 1, NQ = (kTI + 1) * HS * 8;  // 8 uint4 per cell
-    constexpr int IT = (NQ + kStreamVisThreads - 1) / kStreamVisThreads;
-    constexpr int B = 5;  // loads in flight per thread
-    const int W = a.g.W, Wc = a.g.Wc;
-    const uint4* hw = reinterpret_cast<const uint4*>(a.h + static_cast<size_t>(w) * a.g.n_cells * 32);
+// A tile of the lane-uniform sweep: ni x nj cells from (i0, j0), nseg segments
+// per row.
+struct RowTile {
+    int i0, j0, ni, nj, nseg;
+    uint32_t magic;  // u / nseg = umulhi(u, magic): u < 2^16, nseg <= 6 and no power of two but 1, 2, 4
+    __device__ __forceinline__ RowTile(const Geometry& g, int tile, const RowCut& cut) {
+        const int tile_seg = cut.seg;
+        const int tiles_j = (g.Wc + 3 * tile_seg - 1) / (3 * tile_seg);
+        i0 = (tile / tiles_j) * cut.rows;
+        j0 = (tile % tiles_j) * 3 * tile_seg;
+        ni = min(cut.rows, g.W - i0);
+        nj = min(3 * tile_seg, g.Wc - j0);
+        nseg = (nj + 2) / 3;
+        magic = nseg > 1 ? 0xFFFFFFFFu / static_cast<uint32_t>(nseg) + 1u : 0u;
+    }
+    // segment u: tile row r, segment s of it
+    __device__ __forceinline__ void segment(int u, int& r, int& s, int& n) const {
+        r = nseg > 1 ? static_cast<int>(__umulhi(static_cast<uint32_t>(u), magic)) : u;
+        s = u - r * nseg;
+        n = min(3, nj - 3 * s);
+    }
+};
+
+// The words of the tile's segments and of the row of segments below (wrapped) to
+// rows[u * 32 + lane] by shared address, four segments' loads in flight a warp.
+__device__ __forceinline__ void stage_rows(const SweepArgs& a, int w, const RowTile& t, uint32_t rows, int warp, int lane) {
+    const Geometry& g = a.g;
+    const uint32_t* vw = a.v + vidx(w, g.N, 0);  // site s of half-word w at vw[2 s]
+    constexpr int nwarp = kStreamThreads / 32;
+    const int n_seg = (t.ni + 1) * t.nseg;
+    const Transpose32 transpose(lane);
+    const SegmentSites site(g.Lc, lane);
+    for (int u0 = warp; u0 < n_seg; u0 += 4 * nwarp) {
+        uint32_t v[4];
 #pragma unroll
-    for (int k0 = 0; k0 < IT; k0 += B) {
-        uint4 val[B];
-#pragma unroll
-        for (int k = 0; k < B; ++k) {
-            const int x = threadIdx.x + (k0 + k) * kStreamVisThreads;
-            const int lcell = x >> 3, q = x & 7;
-            const int li = lcell / HS, lj = lcell - (lcell / HS) * HS;
-            int gi = i0 - 1 + li, gj = j0 - 1 + lj;
-            if (kOneWrap) {
-                gi += gi < 0 ? W : 0;
-                gi -= gi >= W ? W : 0;
-                gj += gj < 0 ? Wc : 0;
-                gj -= gj >= Wc ? Wc : 0;
-            } else {
-                gi = (gi % W + W) % W;
-                gj = (gj % Wc + Wc) % Wc;
+        for (int k = 0; k < 4; ++k) {
+            const int u = u0 + k * nwarp;
+            v[k] = 0u;
+            if (u < n_seg) {
+                int r, s, n;
+                t.segment(u, r, s, n);
+                const int i = t.i0 + r == g.W ? 0 : t.i0 + r, j = t.j0 + 3 * s;
+                const int sx = site(lane, i, j, n, j + n == g.Wc ? 0 : j + n);
+                if (lane >= 14 && lane < 16 + 4 * n) v[k] = vw[2 * sx];
             }
-            val[k] = make_uint4(0u, 0u, 0u, 0u);
-            if (k0 + k < IT && x < NQ) val[k] = hw[(gi * Wc + gj) * 8 + q];
         }
 #pragma unroll
-        for (int k = 0; k < B; ++k) {
-            const int x = threadIdx.x + (k0 + k) * kStreamVisThreads;
-            if (k0 + k < IT && x < NQ) reinterpret_cast<uint4*>(s_h)[x] = val[k];
-        }
+        for (int k = 0; k < 4; ++k)
+            if (u0 + k * nwarp < n_seg)
+                sts32(rows + 128u * static_cast<uint32_t>(u0 + k * nwarp) + 4u * static_cast<uint32_t>(lane), transpose(v[k]));
     }
 }
 
-// Hidden half-step of one tile: v tile rows 2 i0 .. 2 i0 + 2 TI and columns
-// 2 j0 .. 2 j0 + 2 TJ (wrapped), the lanes' hidden words out to
-// h[word][cell][32].
+// Dynamic shared memory of the hidden half-step: rungs and the tile's rows below
+// the tables (at shared address 16384, see kReservedSmem), then the call words.
+constexpr int kHidRowsByte = 128, kHidTabByte = 16384 - kReservedSmem, kHidCallByte = kHidTabByte + kCanonAccByte,
+              kHidSmem = kHidCallByte + 32 * kTI * kMaxTileCols;
+static_assert(kHidRowsByte + 128 * (kTI + 1) * kMaxTileSeg <= kHidTabByte && kHidCallByte % 16 == 0, "rows fit below the tables");
+
+// Hidden half-step of one tile: spins in, the lanes' hidden words out to
+// h[word][cell][32] (a warp's store of a cell is one 128-byte line).
 template <bool kPaper>
-__global__ void __launch_bounds__(kStreamThreads, CRBM_STREAM_MIN_BLOCKS) k_stream_hidden(const SweepArgs a, uint32_t t) {
-    __shared__ __align__(16) uint32_t s_th[kCanonTh];
-    __shared__ uint32_t s_v[(2 * kTI + 1) * (2 * kTJ + 1)];
-    __shared__ __align__(16) uint32_t s_h[kTI * kTJ * 32];
-    __shared__ uint4 s_q[kTI * kTJ][2];  // per tile cell: hidden_call_words
-    __shared__ int s_bos[32];            // rung of each replica slot
+__global__ void __launch_bounds__(kStreamThreads, kStreamMinBlocks) k_stream_hidden(const SweepArgs a, uint32_t t, RowCut cut) {
+    extern __shared__ __align__(128) char smem[];
     const Geometry& g = a.g;
-    const int W = g.W, Wc = g.Wc;
-    const int w = blockIdx.y;
-    const int tiles_j = (Wc + kTJ - 1) / kTJ;
-    const int i0 = (blockIdx.x / tiles_j) * kTI, j0 = (blockIdx.x % tiles_j) * kTJ;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-    const uint32_t* gt = a.ctab + static_cast<size_t>(w) * kCanonTab;
-    for (int x = threadIdx.x; x < kCanonTh; x += blockDim.x) s_th[x] = gt[x];
-    constexpr int VS = 2 * kTJ + 1;
-    stage_spin_tile(a, w, i0, j0, s_v);
+    const int w = blockIdx.y, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);
+    constexpr int nwarp = kStreamThreads / 32;
+    const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(smem)), tab = base + kHidTabByte;
+    if (tab & 16383u) return;  // (the launcher has checked it)
+    const RowTile tile(g, blockIdx.x, cut);
+    int* s_bos = reinterpret_cast<int*>(smem);
     stage_rungs(a, w, s_bos);
-    const uint32_t chain = static_cast<uint32_t>(w) * 32u + lane;
-    const Round0Lane r0l = round0_lane(chain);
-    const Round1Sweep rs = round1_sweep(r0l.hi ^ t ^ a.rk[0], a.rk);
-    const int ni = min(kTI, W - i0), nj = min(kTJ, Wc - j0);
+    const uint32_t rows = base + kHidRowsByte, calls = base + kHidCallByte;
+    stage_rows(a, w, tile, rows, warp, lane);
+    build_threshold_tables(smem + kHidTabByte, a.ctab + static_cast<size_t>(w) * kCanonTab, threadIdx.x, kStreamThreads);
     // the warp-uniform Philox words of each cell, once per CTA instead of once per warp-cell
-    for (int x = threadIdx.x; x < kTI * kTJ; x += blockDim.x) {
-        const int li = x / kTJ, lj = x - li * kTJ;
-        if (li < ni && lj < nj)
-            hidden_call_words(static_cast<uint32_t>((i0 + li) * Wc + j0 + lj), a.rk, s_q[x][0], s_q[x][1]);
+    for (int x = threadIdx.x; x < tile.ni * 3 * tile.nseg; x += kStreamThreads) {
+        const int r = x / (3 * tile.nseg), c = x - r * 3 * tile.nseg;
+        uint4* q = reinterpret_cast<uint4*>(smem + kHidCallByte) + 2 * x;
+        if (c < tile.nj) hidden_call_words(static_cast<uint32_t>((tile.i0 + r) * g.Wc + tile.j0 + c), a.rk, q[0], q[1]);
     }
-    __syncthreads();
-    const LaneConst lc = lane_const(lane, s_bos[lane]);
-    // warp = columns lj of the tile, cells walked down the column
-    for (int lj = warp; lj < nj; lj += nwarp) {
-        const uint32_t* v = s_v + 2 * lj;
-        uint32_t* hp = s_h + lj * 32 + lane;
-        const uint4* q = s_q[lj];
-        for (int li = 0; li < ni; ++li, v += 2 * VS, hp += kTJ * 32, q += 2 * kTJ)
-            *hp = kPaper ? hidden_cell_paper(v, VS, s_th, rs, r0l.lo, q[0], q[1], a.rk, lc)
-                         : hidden_cell(v, VS, s_th, rs, r0l.lo, q[0], q[1], a.rk, lc);
-    }
-    __syncthreads();
-    // tile rows of hidden words are contiguous runs of nj * 32 words in h
-    for (int x = threadIdx.x; x < kTI * kTJ * 8; x += blockDim.x) {
-        const int li = x / (kTJ * 8), rest = x - li * (kTJ * 8);
-        if (li >= ni || rest >= nj * 8) continue;
-        reinterpret_cast<uint4*>(a.h + (static_cast<size_t>(w) * g.n_cells + (i0 + li) * Wc + j0) * 32)[rest] =
-            reinterpret_cast<const uint4*>(s_h)[x];
-    }
-}
-
-// Visible half-step of one tile: hidden words of the tile cells plus the row
-// of cells above and the column to the left (wrapped), new spins out.
-// Three CTAs per SM (its shared memory) leave room for 85 registers a thread:
-// paper precision takes 72 (0.9 % faster than at 64); exact precision is
-// 0.4 % faster held to 64.
-template <bool kPaper>
-__global__ void __launch_bounds__(kStreamVisThreads, kPaper ? 3 : CRBM_STREAM_VIS_MIN_BLOCKS)
-    k_stream_visible(const SweepArgs a, uint32_t t) {
-    __shared__ __align__(16) uint32_t s_tv[4 * 32 * 32];
-    __shared__ __align__(16) uint32_t s_h[(kTI + 1) * (kTJ + 1) * 32];
-    __shared__ uint32_t s_o[2 * kTI * 2 * kTJ];
-    __shared__ uint4 s_q[kTI * kTJ];  // per tile cell: visible_call_words
-    __shared__ int s_bos[32];         // rung of each replica slot
-    const Geometry& g = a.g;
-    const int L = g.L, Lc = g.Lc, W = g.W, Wc = g.Wc, N = g.N;
-    const int w = blockIdx.y;
-    const int tiles_j = (Wc + kTJ - 1) / kTJ;
-    const int i0 = (blockIdx.x / tiles_j) * kTI, j0 = (blockIdx.x % tiles_j) * kTJ;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-    const uint4* gt = reinterpret_cast<const uint4*>(a.ctab + static_cast<size_t>(w) * kCanonTab + kCanonTh);
-    for (int x = threadIdx.x; x < 4 * 32 * 32 / 4; x += blockDim.x) reinterpret_cast<uint4*>(s_tv)[x] = gt[x];
-    constexpr int HS = kTJ + 1;
-    if (W > kTI && Wc > kTJ)
-        stage_hidden_halo<true>(a, w, i0, j0, s_h);
-    else
-        stage_hidden_halo<false>(a, w, i0, j0, s_h);
-    stage_rungs(a, w, s_bos);
     const uint32_t chain = static_cast<uint32_t>(w) * 32u + lane;
     const Round0Lane r0l = round0_lane(chain);
     const Round1Sweep rs = round1_sweep(r0l.hi ^ t ^ a.rk[0], a.rk);
-    constexpr int VO = 2 * kTJ;
-    const int ni = min(kTI, W - i0), nj = min(kTJ, Wc - j0);
-    for (int x = threadIdx.x; x < kTI * kTJ; x += blockDim.x) {
-        const int li = x / kTJ, lj = x - li * kTJ;
-        if (li < ni && lj < nj) {
-            const uint32_t cell = static_cast<uint32_t>((i0 + li) * Wc + j0 + lj);
-            s_q[x] = kPaper ? visible_call_words_paper(cell, a.rk) : visible_call_words(cell, a.rk);
+    __syncthreads();
+    const uint32_t tab8 = tab + 8u * static_cast<uint32_t>(s_bos[lane]), tab4 = tab + 4u * static_cast<uint32_t>(s_bos[lane]);
+    const uint32_t row_lane = rows + 4u * static_cast<uint32_t>(lane);
+    uint32_t* hw = a.h + static_cast<size_t>(w) * g.n_cells * 32 + lane;
+    for (int u = warp; u < tile.ni * tile.nseg; u += nwarp) {
+        int r, s, n;
+        tile.segment(u, r, s, n);
+        Windows win(lds32(row_lane + 128u * static_cast<uint32_t>(u)), lds32(row_lane + 128u * static_cast<uint32_t>(u + tile.nseg)), n);
+        const uint32_t q = calls + 96u * static_cast<uint32_t>(u);  // (three cells per segment)
+        uint32_t* h = hw + static_cast<size_t>((tile.i0 + r) * g.Wc + tile.j0 + 3 * s) * 32;
+        auto one = [&](auto jc) {
+            constexpr int j = decltype(jc)::value;
+            const HiddenThresholds th(win, tab8, tab4);
+            const uint4 q0 = lds128<32 * j>(q), q1 = lds128<32 * j + 16>(q);
+            uint2 vis;
+            h[32 * j] = kPaper ? hidden_row_cell_paper(th, q0, q1, rs, r0l.lo, a.rk, vis)
+                               : hidden_row_cell<false>(th, q0, q1, rs, r0l.lo, a.rk);
+            win.next();
+        };
+        one(Cell<0>());
+        if (n > 1) {
+            one(Cell<1>());
+            if (n > 2) one(Cell<2>());
         }
     }
-    __syncthreads();
-    const LaneConst lc = lane_const(lane, s_bos[lane]);
-    for (int lj = warp; lj < nj; lj += nwarp) {
-        const uint32_t* ho = s_h + (HS + lj + 1) * 32 + lane;
-        uint32_t* o = s_o + 2 * lj;
-        const uint4* q = s_q + lj;
-        for (int li = 0; li < ni; ++li, ho += HS * 32, o += 2 * VO, q += kTJ) {
-            if (kPaper)
-                visible_cell_paper(o, VO, ho[0], ho[-HS * 32], ho[-32], s_tv, rs, r0l.lo, *q, a.rk, lc);
-            else
-                visible_cell(o, VO, ho[0], ho[-HS * 32], ho[-32], s_tv, rs, r0l.lo, *q, a.rk, lc);
-        }
+}
+
+// Dynamic shared memory of the visible half-step: rungs, the visible tables (at
+// shared address 4096: their loads merge the index by OR), the hidden words of
+// the tile with the row above and the column to the left, the call words.
+constexpr int kVisTabByte = 4096 - kReservedSmem, kVisWordByte = kVisTabByte + 16384;
+__host__ __device__ inline int vis_call_byte(int tile_seg) { return kVisWordByte + 128 * (kTI + 1) * (3 * tile_seg + 1); }
+__host__ __device__ inline int vis_smem(int tile_seg) { return vis_call_byte(tile_seg) + 16 * kTI * 3 * tile_seg; }
+
+// Visible half-step of one tile: hidden words in, new spins out.  Three CTAs per
+// SM (its shared memory) leave room for 80 registers a thread, which the three
+// calls of a segment side by side use.
+template <bool kPaper>
+__global__ void __launch_bounds__(kStreamVisThreads, 3) k_stream_visible(const SweepArgs a, uint32_t t, RowCut cut) {
+    extern __shared__ __align__(128) char smem[];
+    const Geometry& g = a.g;
+    const int w = blockIdx.y, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);
+    constexpr int nwarp = kStreamVisThreads / 32;
+    const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(smem)), tab = base + kVisTabByte;
+    if (tab & 4095u) return;  // (the launcher has checked it)
+    const RowTile tile(g, blockIdx.x, cut);
+    int* s_bos = reinterpret_cast<int*>(smem);
+    stage_rungs(a, w, s_bos);
+    auto copy16 = [](uint32_t dst, const uint4* src) {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+    };
+    // hidden words of cells (i0 - 1 .. i0 + ni - 1) x (j0 - 1 .. j0 + nj - 1), wrapped; tile row 0 and
+    // column 0 are the halo
+    const uint32_t words = base + kVisWordByte, wrow = 128u * static_cast<uint32_t>(3 * cut.seg + 1);
+    const uint4* hw = reinterpret_cast<const uint4*>(a.h + static_cast<size_t>(w) * g.n_cells * 32);
+    const int iu = tile.i0 > 0 ? tile.i0 - 1 : g.W - 1, jl = tile.j0 > 0 ? tile.j0 - 1 : g.Wc - 1;
+    for (int r = warp; r <= tile.ni; r += nwarp) {
+        const uint4* row = hw + static_cast<size_t>((r > 0 ? tile.i0 + r - 1 : iu) * g.Wc) * 8;
+        const uint32_t dst = words + wrow * static_cast<uint32_t>(r);
+        if (lane < 8) copy16(dst + 16u * static_cast<uint32_t>(lane), row + jl * 8 + lane);
+        for (int x = lane; x < 8 * tile.nj; x += 32) copy16(dst + 128u + 16u * static_cast<uint32_t>(x), row + tile.j0 * 8 + x);
     }
+    const uint4* gt = reinterpret_cast<const uint4*>(a.ctab + static_cast<size_t>(w) * kCanonTab + kCanonTh);
+    for (int x = threadIdx.x; x < 4 * 32 * 32 / 4; x += kStreamVisThreads) copy16(tab + 16u * static_cast<uint32_t>(x), gt + x);
+    const uint32_t calls = base + static_cast<uint32_t>(vis_call_byte(cut.seg));
+    for (int x = threadIdx.x; x < tile.ni * 3 * tile.nseg; x += kStreamVisThreads) {
+        const int r = x / (3 * tile.nseg), c = x - r * 3 * tile.nseg;
+        if (c < tile.nj)
+            reinterpret_cast<uint4*>(smem + vis_call_byte(cut.seg))[x] =
+                visible_call_words(static_cast<uint32_t>((tile.i0 + r) * g.Wc + tile.j0 + c), kPaper ? 1u : kTagVis, a.rk);
+    }
+    const uint32_t chain = static_cast<uint32_t>(w) * 32u + lane;
+    const Round0Lane r0l = round0_lane(chain);
+    const Round1Sweep rs = round1_sweep(r0l.hi ^ t ^ a.rk[0], a.rk);
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    for (int x = threadIdx.x; x < 2 * kTI * VO; x += blockDim.x) {
-        const int r = x / VO, c = x - (x / VO) * VO;
-        const int R = 2 * i0 + r, C = 2 * j0 + c;
-        if (R >= L || C >= Lc) continue;
-        a.v[vidx(w, N, R * Lc + C)] = s_o[x];
+    const uint32_t tab4 = tab + 4u * static_cast<uint32_t>(s_bos[lane]);
+    uint32_t* vw = a.v + vidx(w, g.N, 0);
+    const Transpose32 transpose(lane);
+    const SegmentSites site(g.Lc, lane);
+    for (int u = warp; u < tile.ni * tile.nseg; u += nwarp) {
+        int r, s, n;
+        tile.segment(u, r, s, n);
+        const uint32_t q = calls + 48u * static_cast<uint32_t>(u);
+        const uint32_t own = words + wrow * static_cast<uint32_t>(r + 1) + 128u * static_cast<uint32_t>(3 * s + 1) + 4u * static_cast<uint32_t>(lane);
+        uint32_t left = lds32(own - 128u), o = 0u;
+        auto draw = [&](auto jc) {
+            const U4 x = visible_draw(lds128<16 * decltype(jc)::value>(q), rs, r0l.lo, a.rk);
+            return kPaper ? U4{x.y << 16, x.y, x.z << 16, x.z} : x;
+        };
+        auto decide = [&](auto jc, const U4& x) {
+            constexpr uint32_t off = 128u * decltype(jc)::value;
+            const uint32_t wo = lds32(own + off);
+            o = visible_row_cell<0>(merge_words(wo, lds32(own + off - wrow), left), x, tab4, o);
+            left = wo;
+        };
+        if (n == 3) {  // the three calls side by side
+            const U4 x0 = draw(Cell<0>()), x1 = draw(Cell<1>()), x2 = draw(Cell<2>());
+            decide(Cell<0>(), x0);
+            decide(Cell<1>(), x1);
+            decide(Cell<2>(), x2);
+        } else {
+            decide(Cell<0>(), draw(Cell<0>()));
+            if (n > 1) decide(Cell<1>(), draw(Cell<1>()));
+        }
+        const uint32_t v = transpose(o << 16);  // lane = bit: a site's word
+        const int j = tile.j0 + 3 * s;
+        if (lane >= 16 && lane < 16 + 4 * n) vw[2 * site(lane, tile.i0 + r, j, n, j + n)] = v;
     }
 }
 
@@ -368,7 +426,7 @@ __global__ void __launch_bounds__(kStreamThreads) k_stream_bp_hidden(const Sweep
 
 // Visible half-step of one tile: the hidden words of the tile's cells and of
 // the row above and the column to the left (wrapped) in, new spins out.
-__global__ void __launch_bounds__(kStreamVisThreads, CRBM_STREAM_MIN_BLOCKS) k_stream_bp_visible(const SweepArgs a, uint32_t t) {
+__global__ void __launch_bounds__(kStreamVisThreads, kStreamMinBlocks) k_stream_bp_visible(const SweepArgs a, uint32_t t) {
     constexpr int HS = kTJ + 1;
     __shared__ __align__(16) uint32_t s_tab[kBpTab];
     __shared__ uint32_t s_h[(kTI + 1) * HS * 10];
@@ -499,25 +557,25 @@ __global__ void __launch_bounds__(kStreamVisThreads, CRBM_STREAM_MIN_BLOCKS) k_s
 }
 
 // Measurement counts of one tile (anti-aligned J / J' filters and +1 spins
-// per chain), summed over the CTA in shared memory, then into cnt[chain][3].
-__global__ void __launch_bounds__(kStreamThreads, CRBM_STREAM_MIN_BLOCKS) k_stream_count(const SweepArgs a) {
-    __shared__ uint32_t s_v[(2 * kTI + 1) * (2 * kTJ + 1)];
+// per chain) from its rows, summed over the CTA in shared memory, then into
+// cnt[chain][3].
+__global__ void __launch_bounds__(kStreamThreads) k_stream_count(const SweepArgs a, RowCut cut) {
+    __shared__ uint32_t s_rows[(kTI + 1) * kMaxTileSeg * 32];
     __shared__ int s_cnt[96];
-    const Geometry& g = a.g;
-    const int W = g.W, Wc = g.Wc;
-    const int w = blockIdx.y;
-    const int tiles_j = (Wc + kTJ - 1) / kTJ;
-    const int i0 = (blockIdx.x / tiles_j) * kTI, j0 = (blockIdx.x % tiles_j) * kTJ;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-    constexpr int VS = 2 * kTJ + 1;
-    stage_spin_tile(a, w, i0, j0, s_v);
-    for (int x = threadIdx.x; x < 96; x += blockDim.x) s_cnt[x] = 0;
+    const int w = blockIdx.y, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);
+    const RowTile tile(a.g, blockIdx.x, cut);
+    const uint32_t rows = static_cast<uint32_t>(__cvta_generic_to_shared(s_rows));
+    if (threadIdx.x < 96) s_cnt[threadIdx.x] = 0;
+    stage_rows(a, w, tile, rows, warp, lane);
     __syncthreads();
     int anti0 = 0, anti1 = 0, pos = 0;
-    const int ni = min(kTI, W - i0), nj = min(kTJ, Wc - j0);
-    for (int lj = warp; lj < nj; lj += nwarp)
-        for (int li = 0; li < ni; ++li)
-            count_cell(s_v + 2 * li * VS + 2 * lj, 0, VS, 2 * VS, 0, 1, 2, lane, anti0, anti1, pos);
+    for (int u = warp; u < tile.ni * tile.nseg; u += kStreamThreads / 32) {
+        int r, s, n;
+        tile.segment(u, r, s, n);
+        const uint32_t x = rows + 128u * static_cast<uint32_t>(u) + 4u * static_cast<uint32_t>(lane);
+        count_segment(lds32(x), lds32(x + 128u * static_cast<uint32_t>(tile.nseg)), n, anti0, anti1, pos);
+    }
     atomicAdd(&s_cnt[lane], anti0);
     atomicAdd(&s_cnt[32 + lane], anti1);
     atomicAdd(&s_cnt[64 + lane], pos);
@@ -603,26 +661,38 @@ __global__ void __launch_bounds__(32) k_stream_post_pt(const SweepArgs a, int64_
 }  // namespace
 
 cudaError_t launch_sweep_stream(const SweepArgs& a, cudaStream_t st, int64_t* launches) {
-    const int tiles = ((a.g.W + kTI - 1) / kTI) * ((a.g.Wc + kTJ - 1) / kTJ);
-    const dim3 grid(tiles, a.n_words);
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const RowCut cut = row_cut(a.g, a.n_words, sms);
+    const dim3 grid(((a.g.W + kTI - 1) / kTI) * ((a.g.Wc + kTJ - 1) / kTJ), a.n_words);  // bit-plane tiles
+    const dim3 row_grid(((a.g.W + cut.rows - 1) / cut.rows) * ((a.g.Wc + 3 * cut.seg - 1) / (3 * cut.seg)), a.n_words);
+    const auto hidden = a.g.paper ? k_stream_hidden<true> : k_stream_hidden<false>;
+    const auto visible = a.g.paper ? k_stream_visible<true> : k_stream_visible<false>;
+    if (!a.g.bitplane && a.n_sweeps > 0) {
+        int reserved = 0;
+        e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
+        if (e == cudaSuccess && reserved != kReservedSmem) e = cudaErrorInvalidConfiguration;
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(hidden, cudaFuncAttributeMaxDynamicSharedMemorySize, kHidSmem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(visible, cudaFuncAttributeMaxDynamicSharedMemorySize, vis_smem(kMaxTileSeg));
+        if (e != cudaSuccess) return e;
+    }
     int64_t meas = a.meas0;
     for (int it = 0; it < a.n_sweeps; ++it) {
         const uint32_t t = a.t0 + static_cast<uint32_t>(it);
         if (a.g.bitplane) {
             k_stream_bp_hidden<<<grid, kStreamThreads, 0, st>>>(a, t);
             k_stream_bp_visible<<<grid, kStreamVisThreads, 0, st>>>(a, t);
-        } else if (a.g.paper) {
-            k_stream_hidden<true><<<grid, kStreamThreads, 0, st>>>(a, t);
-            k_stream_visible<true><<<grid, kStreamVisThreads, 0, st>>>(a, t);
         } else {
-            k_stream_hidden<false><<<grid, kStreamThreads, 0, st>>>(a, t);
-            k_stream_visible<false><<<grid, kStreamVisThreads, 0, st>>>(a, t);
+            hidden<<<row_grid, kStreamThreads, kHidSmem, st>>>(a, t, cut);
+            visible<<<row_grid, kStreamVisThreads, vis_smem(cut.seg), st>>>(a, t, cut);
         }
         *launches += 2;
         const bool do_meas = a.measure_every > 0 && (t + 1u) % static_cast<uint32_t>(a.measure_every) == 0u;
         const bool do_swap = a.swap_every > 0 && (t + 1u) % static_cast<uint32_t>(a.swap_every) == 0u;
         if (do_meas || do_swap) {
-            k_stream_count<<<grid, kStreamThreads, 0, st>>>(a);
+            k_stream_count<<<row_grid, kStreamThreads, 0, st>>>(a, cut);
             if (a.swap_every > 0)
                 k_stream_post_pt<<<a.n_words, 32, 0, st>>>(a, meas, t, do_meas ? 1 : 0, do_swap ? 1 : 0);
             else
@@ -631,7 +701,7 @@ cudaError_t launch_sweep_stream(const SweepArgs& a, cudaStream_t st, int64_t* la
             *launches += 2;
             if (do_meas) ++meas;
         }
-        const cudaError_t e = cudaGetLastError();
+        e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
