@@ -9,6 +9,8 @@
 // a broadcast, and each lane only extracts its own bit, draws its own Philox
 // words and compares against its own threshold column; __ballot_sync packs
 // the 32 decisions back into one word.  Everything is integer arithmetic.
+#include <algorithm>
+
 #include "crbm_generic_body.cuh"
 
 namespace crbm {
@@ -37,14 +39,36 @@ __global__ void k_init(const Geometry g, uint32_t* v, int n_words, uint32_t k0, 
     }
 }
 
+// Spins as int8, [chain][site].  A warp takes 128 sites of a packed word: lane l
+// loads the words of sites 4 l .. 4 l + 3 and writes, chain by chain, their four
+// bytes, 128 bytes a row (N a multiple of 4, as every even lattice's; other
+// lattices write byte by byte).  Bound by the write: 113 MB in 200 us with a
+// thread per byte, two 64-bit divisions and a byte store each, 25 now.
 __global__ void k_unpack(const Geometry g, const uint32_t* v, int8_t* out, int n_words) {
-    const long long total = static_cast<long long>(n_words) * 32 * g.N;
-    for (long long x = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; x < total;
-         x += static_cast<long long>(gridDim.x) * blockDim.x) {
-        const long long chain = x / g.N;
-        const int s = static_cast<int>(x - chain * g.N);
-        const uint32_t w = v[word_index(g.vil, static_cast<int>(chain >> 5), g.N, s)];
-        out[x] = ((w >> (chain & 31)) & 1u) ? 1 : -1;
+    const int lane = threadIdx.x & 31, N = g.N, blocks = (N + 127) / 128;
+    const long long n = static_cast<long long>(n_words) * blocks, step = static_cast<long long>(gridDim.x) * (blockDim.x >> 5);
+    const bool by4 = N % 4 == 0;
+    for (long long x = blockIdx.x * static_cast<long long>(blockDim.x >> 5) + (threadIdx.x >> 5); x < n; x += step) {
+        const int word = static_cast<int>(x / blocks), s0 = static_cast<int>(x - static_cast<long long>(word) * blocks) * 128;
+        uint32_t w[4];
+        int site[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            site[k] = by4 ? s0 + 4 * lane + k : s0 + lane + 32 * k;
+            w[k] = site[k] < N ? v[word_index(g.vil, word, N, site[k])] : 0u;
+        }
+        int8_t* o = out + static_cast<size_t>(word) * 32 * N;
+#pragma unroll 4
+        for (int c = 0; c < 32; ++c, o += N) {
+            if (by4) {  // bytes 0xFF, or 0x01 where the bit is set
+                const uint32_t b = ((w[0] >> c) & 1u) | ((w[1] >> c) & 1u) << 8 | ((w[2] >> c) & 1u) << 16 | ((w[3] >> c) & 1u) << 24;
+                if (site[0] < N) *reinterpret_cast<uint32_t*>(o + site[0]) = ~(b * 0xFEu);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (site[k] < N) o[site[k]] = ((w[k] >> c) & 1u) ? 1 : -1;
+            }
+        }
     }
 }
 
@@ -146,8 +170,8 @@ cudaError_t launch_sweep_generic(const SweepArgs& a, int warps_per_cta, cudaStre
 
 cudaError_t launch_unpack(const Geometry& g, const uint32_t* v, int8_t* out, int n_words,
                           cudaStream_t st) {
-    const long long total = static_cast<long long>(n_words) * 32 * g.N;
-    const int blocks = static_cast<int>((total + 255) / 256 < 152 * 32 ? (total + 255) / 256 : 152 * 32);
+    const long long warps = static_cast<long long>(n_words) * ((g.N + 127) / 128);
+    const int blocks = static_cast<int>(std::min<long long>((warps + 7) / 8, 152 * 32));
     k_unpack<<<blocks, 256, 0, st>>>(g, v, out, n_words);
     return cudaGetLastError();
 }
