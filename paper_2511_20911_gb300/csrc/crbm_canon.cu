@@ -115,6 +115,14 @@ __global__ void __launch_bounds__(kMaxThreads, kMaxThreads == kCtaPair ? 2 : CRB
     }
 }
 
+// Few words: each word's rows of cells split into bands over a cluster of
+// a.n_bands CTAs, so that words that would hold an SM each use up to eight.
+template <int kMode, bool kPaper>
+__global__ void __launch_bounds__(kCtaWide, 1) k_sweep_canon_split(const SweepArgs a) {
+    const int nb = a.n_bands, word = static_cast<int>(blockIdx.x) / nb;
+    sweep_canon_body<kMode, true, kPaper>(a, word, a.t0, a.n_sweeps, a.meas0, static_cast<int>(blockIdx.x) - word * nb, 0);
+}
+
 }  // namespace
 
 size_t smem_bytes_canon(const Geometry& g) {
@@ -202,7 +210,53 @@ PersistentKernel persistent_kernel(int mode, int paper, int cta) {
                              : persistent_kernel<kCtaAny>(mode, paper);
 }
 
-cudaError_t make_plan(const Geometry& g0, int n_words, int warps, int dev, CanonLaunch& p) {
+using SplitKernel = void (*)(const SweepArgs);
+SplitKernel split_kernel(int mode, int paper) {
+    if (paper)
+        return mode == kCanonRec     ? k_sweep_canon_split<kCanonRec, true>
+               : mode == kCanonPlain ? k_sweep_canon_split<kCanonPlain, true>
+                                     : k_sweep_canon_split<kCanonPacked, true>;
+    return mode == kCanonRec     ? k_sweep_canon_split<kCanonRec, false>
+           : mode == kCanonPlain ? k_sweep_canon_split<kCanonPlain, false>
+                                 : k_sweep_canon_split<kCanonPacked, false>;
+}
+cudaLaunchConfig_t split_config(int n_words, int bands, int warps, size_t smem, cudaLaunchAttribute* attr) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(static_cast<unsigned int>(n_words * bands));
+    c.blockDim = dim3(static_cast<unsigned int>(32 * warps));
+    c.dynamicSmemBytes = smem;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = static_cast<unsigned int>(bands);
+    attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+    c.attrs = attr;
+    c.numAttrs = 1;
+    return c;
+}
+
+// The bands a word is split into: the most (a power of two up to 8) with which
+// every cluster is resident at once, an SM per CTA, and a band has at least 20
+// cells (below that the cluster barriers cost more than the cells they save:
+// L = 12 in two bands 2.2 us per sweep, whole 2.1).  1: no split.  Correlations
+// need the whole lattice in one CTA.
+int pick_bands(const Geometry& g0, int n_words, int warps, int sms, bool correlations) {
+    if (correlations || 32 * warps > kCtaWide) return 1;
+    for (int nb = 8; nb > 1; nb /= 2) {
+        if (nb > g0.W || g0.n_cells < 20 * nb || n_words * nb > sms) continue;
+        Geometry g = g0;
+        int mode = 0, clusters = 0;
+        const size_t smem = canon_plan(g, warps, &mode, nb);
+        const SplitKernel k = split_kernel(mode, g.paper);
+        cudaLaunchAttribute attr;
+        const cudaLaunchConfig_t c = split_config(n_words, nb, warps, smem, &attr);
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) == cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&clusters, k, &c) == cudaSuccess && clusters >= n_words)
+            return nb;
+        cudaGetLastError();  // (not sticky: no split of this size)
+    }
+    return 1;
+}
+
+cudaError_t make_plan(const Geometry& g0, int n_words, int warps, int dev, bool correlations, CanonLaunch& p) {
     Geometry g = g0;
     p = CanonLaunch();
     p.smem = canon_plan(g, warps, &p.mode);
@@ -212,6 +266,15 @@ cudaError_t make_plan(const Geometry& g0, int n_words, int warps, int dev, Canon
     cudaError_t e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&p.sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
+    p.bands = pick_bands(g, n_words, warps, p.sms, correlations);
+    if (p.bands > 1 && reserved == kReservedSmem) {
+        p.smem = canon_plan(g, warps, &p.mode, p.bands);
+        p.seg_cells = g.seg_cells;
+        p.n_seg = g.n_seg;
+        p.warps = warps;
+        p.device = dev;
+        return cudaSuccess;
+    }
     auto occupancy = [&](int cta, int* per_sm) {
         const PersistentKernel k = persistent_kernel(p.mode, g.paper, cta);
         // (always the most a CTA can have: contexts of other sizes share the kernel)
@@ -247,11 +310,18 @@ cudaError_t launch_sweep_canon_persistent(const SweepArgs& a0, int warps_per_cta
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess && (plan.warps != warps_per_cta || plan.device != dev))
-        e = make_plan(a0.g, a0.n_words, warps_per_cta, dev, plan);
+        e = make_plan(a0.g, a0.n_words, warps_per_cta, dev, a0.sq_every > 0, plan);
     if (e != cudaSuccess) return e;
     SweepArgs a = a0;
     a.g.seg_cells = plan.seg_cells;
     a.g.n_seg = plan.n_seg;
+    if (plan.bands > 1) {
+        a.n_bands = plan.bands;
+        cudaLaunchAttribute attr;
+        cudaLaunchConfig_t c = split_config(a.n_words, plan.bands, warps_per_cta, plan.smem, &attr);
+        c.stream = st;
+        return cudaLaunchKernelEx(&c, split_kernel(plan.mode, a.g.paper), a);
+    }
     // no more CTAs per SM than whole words: were every word held at once, SMs with one word more
     // than others would finish last with nothing to claim for the rest
     const int per_sm = std::max(1, std::min(plan.per_sm, a.n_words / plan.sms));

@@ -261,7 +261,7 @@ int default_warps(const Geometry& g, int n_words) {
                                     g.n_cells));
     if (n_words >= 2 * sms && g.n_cells <= 400)  // (larger ones hold one CTA per SM)
         return std::min(kMaxSweepWarps, g.n_cells < 16 ? 4 : g.n_cells < 30 || (g.n_cells >= 50 && g.n_cells <= 144) ? 8 : 12);
-    return std::min(kMaxSweepWarps, g.n_cells < 8 ? 8 : g.n_cells <= 16 ? 12 : g.n_cells <= 600 ? 16 : 32);
+    return std::min(kMaxSweepWarps, g.n_cells < 8 ? 8 : g.n_cells <= 16 ? 12 : g.n_cells <= 600 || 2 * n_words <= sms ? 16 : 32);
 }
 
 }  // namespace

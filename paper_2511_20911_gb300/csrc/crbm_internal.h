@@ -291,7 +291,7 @@ size_t canon_plan(Geometry& g, int warps, int* mode, int bands = 1);
 // A launch's choices, kept by the context between calls of the same shape.
 struct CanonLaunch {
     int warps = 0, device = -1;  // what they were made for
-    int mode = 0, seg_cells = 0, n_seg = 0, cta = 0, per_sm = 0, sms = 0;
+    int mode = 0, seg_cells = 0, n_seg = 0, cta = 0, per_sm = 0, sms = 0, bands = 1;
     size_t smem = 0;
 };
 cudaError_t launch_init(const Geometry& g, uint32_t* v, int n_words, uint32_t key0,

@@ -1,7 +1,9 @@
 """The canonical SMEM sweep's row form (segments of one to three cells of a row
 of cells per word, crbm_row_core.cuh) against the oracle, bit for bit: rows cut
 into segments of every length, one segment per row (its own right neighbour), and
-the lattices whose hidden words or visible draws are kept in their smaller forms."""
+the lattices whose hidden words or visible draws are kept in their smaller forms;
+with two words (split into bands over a cluster from 40 cells up) and with 80
+(a CTA each)."""
 import numpy as np
 import pytest
 
@@ -39,15 +41,37 @@ def check(orc, L, Lc, precision, n, splits, warps, monkeypatch):
 
 
 # one segment per row (4, 6 columns), segments of 2 + 2, 3 + 2, 3 + 3 + 1 cells and of single cells (many warps)
+@pytest.mark.parametrize("n", [37, 2530])
 @pytest.mark.parametrize("precision", [EXACT, PAPER])
 @pytest.mark.parametrize("L,Lc,warps", [(4, 4, 1), (4, 6, 3), (6, 4, 9), (8, 8, 2), (8, 10, 4), (10, 14, 5), (14, 10, 32),
                                         (30, 22, 8)])
-def test_segment_lengths(orc, L, Lc, warps, precision, monkeypatch):
-    check(orc, L, Lc, precision, 37, [1, 6], warps, monkeypatch)
+def test_segment_lengths(orc, L, Lc, warps, precision, n, monkeypatch):
+    check(orc, L, Lc, precision, n, [1, 6], warps, monkeypatch)
 
 
 # records from global memory (64 x 64, 18 x 96: long rows), 16-bit hidden words (68, 76), visible draws made twice (38 x 52)
+@pytest.mark.parametrize("n", [33, 2530])
 @pytest.mark.parametrize("L,Lc,precision", [(64, 64, EXACT), (18, 96, EXACT), (68, 68, EXACT), (76, 76, EXACT),
                                             (56, 96, EXACT), (38, 52, PAPER), (18, 96, PAPER)])
-def test_large_lattices(orc, L, Lc, precision, monkeypatch):
-    check(orc, L, Lc, precision, 33, [3], 16, monkeypatch)
+def test_large_lattices(orc, L, Lc, precision, n, monkeypatch):
+    check(orc, L, Lc, precision, n, [2], 16, monkeypatch)
+
+
+@pytest.mark.parametrize("ladders,precision", [(1, EXACT), (3, PAPER), (17, EXACT)])
+def test_split_ladders_match_whole_words(orc, ladders, precision):
+    """Few ladders run split over clusters; the same ladders as members of a context of 96 run whole."""
+    L, n = 18, 32 * ladders
+    beta = list(0.25 * 32.0 ** (np.arange(32) / 31.0))
+    params = dict(J=[1.0] * 32, Jp=[1.5] * 32, h=[1.0] * 32, beta=beta)
+    kw = dict(seed=5, measure_every=1, swap_every=2, series_len=6, precision=precision)
+    few = crbm.Sampler(L, params, n, chain_param=np.tile(np.arange(32), ladders).astype(np.int32), **kw)
+    many = crbm.Sampler(L, params, 32 * 96, chain_param=np.tile(np.arange(32), 96).astype(np.int32), **kw)
+    for s in (few, many):
+        s.set_targets([-16 * L * L] * 32)
+        s.sweep(5)
+        s.sweep(4)
+    assert np.array_equal(few.get_spins(), many.get_spins()[:n])
+    assert np.array_equal(few.observables(), many.observables()[:n])
+    assert np.array_equal(few.series(), many.series()[:, :n])
+    assert np.array_equal(few.permutation(), many.permutation()[:n])
+    assert np.array_equal(few.first_hits(), many.first_hits()[:n])
