@@ -7,9 +7,9 @@
 // Philox((cell, sweep, word, kTagBitplane + 8 node + j)), four planes per
 // call, most significant plane first.  The thresholds are held the same way
 // (per word, one bit-plane word per configuration and plane), so the 32
-// comparisons u_l < t_l run as one word-parallel comparison, most significant
-// bit first: a chain is decided at the first plane where its uniform and
-// threshold bits differ (below when the threshold bit is the 1).  Every node
+// comparisons u_l < t_l run as one word-parallel comparison: a chain is
+// decided by the most significant plane where its uniform and threshold bits
+// differ (below when the threshold bit is the 1).  Every node
 // draws two calls (eight planes); the nodes with chains still open after them
 // (about 12 %) go to a straggler list, which the CTA's warps then take 32 at a
 // time, drawing further calls while any of a warp's stragglers is open.  The

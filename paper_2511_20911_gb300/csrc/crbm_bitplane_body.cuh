@@ -105,10 +105,9 @@ __device__ __forceinline__ void sweep_bitplane_body(const SweepArgs& a, const ui
             fl1 = s_tab[kBpFlip + 1];
         }
         // hidden half-step (Eq. 9): thread = hidden node (cell, k).  Its endpoints select per chain
-        // the threshold planes of m = e1 + s e2 (P: m = 2, M: m = -2, Z: m = 0, whose threshold 2^31
-        // has only plane 0 set)
+        // the threshold planes of m = e1 + s e2 (Z: the chains with m = 0)
         struct Hid {
-            uint32_t P, M, Z, c2;
+            uint32_t e1, Z, c2;
             const uint32_t* tp;
             Round2Cell r2;
         };
@@ -120,7 +119,7 @@ __device__ __forceinline__ void sweep_bitplane_body(const SweepArgs& a, const ui
             const uint32_t e1 = s_v[r & 0xFFFFu];
             const uint32_t e2 = s_v[r >> 16] ^ (cls ? fl1 : fl0);
             const uint64_t pc = static_cast<uint64_t>(kPhiloxM0) * cell;
-            return Hid{e1 & e2, ~(e1 | e2), e1 ^ e2,
+            return Hid{e1, e1 ^ e2,
                        static_cast<uint32_t>(pc >> 32) ^ a.rk[1] ^ (kTagBitplane + 8u * k),
                        s_tab + kBpHidPlanes + cls * 96u, round2_cell(rs.hik ^ static_cast<uint32_t>(pc))};
         };
@@ -128,20 +127,18 @@ __device__ __forceinline__ void sweep_bitplane_body(const SweepArgs& a, const ui
             const int node = base + lane;
             const bool valid = node < nh;
             const Hid hn = hidden_node(valid ? node : 0);
-            uint32_t lt = 0u, eq = valid ? 0xffffffffu : 0u;
-            auto planes = [&](const U4& q, uint32_t j) {
-                bp::hidden_planes(q, hn.tp + 4u * j, hn.P, hn.M, j == 0u ? hn.Z : 0u, lt, eq);
-            };
+            uint32_t lt, eq;
             // calls 0 and 1 together, then the open nodes to the straggler list
             const U4 q0 = philox_from_round2(Yw, rs, hn.r2, hn.c2, a.rk);
             const U4 q1 = philox_from_round2(Yw, rs, hn.r2, hn.c2 ^ 1u, a.rk);
-            planes(q0, 0u);
-            planes(q1, 1u);
+            hidden_first(q0, q1, hn.tp, hn.e1, hn.Z, lt, eq);
+            eq = valid ? eq : 0u;
             if (push_straggler(static_cast<uint32_t>(node), eq, s_nst, s_list, cap, lane)) eq = 0u;
 #pragma unroll 1
             for (uint32_t j = 2; j < 8u; ++j) {  // only where the list was full
                 if (!__any_sync(0xffffffffu, eq != 0u)) break;
-                planes(philox_from_round2(Yw, rs, hn.r2, hn.c2 ^ j, a.rk), j);
+                planes_below(philox_from_round2(Yw, rs, hn.r2, hn.c2 ^ j, a.rk), hidden_planes(hn.tp + 4u * j, hn.e1), lt,
+                             eq);
             }
             if (valid) s_h[node] = lt;  // final, or the decided part of a straggler
         }
@@ -157,8 +154,8 @@ __device__ __forceinline__ void sweep_bitplane_body(const SweepArgs& a, const ui
 #pragma unroll 1
                 for (uint32_t j = 2; j < 8u; ++j) {
                     if (!__any_sync(0xffffffffu, eq != 0u)) break;
-                    bp::hidden_planes(philox_from_round2(Yw, rs, hn.r2, hn.c2 ^ j, a.rk), hn.tp + 4u * j, hn.P, hn.M,
-                                      0u, lt, eq);
+                    planes_below(philox_from_round2(Yw, rs, hn.r2, hn.c2 ^ j, a.rk),
+                                 hidden_planes(hn.tp + 4u * j, hn.e1), lt, eq);
                 }
                 if (valid) s_h[node] = lt;
             }
@@ -182,25 +179,23 @@ __device__ __forceinline__ void sweep_bitplane_body(const SweepArgs& a, const ui
                        bp::count4(h0, h1, h2, h3), round2_cell(rs.hik ^ static_cast<uint32_t>(pc))};
         };
         const uint32_t* tv = s_tab + kBpVisPlanes;  // [count][J' bit][32]
-        auto vis_planes = [&](const Vis& vn, const U4& q, uint32_t j, uint32_t& lt, uint32_t& eq) {
-            const uint4 T = bp::visible_planes(tv + 4u * j, vn.hp, vn.n4);
-            bp::plane_step(q.x, T.x, lt, eq);
-            bp::plane_step(q.y, T.y, lt, eq);
-            bp::plane_step(q.z, T.z, lt, eq);
-            bp::plane_step(q.w, T.w, lt, eq);
+        auto vis_below = [&](const Vis& vn, uint32_t j, uint32_t& lt, uint32_t& eq) {
+            planes_below(philox_from_round2(Yw, rs, vn.r2, vn.c2 ^ j, a.rk), visible_planes(tv + 4u * j, vn.hp, vn.n4), lt,
+                         eq);
         };
         for (int base = warp * 32; base < N; base += nwarp * 32) {
             const int sx = base + lane;
             const bool valid = sx < N;
             const Vis vn = visible_node(valid ? sx : 0);
-            uint32_t lt = 0u, eq = valid ? 0xffffffffu : 0u;
-            vis_planes(vn, philox_from_round2(Yw, rs, vn.r2, vn.c2, a.rk), 0u, lt, eq);
-            vis_planes(vn, philox_from_round2(Yw, rs, vn.r2, vn.c2 ^ 1u, a.rk), 1u, lt, eq);
+            uint32_t lt = 0u, ne = 0u;
+            planes_step(philox_from_round2(Yw, rs, vn.r2, vn.c2 ^ 1u, a.rk), visible_planes(tv + 4, vn.hp, vn.n4), lt, ne);
+            planes_step(philox_from_round2(Yw, rs, vn.r2, vn.c2, a.rk), visible_planes(tv, vn.hp, vn.n4), lt, ne);
+            uint32_t eq = valid ? ~ne : 0u;
             if (push_straggler(static_cast<uint32_t>(sx), eq, s_nst + 1, s_list, cap, lane)) eq = 0u;
 #pragma unroll 1
             for (uint32_t j = 2; j < 8u; ++j) {  // only where the list was full
                 if (!__any_sync(0xffffffffu, eq != 0u)) break;
-                vis_planes(vn, philox_from_round2(Yw, rs, vn.r2, vn.c2 ^ j, a.rk), j, lt, eq);
+                vis_below(vn, j, lt, eq);
             }
             if (valid) s_v[sx] = lt;  // no spin is read in this half-step
         }
@@ -216,7 +211,7 @@ __device__ __forceinline__ void sweep_bitplane_body(const SweepArgs& a, const ui
 #pragma unroll 1
                 for (uint32_t j = 2; j < 8u; ++j) {
                     if (!__any_sync(0xffffffffu, eq != 0u)) break;
-                    vis_planes(vn, philox_from_round2(Yw, rs, vn.r2, vn.c2 ^ j, a.rk), j, lt, eq);
+                    vis_below(vn, j, lt, eq);
                 }
                 if (valid) s_v[sx] = lt;
             }

@@ -11,13 +11,28 @@ namespace bp {
 using dev::transpose32;
 using dev::U4;
 
-// One plane of the comparison u < t, most significant bit first: lt collects
-// the chains found below, eq the chains whose uniform and threshold agree on
-// every plane so far (still open).  U, T: the plane of the uniforms and of
-// the thresholds.
-__device__ __forceinline__ void plane_step(uint32_t U, uint32_t T, uint32_t& lt, uint32_t& eq) {
-    lt |= eq & T & ~U;
-    eq &= ~(T ^ U);
+// One plane of the comparison u < t, least significant bit first: lt collects
+// the chains with u < t on the planes so far (the borrow of u - t), ne the
+// chains with u != t there.  One LOP3 each; the other direction carries the
+// open chains from plane to plane and takes three.  U, T: the plane of the
+// uniforms and of the thresholds.
+__device__ __forceinline__ void plane_step(uint32_t U, uint32_t T, uint32_t& lt, uint32_t& ne) {
+    lt = (~U & T) | (~(U ^ T) & lt);
+    ne |= U ^ T;
+}
+__device__ __forceinline__ void planes_step(const U4& q, const uint4& T, uint32_t& lt, uint32_t& ne) {
+    plane_step(q.w, T.w, lt, ne);
+    plane_step(q.z, T.z, lt, ne);
+    plane_step(q.y, T.y, lt, ne);
+    plane_step(q.x, T.x, lt, ne);
+}
+// The planes of a further call, below those compared so far: eq, the chains
+// that agree on all of them, are decided by it where they differ.
+__device__ __forceinline__ void planes_below(const U4& q, const uint4& T, uint32_t& lt, uint32_t& eq) {
+    uint32_t l = 0u, ne = 0u;
+    planes_step(q, T, l, ne);
+    lt |= eq & l;
+    eq &= ~ne;
 }
 
 // Four consecutive threshold planes of one row: the planes of one Philox
@@ -25,17 +40,27 @@ __device__ __forceinline__ void plane_step(uint32_t U, uint32_t T, uint32_t& lt,
 // boundary and calls on a multiple of four planes).
 __device__ __forceinline__ uint4 planes4(const uint32_t* p) { return *reinterpret_cast<const uint4*>(p); }
 
-// The four planes of one Philox call of a hidden node: P, M select the chains
-// with m = 2 and m = -2, tb points at the call's first plane of the m = -2 row
-// (m = 2 row 64 words further); Z0 = the chains with m = 0 on the first call
-// (their threshold 2^31 has only its top plane set), 0 on later calls.
-__device__ __forceinline__ void hidden_planes(const U4& q, const uint32_t* tb, uint32_t P, uint32_t M, uint32_t Z0,
-                                              uint32_t& lt, uint32_t& eq) {
-    const uint4 tm = planes4(tb), tp = planes4(tb + 64);
-    plane_step(q.x, (P & tp.x) | (M & tm.x) | Z0, lt, eq);
-    plane_step(q.y, (P & tp.y) | (M & tm.y), lt, eq);
-    plane_step(q.z, (P & tp.z) | (M & tm.z), lt, eq);
-    plane_step(q.w, (P & tp.w) | (M & tm.w), lt, eq);
+__device__ __forceinline__ uint4 mux4(uint32_t s, const uint4& x1, const uint4& x0) {
+    return make_uint4((s & x1.x) | (~s & x0.x), (s & x1.y) | (~s & x0.y), (s & x1.z) | (~s & x0.z),
+                      (s & x1.w) | (~s & x0.w));
+}
+
+// The four threshold planes of one Philox call of a hidden node with endpoints
+// e1, e2: e1 picks m = 2 or m = -2 (tb points at the call's first plane of the
+// m = -2 row, m = 2 row 64 words further).  Chains with m = 0 (e1 != e2) take no notice of them:
+// their threshold 2^31 is the top plane of the uniform alone (hidden_first).
+__device__ __forceinline__ uint4 hidden_planes(const uint32_t* tb, uint32_t e1) {
+    return mux4(e1, planes4(tb + 64), planes4(tb));
+}
+// Calls 0 and 1 of a hidden node (Z: the chains with m = 0): lt the chains
+// below their threshold, eq the chains still open.
+__device__ __forceinline__ void hidden_first(const U4& q0, const U4& q1, const uint32_t* tb, uint32_t e1, uint32_t Z,
+                                             uint32_t& lt, uint32_t& eq) {
+    uint32_t l = 0u, ne = Z;
+    planes_step(q1, hidden_planes(tb + 4, e1), l, ne);
+    planes_step(q0, hidden_planes(tb, e1), l, ne);
+    lt = (Z & ~q0.x) | (~Z & l);
+    eq = ~ne;
 }
 
 // Count of set bits among h0..h3 per chain, c0 + 2 c1 + 4 c2, bit-sliced.
@@ -53,14 +78,10 @@ __device__ __forceinline__ Count4 count4(uint32_t h0, uint32_t h1, uint32_t h2, 
 // J' bit, n the count of the J incidences.  A mux tree per plane: the J' bit,
 // then count bits 0, 1, 2 (a count of 4 has bits 0 and 1 clear).
 __device__ __forceinline__ uint4 visible_planes(const uint32_t* tb, uint32_t hp, const Count4& n) {
-    auto mux = [](uint32_t s, const uint4& x1, const uint4& x0) {
-        return make_uint4((s & x1.x) | (~s & x0.x), (s & x1.y) | (~s & x0.y), (s & x1.z) | (~s & x0.z),
-                          (s & x1.w) | (~s & x0.w));
-    };
-    auto sel = [&](int c) { return mux(hp, planes4(tb + (2 * c + 1) * 32), planes4(tb + 2 * c * 32)); };
-    const uint4 m01 = mux(n.c0, sel(1), sel(0));
-    const uint4 m23 = mux(n.c0, sel(3), sel(2));
-    return mux(n.c2, sel(4), mux(n.c1, m23, m01));
+    auto sel = [&](int c) { return mux4(hp, planes4(tb + (2 * c + 1) * 32), planes4(tb + 2 * c * 32)); };
+    const uint4 m01 = mux4(n.c0, sel(1), sel(0));
+    const uint4 m23 = mux4(n.c0, sel(3), sel(2));
+    return mux4(n.c2, sel(4), mux4(n.c1, m23, m01));
 }
 
 // Appends the lanes whose comparison is still open (open != 0: its

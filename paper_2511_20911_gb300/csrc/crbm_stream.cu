@@ -357,10 +357,10 @@ __global__ void __launch_bounds__(kStreamThreads) k_stream_bp_hidden(const Sweep
     const uint64_t pw = static_cast<uint64_t>(kPhiloxM1) * static_cast<uint32_t>(w);
     const uint32_t Yw = static_cast<uint32_t>(pw);
     const Round1Sweep rs = round1_sweep(static_cast<uint32_t>(pw >> 32) ^ a.rk[0] ^ t, a.rk);
-    // node nd of the tile: its threshold planes (P: m = 2, M: m = -2, Z: m = 0), Philox cell words
-    // and the index of its hidden word in s_h
+    // node nd of the tile: its first endpoint, the chains with m = 0, the threshold planes, Philox
+    // cell words and the index of its hidden word in s_h
     struct Hid {
-        uint32_t P, M, Z, c2;
+        uint32_t e1, Z, c2;
         const uint32_t* tp;
         Round2Cell r2;
         int out;
@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(kStreamThreads) k_stream_bp_hidden(const Sweep
         const uint32_t e2 = v[s_off[1][k]] ^ (cls ? fl1 : fl0);
         const uint32_t cell = static_cast<uint32_t>((i0 + li) * Wc + j0 + lj);
         const uint64_t pc = static_cast<uint64_t>(kPhiloxM0) * cell;
-        return Hid{e1 & e2, ~(e1 | e2), e1 ^ e2,
+        return Hid{e1, e1 ^ e2,
                    static_cast<uint32_t>(pc >> 32) ^ a.rk[1] ^ (kTagBitplane + 8u * static_cast<uint32_t>(k)),
                    s_tab + kBpHidPlanes + cls * 96u, round2_cell(rs.hik ^ static_cast<uint32_t>(pc)),
                    (li * kTJ + lj) * 10 + k};
@@ -383,20 +383,18 @@ __global__ void __launch_bounds__(kStreamThreads) k_stream_bp_hidden(const Sweep
         const int node = base + lane;
         const bool valid = node < nn;
         const Hid hn = hidden_node(valid ? node : 0);
-        uint32_t lt = 0u, eq = valid ? 0xffffffffu : 0u;
-        auto planes = [&](const U4& q, uint32_t j) {
-            bp::hidden_planes(q, hn.tp + 4u * j, hn.P, hn.M, j == 0u ? hn.Z : 0u, lt, eq);
-        };
+        uint32_t lt, eq;
         // calls 0 and 1 together, then the open nodes to the straggler list
         const U4 q0 = philox_from_round2(Yw, rs, hn.r2, hn.c2, a.rk);
         const U4 q1 = philox_from_round2(Yw, rs, hn.r2, hn.c2 ^ 1u, a.rk);
-        planes(q0, 0u);
-        planes(q1, 1u);
+        bp::hidden_first(q0, q1, hn.tp, hn.e1, hn.Z, lt, eq);
+        eq = valid ? eq : 0u;
         if (bp::push_straggler(static_cast<uint32_t>(node), eq, &s_nst, s_list, kCap, lane)) eq = 0u;
 #pragma unroll 1
         for (uint32_t j = 2; j < 8u; ++j) {  // only where the list was full
             if (!__any_sync(0xffffffffu, eq != 0u)) break;
-            planes(philox_from_round2(Yw, rs, hn.r2, hn.c2 ^ j, a.rk), j);
+            bp::planes_below(philox_from_round2(Yw, rs, hn.r2, hn.c2 ^ j, a.rk), bp::hidden_planes(hn.tp + 4u * j, hn.e1),
+                             lt, eq);
         }
         if (valid) s_h[hn.out] = lt;  // final, or the decided part of a straggler
     }
@@ -410,8 +408,8 @@ __global__ void __launch_bounds__(kStreamThreads) k_stream_bp_hidden(const Sweep
 #pragma unroll 1
         for (uint32_t j = 2; j < 8u; ++j) {
             if (!__any_sync(0xffffffffu, eq != 0u)) break;
-            bp::hidden_planes(philox_from_round2(Yw, rs, hn.r2, hn.c2 ^ j, a.rk), hn.tp + 4u * j, hn.P, hn.M, 0u, lt,
-                              eq);
+            bp::planes_below(philox_from_round2(Yw, rs, hn.r2, hn.c2 ^ j, a.rk), bp::hidden_planes(hn.tp + 4u * j, hn.e1),
+                             lt, eq);
         }
         if (valid) s_h[hn.out] = lt;
     }
@@ -509,27 +507,27 @@ __global__ void __launch_bounds__(kStreamVisThreads, kStreamMinBlocks) k_stream_
                    static_cast<uint32_t>(pc >> 32) ^ a.rk[1] ^ (kTagBitplane + 8u * (10u + static_cast<uint32_t>(x))),
                    bp::count4(h0, h1, h2, h3), round2_cell(rs.hik ^ static_cast<uint32_t>(pc)), R * VO + C};
     };
-    auto planes = [&](const Vis& vn, const U4& q, uint32_t j, uint32_t& lt, uint32_t& eq) {
-        const uint4 T = bp::visible_planes(tv + 4u * j, vn.hp, vn.n4);
-        bp::plane_step(q.x, T.x, lt, eq);
-        bp::plane_step(q.y, T.y, lt, eq);
-        bp::plane_step(q.z, T.z, lt, eq);
-        bp::plane_step(q.w, T.w, lt, eq);
+    auto below = [&](const Vis& vn, uint32_t j, uint32_t& lt, uint32_t& eq) {
+        bp::planes_below(philox_from_round2(Yw, rs, vn.r2, vn.c2 ^ j, a.rk),
+                         bp::visible_planes(tv + 4u * j, vn.hp, vn.n4), lt, eq);
     };
     for (int base = warp * 32; base < nn; base += nwarp * 32) {
         const int sx = base + lane;
         const bool valid = sx < nn;
         const Vis vn = visible_node(valid ? sx : 0);
-        uint32_t lt = 0u, eq = valid ? 0xffffffffu : 0u;
-        // calls 0 and 1 (a loop, so that the threshold planes are not held in registers across
+        uint32_t lt = 0u, ne = 0u;
+        // calls 1 and 0 (a loop, so that the threshold planes are not held in registers across
         // tiles), then the open spins to the straggler list
 #pragma unroll 1
-        for (uint32_t j = 0; j < 2u; ++j) planes(vn, philox_from_round2(Yw, rs, vn.r2, vn.c2 ^ j, a.rk), j, lt, eq);
+        for (int j = 1; j >= 0; --j)
+            bp::planes_step(philox_from_round2(Yw, rs, vn.r2, vn.c2 ^ static_cast<uint32_t>(j), a.rk),
+                            bp::visible_planes(tv + 4 * j, vn.hp, vn.n4), lt, ne);
+        uint32_t eq = valid ? ~ne : 0u;
         if (bp::push_straggler(static_cast<uint32_t>(sx), eq, &s_nst, s_list, kCap, lane)) eq = 0u;
 #pragma unroll 1
         for (uint32_t j = 2; j < 8u; ++j) {  // only where the list was full
             if (!__any_sync(0xffffffffu, eq != 0u)) break;
-            planes(vn, philox_from_round2(Yw, rs, vn.r2, vn.c2 ^ j, a.rk), j, lt, eq);
+            below(vn, j, lt, eq);
         }
         if (valid) s_o[vn.out] = lt;  // final, or the decided part of a straggler
     }
@@ -543,7 +541,7 @@ __global__ void __launch_bounds__(kStreamVisThreads, kStreamMinBlocks) k_stream_
 #pragma unroll 1
         for (uint32_t j = 2; j < 8u; ++j) {
             if (!__any_sync(0xffffffffu, eq != 0u)) break;
-            planes(vn, philox_from_round2(Yw, rs, vn.r2, vn.c2 ^ j, a.rk), j, lt, eq);
+            below(vn, j, lt, eq);
         }
         if (valid) s_o[vn.out] = lt;
     }
