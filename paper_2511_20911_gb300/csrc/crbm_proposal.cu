@@ -596,8 +596,8 @@ __device__ __forceinline__ float bf16r(float x) { return __bfloat162float(__floa
 // share the weights; a slot takes examples in turn, one at a time, its
 // activations and deltas in shared memory and its gradient sums in registers
 // over all its examples (added up per CTA at the end, then one atomic per
-// parameter and CTA).  grad and loss accumulate (the loss in 64 bits: 1216 slots
-// add to it).
+// parameter and CTA).  grad and loss accumulate in 64 bits: 152 CTAs add to a
+// parameter and 1216 slots to the loss.
 // What bounds it: 0.37 M multiply-adds per example on the FP32 pipe (38 us for
 // 4096 examples at its peak).  With a thread per output or per parameter every
 // multiply-add took two shared-memory loads (773 us); here a thread holds a tile
@@ -624,7 +624,7 @@ static_assert(tSlot % 4 == 0 && kSlotFloats % 4 == 0 && uA1 % 4 == 0 && uD1 % 4 
 __device__ __forceinline__ void slot_sync(int slot) { asm volatile("bar.sync %0, 64;" ::"r"(1 + slot) : "memory"); }
 
 __global__ void __launch_bounds__(kTrainThreads, 1) k_prop_train(const float* __restrict__ w, const Example* ex, int n,
-                                                                 float* grad, double* loss) {
+                                                                 double* grad, double* loss) {
     extern __shared__ __align__(16) float sm[];
     const int slot = threadIdx.x >> 6, tid = threadIdx.x & 63, wid = tid >> 5, lane = tid & 31;
     float* S = sm + tSlot + slot * kSlotFloats;
@@ -951,16 +951,16 @@ __global__ void __launch_bounds__(kTrainThreads, 1) k_prop_train(const float* __
         if (tid == 0 && lsum != 0.f) atomicAdd(loss, static_cast<double>(lsum) / (static_cast<double>(n) * kK * kK));
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < kNP; i += kTrainThreads) atomicAdd(&grad[i], G[i]);
+    for (int i = threadIdx.x; i < kNP; i += kTrainThreads) atomicAdd(&grad[i], static_cast<double>(G[i]));
 }
 
 // Adam (Kingma & Ba) on the fp32 master weights; also refreshes the
 // bf16-rounded copy the kernels read.
-__global__ void k_prop_adam(float* w, float* wb, float* m, float* v2, const float* grad, int n, float lr,
+__global__ void k_prop_adam(float* w, float* wb, float* m, float* v2, const double* grad, int n, float lr,
                             float b1, float b2, float eps, float c1, float c2) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const float g = grad[i];
+    const float g = static_cast<float>(grad[i]);
     m[i] = b1 * m[i] + (1.f - b1) * g;
     v2[i] = b2 * v2[i] + (1.f - b2) * g * g;
     w[i] -= lr * (m[i] / c1) / (sqrtf(v2[i] / c2) + eps);
@@ -1048,7 +1048,7 @@ struct crbm_proposal {
     float* wb = nullptr;     // bf16-rounded copy
     float* m = nullptr;      // Adam moments
     float* v2 = nullptr;
-    float* grad = nullptr;
+    double* grad = nullptr;
     double* loss = nullptr;  // [kLossCap], a training step each
     uint16_t* bmat = nullptr;  // tensor-core B operands (bf16)
     float* bias = nullptr;     // b2, b3
@@ -1247,9 +1247,10 @@ int crbm_proposal_create(crbm_proposal** out, int32_t block, uint64_t seed) {
     p->seed = seed;
     cudaGetDevice(&p->device);
     cudaError_t e = cudaSuccess;
-    float** bufs[] = {&p->w, &p->wb, &p->m, &p->v2, &p->grad};
+    float** bufs[] = {&p->w, &p->wb, &p->m, &p->v2};
     for (float** b : bufs)
         if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(b), kNP * sizeof(float));
+    if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&p->grad), kNP * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&p->loss), kLossCap * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&p->bmat), crbm::kBElems * sizeof(uint16_t));
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&p->bias), 33 * sizeof(float));
@@ -1319,17 +1320,21 @@ int crbm_proposal_loss_grad(crbm_proposal* p, const int8_t* spins, int32_t L, co
     cudaError_t e = cudaMemcpy(p->raw, spins, b_spins, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(d_origins, origins, 8 * static_cast<size_t>(n), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(d_bh, beta_h, 8 * static_cast<size_t>(n), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemsetAsync(p->grad, 0, kNP * 4, nullptr);
+    if (e == cudaSuccess) e = cudaMemsetAsync(p->grad, 0, kNP * sizeof(double), nullptr);
     if (e == cudaSuccess) e = cudaMemsetAsync(p->loss, 0, sizeof(double), nullptr);
     if (e == cudaSuccess) {
         crbm::k_prop_gather<<<(n + 3) / 4, 128>>>(reinterpret_cast<const int8_t*>(p->raw), L, d_origins, d_bh, p->ex, n);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = launch_train(p, n, p->loss, nullptr);
-    if (e == cudaSuccess) e = cudaMemcpy(grad, p->grad, kNP * 4, cudaMemcpyDeviceToHost);
+    double g[kNP];
+    if (e == cudaSuccess) e = cudaMemcpy(g, p->grad, sizeof(g), cudaMemcpyDeviceToHost);
     double sum = 0.0;
     if (e == cudaSuccess) e = cudaMemcpy(&sum, p->loss, sizeof(sum), cudaMemcpyDeviceToHost);
-    if (e == cudaSuccess) *loss = static_cast<float>(sum);
+    if (e == cudaSuccess) {
+        *loss = static_cast<float>(sum);
+        for (int i = 0; i < kNP; ++i) grad[i] = static_cast<float>(g[i]);
+    }
     return e == cudaSuccess ? CRBM_OK : prop_fail(CRBM_ECUDA, cudaGetErrorString(e));
 }
 
@@ -1349,7 +1354,7 @@ int crbm_proposal_train(crbm_proposal* p, crbm_ctx* ctx, int32_t steps, int32_t 
             ctx->g, ctx->d.v, ctx->d.chain_bh, ctx->n_chains, p->ex, batch,
             static_cast<uint32_t>(p->adam_t), static_cast<uint32_t>(p->seed), static_cast<uint32_t>(p->seed >> 32));
         cudaError_t e = cudaGetLastError();
-        if (e == cudaSuccess) e = cudaMemsetAsync(p->grad, 0, kNP * 4, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(p->grad, 0, kNP * sizeof(double), st);
         if (e == cudaSuccess && s % kLossCap == 0) e = cudaMemsetAsync(p->loss, 0, kLossCap * sizeof(double), st);
         if (e == cudaSuccess) e = launch_train(p, batch, step_loss, st);
         ++p->adam_t;
