@@ -34,6 +34,15 @@ using namespace bp;
 
 constexpr int kBpMaxThreads = CRBM_SWEEP_MAX_THREADS;  // largest CTA the launch takes
 
+// What bounds it: the half-steps' barriers and the ALU pipe (L=18, 384 words:
+// ALU 47 %, with the wide multiplies' share 74 % of its slots; 5.7 of 13.6
+// stalled warps at barriers).
+// Default CTA (default_warps): with less than three words per SM one round of
+// node groups, up to 16 warps, finishes a word's half-step soonest; with more,
+// smaller CTAs, of which more are resident, fill each other's barriers.  us per
+// sweep, a warp per six cells always -> by this rule: L=6 3.2 -> 2.8 (152
+// words), L=12 3.4 -> 3.05 (8), 5.0 -> 4.7 (384), 8.3 -> 7.5 (800), L=18 10.1 ->
+// 9.2 (530), 16.2 -> 12.9 (800), L=24 22.9 -> 19.9 (800).
 // Persistent grid over (word, chunk of sweeps) items (claim_word): the node
 // records are staged once per CTA, then each claimed chunk runs the body.
 // At most 56 registers a thread, so that three CTAs of 12 warps (the shape

@@ -251,11 +251,19 @@ int default_warps(const Geometry& g, int n_words) {
         const int w = std::atoi(env);
         if (w >= 1 && w <= kMaxSweepWarps) return w;
     }
-    if (g.bitplane) return std::max(1, std::min(std::min(16, kMaxSweepWarps), (g.n_cells + 5) / 6));
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
         sms = 152;
+    if (g.bitplane) {  // see launch_sweep_bitplane
+        const int groups = (g.n_cells * 10 + 31) / 32;
+        const int round = (groups + 3) & ~3;  // one round of hidden groups
+        const int w = n_words >= 5 * sms   ? (groups <= 12 ? 4 : 8)
+                      : n_words >= 3 * sms ? (groups <= 12 ? std::min(8, round) : 12)
+                      : groups <= 16       ? std::min(12, round)
+                                           : (g.n_cells + 5) / 6;
+        return std::max(1, std::min(std::min(16, kMaxSweepWarps), w));
+    }
     if (!g.canonical)
         return std::max(1, std::min(std::min(n_words <= sms ? 16 : n_words < 3 * sms || g.n_cells >= 64 ? 8 : 4, kMaxSweepWarps),
                                     g.n_cells));
