@@ -48,14 +48,14 @@ CALLS_PER_CELL_PAPER_STREAM = 3  # streamed paper precision: the visible half-st
 # launch of k_sweep_canon_persistent (2000 sweeps of the L=18 grid), and one
 # streamed sweep of the L=384 lattice (k_stream_hidden + k_stream_visible).
 MEASURED_TRAFFIC = {
-    "grid": (8.73e6 + 0.84e6, "per launch; profiles/launches_L18_grid.md"),
-    "grid_sq": (10.91e6 + 0.87e6, "per launch with S(q) every 100 sweeps; profiles/launches_L18_grid.md"),
-    "stream": (56.74e6 + 392.31e6 + 454.82e6 + 48.83e6, "per sweep (two launches); profiles/k_stream_L384.md"),
-    "grid_paper": (8.34e6 + 0.78e6, "per launch; profiles/k_sweep_canon_persistent_L18_grid_paper.md"),
-    "grid_paper_sq": (10.46e6 + 0.77e6,
+    "grid": (8.96e6 + 0.09e6, "per launch; profiles/launches_L18_grid.md"),
+    "grid_sq": (10.60e6 + 0.11e6, "per launch with S(q) every 100 sweeps; profiles/launches_L18_grid.md"),
+    "stream": (56.93e6 + 390.50e6 + 454.58e6 + 45.85e6, "per sweep (two launches); profiles/k_stream_L384.md"),
+    "grid_paper": (8.66e6 + 0.10e6, "per launch; profiles/k_sweep_canon_persistent_L18_grid_paper.md"),
+    "grid_paper_sq": (10.77e6 + 0.09e6,
                       "per launch with S(q) every 100 sweeps; profiles/k_sweep_canon_persistent_L18_grid_paper.md"),
-    "stream_paper": (56.76e6 + 390.29e6 + 454.76e6 + 45.71e6, "per sweep (two launches); profiles/k_stream_L384.md"),
-    "grid_bitplane": (2.48e6 + 0.78e6, "per launch; profiles/k_sweep_bitplane_L18_grid.md"),
+    "stream_paper": (56.75e6 + 390.68e6 + 454.88e6 + 45.83e6, "per sweep (two launches); profiles/k_stream_L384.md"),
+    "grid_bitplane": (2.46e6 + 0.78e6, "per launch; profiles/k_sweep_bitplane_L18_grid.md"),
     "stream_bitplane": (56.88e6 + 82.96e6 + 141.80e6 + 29.02e6, "per sweep (two launches); profiles/k_stream_bp_L384.md"),
 }
 
@@ -70,7 +70,9 @@ def bitplane_expected_calls(n_nodes):
     comparison with probability 1/2, so it is still open after 4 m planes with
     probability 2^-4m, independently; the number of stragglers is binomial.
     (A node past the list's capacity, a quarter of the half-step, finishes in
-    place; its probability is negligible and not modelled.)"""
+    place; its probability is negligible and not modelled.)  An upper bound
+    for hidden units: their chains with m = 0 (threshold 2^31) are decided by
+    the top plane and never open, which would need the spins to count."""
     def node_open(m):                         # any of the node's 32 chains open after m calls
         return -math.expm1(32.0 * math.log1p(-(2.0 ** (-4 * m))))
     p2 = node_open(2)
