@@ -112,13 +112,19 @@ struct CanonSmem {
     int segmask;  // [32]
     int seg;      // [33]; [33], [34]: the persistent scheduler's word and chunk
     int u;        // [32] uniforms of a swap round
-    int w;        // [n_cells][32] hidden words (kCanonPacked, exact precision: 16-bit)
+    int w;        // [n_cells][32] hidden words (kCanonPacked, exact precision: 16-bit); a correlation sample's scratch
     int pw;       // [n_cells][32] pairs (paper precision unless kCanonPacked): visible draws
     int rec;      // [n_cells][kCellRec * 4] (kCanonRec)
     int rows;     // [W][n_seg][32] spins of a row segment of cells
     int expand;   // [1024] 32-bit form of a 16-bit hidden word (kCanonPacked, exact precision)
     int total;
 };
+// Words of scratch that a correlation sample (square lattices) writes over the hidden
+// words, dead by then: a word per row and chain up to L = 32, else a word per site.
+// More than the 16-bit hidden words of L = 4 and 6, less than any other form's.
+__host__ __device__ inline int canon_corr_scratch(const Geometry& g) {
+    return g.L != g.Lc ? 0 : g.L <= 32 ? g.L * 32 : g.N;
+}
 __host__ __device__ inline CanonSmem canon_smem(const Geometry& g, int mode) {
     CanonSmem s;
     int low = 260, high = kCanonTabWord + kCanonTabBytes / 4;
@@ -134,7 +140,8 @@ __host__ __device__ inline CanonSmem canon_smem(const Geometry& g, int mode) {
     s.segmask = 160;
     s.seg = 192;
     s.u = 228;
-    s.w = place(g.n_cells * (mode == kCanonPacked && !g.paper ? 16 : 32));
+    const int w = g.n_cells * (mode == kCanonPacked && !g.paper ? 16 : 32);
+    s.w = place(w > canon_corr_scratch(g) ? w : canon_corr_scratch(g));
     s.pw = place(g.paper && mode != kCanonPacked ? g.n_cells * 64 : 0);
     s.rec = place(mode == kCanonRec ? g.n_cells * kCellRec * 4 : 0);
     s.rows = place(g.W * g.n_seg * 32);

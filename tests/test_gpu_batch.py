@@ -239,3 +239,24 @@ def test_batch_wide_ctas_match_individual_sweeps(monkeypatch):
     for a, b in zip(batched, twins):
         same(a, b)
     batch.close()
+
+
+@pytest.mark.parametrize("L", [4, 6, 8])
+def test_batch_correlations_beside_a_large_member(L):
+    """A member too large for its records in shared memory (L = 64) puts every canonical member in the form with
+    16-bit hidden words, which take less room than a small lattice's correlation samples."""
+    rng = np.random.default_rng(70 + L)
+    specs = [dict(L=L, params=workloads.random_params(rng, 3), n_chains=70, chain_param=rng.integers(0, 3, 70).astype(np.int32),
+                  seed=31, measure_every=2, sq_every=sq, series_len=8) for sq in (1, 3)]
+    specs.append(dict(L=64, params=workloads.random_params(rng, 2), n_chains=33,
+                      chain_param=rng.integers(0, 2, 33).astype(np.int32), seed=32, measure_every=2))
+    batched = [make(s) for s in specs]
+    twins = [make(s) for s in specs]
+    batch = crbm.Batch(batched)
+    for n in (1, 7, 8):
+        batch.sweep(n)
+        for t in twins:
+            t.sweep(n)
+        for a, b in zip(batched, twins):
+            same(a, b)
+    batch.close()
