@@ -24,7 +24,10 @@ namespace {
 
 // ----------------------------------------------------------------- cache
 // One line per tuned shape: "<key> <warps>"; the key names the GPU, the
-// lattice, the filter set and the number of packed words.
+// lattice, the filter set, the number of packed words, what else chooses the
+// kernel, and the revision of the kernels: shapes tuned for earlier ones are
+// not taken (raise it with any change that moves the best shape).
+constexpr int kShapeRevision = 2;
 std::mutex g_cache_mutex;
 
 std::string cache_path() {
@@ -39,7 +42,8 @@ std::string shape_key(const crbm_ctx* ctx) {
     std::ostringstream k;
     k << prop.name << "|sm" << prop.multiProcessorCount << "|L" << ctx->g.L << "|p" << ctx->g.periodic << "|c"
       << ctx->g.canonical << "|nb" << ctx->g.nb << "|w" << ctx->n_words << "|x" << (ctx->swap_every > 0)
-      << "|q" << ctx->g.paper << "|bp" << ctx->g.bitplane << "|Lc" << ctx->g.Lc << "|pc" << ctx->g.pc << "|v" << ctx->g.n_vis_tab;
+      << "|q" << ctx->g.paper << "|bp" << ctx->g.bitplane << "|Lc" << ctx->g.Lc << "|pc" << ctx->g.pc << "|v" << ctx->g.n_vis_tab
+      << "|s" << (ctx->sq_every > 0) << "|r" << kShapeRevision;
     std::string s = k.str();
     std::replace(s.begin(), s.end(), ' ', '_');
     return s;
@@ -57,11 +61,13 @@ size_t member_smem(const crbm_ctx* ctx, int warps, int canon_mode, int bands) {
     return sizeof(uint32_t) * static_cast<size_t>(canon_smem(g, canon_mode).total);
 }
 
-cudaError_t launch_one(const SweepArgs& a, const crbm_ctx* ctx, int warps) {
+// One launch as crbm_sweep makes it; plan: the canonical sweep's choices for
+// `warps`, made by the first launch with it (host queries that a timed launch
+// must not include).
+cudaError_t launch_one(const SweepArgs& a, const crbm_ctx* ctx, int warps, CanonLaunch& plan) {
     if (!ctx->g.canonical) return launch_sweep_generic(a, warps, ctx->stream);
     const int chunk = std::max(8, (a.n_sweeps + CRBM_CHUNKS_PER_WORD - 1) / CRBM_CHUNKS_PER_WORD);  // as crbm_sweep does
     if (ctx->g.bitplane) return launch_sweep_bitplane(a, warps, chunk, ctx->d.sched, ctx->stream);
-    CanonLaunch plan;
     return launch_sweep_canon_persistent(a, warps, ctx->d.sched, plan, ctx->stream);
 }
 
@@ -97,10 +103,13 @@ int crbm_autotune(crbm_ctx* ctx, int64_t probe_sweeps, int32_t* best_warps) {
     uint32_t* v2 = nullptr;
     int64_t* s2 = nullptr;
     int32_t* p2 = nullptr;
+    int64_t* c2 = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&v2), ctx->n_words * N * 4);
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&s2), npad * kNSum * 8);
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&p2), npad * 4);
+    if (e == cudaSuccess && ctx->sq_every > 0)
+        e = cudaMalloc(reinterpret_cast<void**>(&c2), static_cast<size_t>(ctx->n_params) * N * 8);
     if (e == cudaSuccess) e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
     int best = ctx->warps;
@@ -123,14 +132,15 @@ int crbm_autotune(crbm_ctx* ctx, int64_t probe_sweeps, int32_t* best_warps) {
         a.sums = s2;
         a.sob = p2;
         a.series_len = 0;
-        a.sq_every = 0;
+        a.corr = c2;  // (correlations stay on: a context that takes them never splits its words)
         a.clock = nullptr;
         a.hit = nullptr;  // the probes record no time to solution
         a.n_sweeps = static_cast<int>(std::max<int64_t>(1, probe_sweeps / 4));
-        e = launch_one(a, ctx, w);  // warm-up
+        CanonLaunch plan;
+        e = launch_one(a, ctx, w, plan);  // warm-up
         a.n_sweeps = static_cast<int>(probe_sweeps);
         if (e == cudaSuccess) e = cudaEventRecord(e0, ctx->stream);
-        if (e == cudaSuccess) e = launch_one(a, ctx, w);
+        if (e == cudaSuccess) e = launch_one(a, ctx, w, plan);
         if (e == cudaSuccess) e = cudaEventRecord(e1, ctx->stream);
         if (e == cudaSuccess) e = cudaEventSynchronize(e1);
         float ms = 0.f;
@@ -145,6 +155,7 @@ int crbm_autotune(crbm_ctx* ctx, int64_t probe_sweeps, int32_t* best_warps) {
     cudaFree(v2);
     cudaFree(s2);
     cudaFree(p2);
+    cudaFree(c2);
     if (e != cudaSuccess) {
         ctx->err = std::string("crbm_autotune: ") + cudaGetErrorString(e);
         return CRBM_ECUDA;

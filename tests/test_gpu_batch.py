@@ -1,6 +1,8 @@
 """Batched launches and the autotuner.  A batch advances every member by one
 kernel launch (graph-captured); each member must stay bit-identical to a twin
 context advanced on its own.  Autotuning must not touch the chains."""
+import time
+
 import numpy as np
 import pytest
 
@@ -260,3 +262,44 @@ def test_batch_correlations_beside_a_large_member(L):
         for a, b in zip(batched, twins):
             same(a, b)
     batch.close()
+
+
+def test_tuned_shapes_are_taken_only_for_the_kernel_they_were_timed_on(tmp_path, monkeypatch):
+    """A context with correlations (which never splits its words over a cluster) does not take the shape of one
+    without, nor does any context take a shape cached under the key of earlier kernels."""
+    torch = pytest.importorskip("torch")
+    cache = tmp_path / "tune.txt"
+    monkeypatch.setenv("CRBM_AUTOTUNE_CACHE", str(cache))
+    spec = dict(L=18, params=workloads.random_params(np.random.default_rng(9), 2), n_chains=64, seed=3)
+    default = make(dict(spec, sq_every=5)).warps
+    make(spec).autotune(4)
+    key = cache.read_text().split()[0]
+    cache.write_text(f"{key} 3\n")
+    assert make(spec).warps == 3
+    assert make(dict(spec, sq_every=5)).warps == default
+    p = torch.cuda.get_device_properties(0)
+    name = p.name.replace(" ", "_")
+    cache.write_text(f"{name}|sm{p.multi_processor_count}|L18|p1|c1|nb10|w2|x0|q0|bp0|Lc18|pc1|v1 3\n")
+    assert make(spec).warps == make(dict(spec, seed=4)).warps != 3
+
+
+def test_autotune_probes_do_the_work_of_the_context(tmp_path, monkeypatch):
+    """Probes of a context with correlations take them too (into scratch), so that they time the kernel that runs.
+    At L = 48 a correlation sample takes twenty times a sweep: a dozen shapes probed without would take less time
+    than three of them with."""
+    torch = pytest.importorskip("torch")
+    monkeypatch.setenv("CRBM_AUTOTUNE_CACHE", str(tmp_path / "tune.txt"))
+    s = make(dict(L=48, params=workloads.random_params(np.random.default_rng(9), 2), n_chains=64, seed=3, sq_every=1))
+
+    def seconds(f):
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        f()
+        torch.cuda.synchronize()
+        return time.perf_counter() - t
+
+    s.sweep(20)
+    sweeps = min(seconds(lambda: s.sweep(20)) for _ in range(3))
+    before = s.correlations()[0]
+    assert seconds(lambda: s.autotune(20)) > 3 * sweeps
+    assert np.array_equal(s.correlations()[0], before)
