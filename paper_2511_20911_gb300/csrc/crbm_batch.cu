@@ -37,11 +37,14 @@ __global__ void k_batch_advance(int64_t* clocks, const int* every, int n_ctx, in
 cudaError_t launch_sweep_batch(const BatchArgs& b, int n_tasks, int cluster, int threads, size_t smem, int modes,
                                cudaStream_t st) {
     const BatchKernel kernel = batch_kernel(cluster > 1, modes, threads);
-    int dev = 0, reserved = 0;  // (the canonical members' table addresses: see kReservedSmem)
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess ||
-        reserved != kReservedSmem)
-        return cudaErrorInvalidConfiguration;
+    bool rows = false;  // members in row form, which find their tables by address
+    for (int c = 0; c < b.n_desc; ++c) rows = rows || (b.d[c].g.canonical && !b.d[c].g.bitplane);
+    if (rows) {
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = check_dynamic_smem_base(reinterpret_cast<const void*>(kernel), dev);
+        if (e != cudaSuccess) return e;
+    }
     if (smem > 48 * 1024) {
         const cudaError_t e =
             cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));

@@ -125,6 +125,15 @@ __global__ void __launch_bounds__(kCtaWide, 1) k_sweep_canon_split(const SweepAr
 
 }  // namespace
 
+cudaError_t check_dynamic_smem_base(const void* kernel, int dev) {
+    int reserved = 0;
+    cudaFuncAttributes at{};
+    cudaError_t e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, kernel);
+    if (e == cudaSuccess && !dynamic_smem_at_base(reserved, at.sharedSizeBytes)) e = cudaErrorInvalidConfiguration;
+    return e;
+}
+
 size_t smem_bytes_canon(const Geometry& g) {
     const size_t words = static_cast<size_t>(kAccWords) + kCanonTab + g.N + static_cast<size_t>(g.n_cells) * 32 + 96 + 33 +
                          32 + 64 + 3;
@@ -262,13 +271,13 @@ cudaError_t make_plan(const Geometry& g0, int n_words, int warps, int dev, bool 
     p.smem = canon_plan(g, warps, &p.mode);
     p.seg_cells = g.seg_cells;
     p.n_seg = g.n_seg;
-    int reserved = 0;
-    cudaError_t e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&p.sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaError_t e = cudaDeviceGetAttribute(&p.sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     p.bands = pick_bands(g, n_words, warps, p.sms, correlations);
-    if (p.bands > 1 && reserved == kReservedSmem) {
+    if (p.bands > 1) {
         p.smem = canon_plan(g, warps, &p.mode, p.bands);
+        if ((e = check_dynamic_smem_base(reinterpret_cast<const void*>(split_kernel(p.mode, g.paper)), dev)) != cudaSuccess)
+            return e;
         p.seg_cells = g.seg_cells;
         p.n_seg = g.n_seg;
         p.warps = warps;
@@ -297,7 +306,9 @@ cudaError_t make_plan(const Geometry& g0, int n_words, int warps, int dev, bool 
         p.cta = kCtaAny;
         p.per_sm = per_sm[0];
     }
-    if (p.per_sm < 1 || reserved != kReservedSmem) return cudaErrorInvalidConfiguration;
+    if (p.per_sm < 1) return cudaErrorInvalidConfiguration;
+    if ((e = check_dynamic_smem_base(reinterpret_cast<const void*>(persistent_kernel(p.mode, g.paper, p.cta)), dev)) != cudaSuccess)
+        return e;
     p.warps = warps;
     p.device = dev;
     return cudaSuccess;

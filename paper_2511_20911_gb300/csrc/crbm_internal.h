@@ -102,6 +102,9 @@ constexpr int kMaxSegCells = 3;  // cells of a row segment, the unit of work of 
 // static shared memory (checked by the launchers); the space below the tables
 // takes what fits of the other arrays, the rest follows the tables.
 constexpr int kReservedSmem = 1024;
+// Whether a kernel's dynamic shared memory starts there: the bytes the driver
+// reserves per CTA, and the kernel's own static shared memory.
+inline bool dynamic_smem_at_base(int reserved, size_t static_bytes) { return reserved == kReservedSmem && static_bytes == 0; }
 constexpr int kCanonTabWord = (16384 - kReservedSmem) / 4;
 constexpr int kCanonTabBytes = 40960;   // a word's tables (crbm_row_core.cuh) ...
 constexpr int kCanonAccByte = 21760;    // ... with room for the running sums inside
@@ -301,6 +304,9 @@ struct CanonLaunch {
     int mode = 0, seg_cells = 0, n_seg = 0, cta = 0, per_sm = 0, sms = 0, bands = 1;
     size_t smem = 0;
 };
+// cudaErrorInvalidConfiguration unless dynamic_smem_at_base holds for `kernel` on device `dev` (a row-form
+// kernel whose tables lie elsewhere returns without work: every launcher asks before its first launch).
+cudaError_t check_dynamic_smem_base(const void* kernel, int dev);
 cudaError_t launch_init(const Geometry& g, uint32_t* v, int n_words, uint32_t key0,
                         uint32_t key1, cudaStream_t st);
 cudaError_t launch_sweep_generic(const SweepArgs& a, int warps_per_cta, cudaStream_t st);

@@ -669,9 +669,8 @@ cudaError_t launch_sweep_stream(const SweepArgs& a, cudaStream_t st, int64_t* la
     const auto hidden = a.g.paper ? k_stream_hidden<true> : k_stream_hidden<false>;
     const auto visible = a.g.paper ? k_stream_visible<true> : k_stream_visible<false>;
     if (!a.g.bitplane && a.n_sweeps > 0) {
-        int reserved = 0;
-        e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
-        if (e == cudaSuccess && reserved != kReservedSmem) e = cudaErrorInvalidConfiguration;
+        e = check_dynamic_smem_base(reinterpret_cast<const void*>(hidden), dev);
+        if (e == cudaSuccess) e = check_dynamic_smem_base(reinterpret_cast<const void*>(visible), dev);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(hidden, cudaFuncAttributeMaxDynamicSharedMemorySize, kHidSmem);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(visible, cudaFuncAttributeMaxDynamicSharedMemorySize, vis_smem(kMaxTileSeg));
         if (e != cudaSuccess) return e;

@@ -1,11 +1,16 @@
 // Prints the canonical SMEM sweep's shared-memory layout (crbm_internal.h), used only by tests.  Reads
 // "L Lc paper n_seg mode" lines on stdin; prints "name first end" triples of the arrays in words, one line
-// per layout.
+// per layout.  With arguments (reserved bytes, static bytes): whether the tables are where the kernels look.
 #include <cstdio>
+#include <cstdlib>
 
 #include "crbm_internal.h"
 
-int main() {
+int main(int argc, char** argv) {
+    if (argc == 3) {
+        std::printf("%d\n", crbm::dynamic_smem_at_base(std::atoi(argv[1]), std::strtoul(argv[2], nullptr, 10)) ? 1 : 0);
+        return 0;
+    }
     crbm::Geometry g{};
     int mode;
     while (std::scanf("%d %d %d %d %d", &g.L, &g.Lc, &g.paper, &g.n_seg, &mode) == 5) {
