@@ -1,0 +1,55 @@
+// Launch shapes by sizes: what the launchers and the context take before a
+// call chooses otherwise.  Host code without CUDA calls.
+#pragma once
+
+#include <algorithm>
+#include <cmath>
+
+#include "crbm_internal.h"
+
+namespace crbm {
+
+// ---- streamed lane-uniform sweep: tiles of `rows` rows of cells by `seg`
+// segments of three, rows in {4, 8, 16}, seg in {4, 5, 6}
+constexpr int kTileRows = 16, kMaxTileSeg = 6;
+struct RowCut {
+    int seg, rows;
+    int64_t tiles(const Geometry& g, int n_words) const {
+        return static_cast<int64_t>((g.W + rows - 1) / rows) * ((g.Wc + 3 * seg - 1) / (3 * seg)) * n_words;
+    }
+};
+// The half-steps' cut: the width that pads the lattice least, then the rows
+// with the least time of the fullest SM: the staging and cells of its k CTAs, and
+// the latency of one CTA, which grows less than its cells.  The constants (us)
+// are fits to both half-steps timed with every cut, 64 x 64 .. 512 x 512 and
+// 34 x 2048 spins in 2 .. 64 words; of the rows their choice is within 1.2 % of
+// the one of fewest CTAs from four per SM up, and up to 20 % faster.  us per
+// sweep with 16, 8 and 4 rows: 384 x 384, 2 words: 39 43 45; 96 x 96, 24 words:
+// 31 31 37; 100 x 100, 16 words: 41 33 29.
+inline RowCut row_cut(const Geometry& g, int n_words, int sms) {
+    RowCut c{5, kTileRows};
+    int waste = 1 << 30;
+    for (int s = 4; s <= kMaxTileSeg; ++s) {
+        const int pad = (g.Wc + 3 * s - 1) / (3 * s) * (3 * s) - g.Wc;
+        if (pad < waste || (pad == waste && s == 5)) {
+            c.seg = s;
+            waste = pad;
+        }
+    }
+    double best = 0.0;
+    int rows = kTileRows;
+    for (c.rows = kTileRows; c.rows >= 4; c.rows /= 2) {
+        const int64_t n = c.tiles(g, n_words), k = (n + sms - 1) / sms;
+        const double mean = static_cast<double>(g.n_cells) * n_words / static_cast<double>(n);
+        const double most = static_cast<double>(std::min(c.rows, g.W)) * std::min(3 * c.seg, g.Wc);
+        const double cost = static_cast<double>(k) * (1.1 + 0.023 * mean + 0.016 * most) + 0.6 * std::sqrt(most);
+        if (c.rows == kTileRows || cost <= best) {
+            best = cost;
+            rows = c.rows;
+        }
+    }
+    c.rows = rows;
+    return c;
+}
+
+}  // namespace crbm

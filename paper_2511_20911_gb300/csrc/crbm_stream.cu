@@ -10,6 +10,7 @@
 // the tag-0 and tag-1 calls and the visible half-step draws the tag-1 call again
 // for its four 16-bit uniforms: three calls per cell instead of four.
 #include "crbm_bitplane_core.cuh"
+#include "crbm_launch.h"
 #include "crbm_row_core.cuh"
 
 namespace crbm {
@@ -18,35 +19,13 @@ namespace {
 using namespace dev;
 using namespace canon;
 
-// Tiles of the lane-uniform sweep and of the count: 4, 8 or 16 rows of cells by 4,
-// 5 or 6 segments of three (RowCut).
-constexpr int kTI = 16;  // tile rows of cells (at most)
-constexpr int kMaxTileSeg = 6, kMaxTileCols = 3 * kMaxTileSeg;
+// Tiles of the lane-uniform sweep and of the count: RowCut (crbm_launch.h).
+constexpr int kTI = kTileRows;  // tile rows of cells (at most)
+constexpr int kMaxTileCols = 3 * kMaxTileSeg;
 // Tiles of the bit-plane sweep.
 constexpr int kTJ = 16;  // tile columns of cells
 constexpr int kStreamThreads = 256;  // every kernel
 constexpr int kStreamVisThreads = kStreamThreads;
-
-// Cut of the lattice into row tiles: the width that pads it least, 16 rows where
-// these make four CTAs per SM and else fewer, down to 4 (100 x 100 spins, 64
-// chains: 27 us per sweep in tiles of 16 rows, 16 in tiles of 4).
-struct RowCut {
-    int seg, rows;
-};
-inline RowCut row_cut(const Geometry& g, int n_words, int sms) {
-    RowCut c{5, kTI};
-    int waste = 1 << 30;
-    for (int s = 4; s <= kMaxTileSeg; ++s) {
-        const int pad = (g.Wc + 3 * s - 1) / (3 * s) * (3 * s) - g.Wc;
-        if (pad < waste || (pad == waste && s == 5)) {
-            c.seg = s;
-            waste = pad;
-        }
-    }
-    const int64_t columns = static_cast<int64_t>((g.Wc + 3 * c.seg - 1) / (3 * c.seg)) * n_words;
-    while (c.rows > 4 && columns * ((g.W + c.rows - 1) / c.rows) < 4 * sms) c.rows /= 2;
-    return c;
-}
 
 __device__ __forceinline__ size_t vidx(int w, int N, int s) {
     return (static_cast<size_t>(w >> 1) * N + s) * 2 + (w & 1);
@@ -665,7 +644,7 @@ cudaError_t launch_sweep_stream(const SweepArgs& a, cudaStream_t st, int64_t* la
     if (e != cudaSuccess) return e;
     const RowCut cut = row_cut(a.g, a.n_words, sms);
     const dim3 grid(((a.g.W + kTI - 1) / kTI) * ((a.g.Wc + kTJ - 1) / kTJ), a.n_words);  // bit-plane tiles
-    const dim3 row_grid(((a.g.W + cut.rows - 1) / cut.rows) * ((a.g.Wc + 3 * cut.seg - 1) / (3 * cut.seg)), a.n_words);
+    const dim3 row_grid(static_cast<unsigned int>(cut.tiles(a.g, 1)), a.n_words);
     const auto hidden = a.g.paper ? k_stream_hidden<true> : k_stream_hidden<false>;
     const auto visible = a.g.paper ? k_stream_visible<true> : k_stream_visible<false>;
     if (!a.g.bitplane && a.n_sweeps > 0) {

@@ -1,0 +1,32 @@
+// Evaluates the launch rules of crbm_launch.h on the host, used only by tests.  Reads "rule arguments" lines on
+// stdin and prints each rule's choice.
+#include <cstdio>
+#include <cstring>
+
+#include "crbm_launch.h"
+
+static crbm::Geometry lattice(int L, int Lc) {
+    crbm::Geometry g{};
+    g.L = L;
+    g.Lc = Lc;
+    g.W = (L + 1) / 2;
+    g.Wc = (Lc + 1) / 2;
+    g.N = L * Lc;
+    g.n_cells = g.W * g.Wc;
+    g.canonical = 1;
+    return g;
+}
+
+int main() {
+    char rule[32];
+    while (std::scanf("%31s", rule) == 1) {
+        int L, Lc, words;
+        if (!std::strcmp(rule, "rows") && std::scanf("%d %d %d", &L, &Lc, &words) == 3) {
+            const crbm::RowCut c = crbm::row_cut(lattice(L, Lc), words, 152);
+            std::printf("%d %d\n", c.seg, c.rows);
+        } else {
+            return 1;
+        }
+    }
+    return 0;
+}

@@ -1,0 +1,41 @@
+"""Launch rules by sizes (crbm_launch.h), evaluated on the host for a GPU of 152 SMs: what they choose at sizes where
+the variants were timed and another choice was found slower."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(os.path.dirname(HERE), "paper_2511_20911_gb300", "csrc")
+
+
+@pytest.fixture(scope="module")
+def rule(tmp_path_factory):
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("nvcc not available")
+    exe = str(tmp_path_factory.mktemp("rules") / "launch_rules_host")
+    subprocess.check_call([nvcc, "-O1", "-std=c++17", "-I", CSRC, "-o", exe, os.path.join(HERE, "launch_rules_host.cu")])
+
+    def ask(*args):
+        out = subprocess.run([exe], input=" ".join(str(a) for a in args) + "\n", capture_output=True, text=True, check=True)
+        return tuple(int(x) for x in out.stdout.split())
+
+    return ask
+
+
+# (two words of 384 x 384 took 43 us a sweep in 768 tiles of 8 rows, 39 in 384 of 16; 100 x 100 is the other way round)
+@pytest.mark.parametrize("L,Lc,words,rows", [(384, 384, 2, 16), (192, 192, 8, 16), (96, 96, 32, 16), (96, 96, 24, 8),
+                                             (250, 198, 4, 8), (64, 64, 2, 4), (100, 100, 16, 4), (96, 96, 2, 4),
+                                             (384, 384, 24, 16), (4, 4, 2, 4)])
+def test_streamed_tile_rows(rule, L, Lc, words, rows):
+    seg, r = rule("rows", L, Lc, words)
+    assert r == rows and 4 <= seg <= 6
+
+
+def test_streamed_tiles_cover_every_lattice(rule):
+    """Rows and segments within the kernels' shared memory, at any size."""
+    for L, Lc, words in [(4, 4096, 2), (4096, 4, 2), (4096, 4096, 2), (6, 8, 65534), (1000, 998, 300)]:
+        seg, r = rule("rows", L, Lc, words)
+        assert r in (4, 8, 16) and seg in (4, 5, 6)
