@@ -51,5 +51,15 @@ inline RowCut row_cut(const Geometry& g, int n_words, int sms) {
     c.rows = rows;
     return c;
 }
+// The count's cut: the half-steps', in taller tiles while a word has more than 64.
+// Every tile adds 96 sums to its word's counts, so many small ones queue at the
+// same addresses (us per sweep, every sweep counted, with 16, 8 and 4 rows: 256 x
+// 256, 2 words: 37 39 43; 512 x 512, 2 words: 87 97 115; with 21 tiles of 8 rows
+// a word, 100 x 100 in 32 words: 65 63 65).
+inline RowCut count_cut(const Geometry& g, int n_words, int sms) {
+    RowCut c = row_cut(g, n_words, sms);
+    while (c.rows < kTileRows && c.tiles(g, 1) > 64) c.rows *= 2;
+    return c;
+}
 
 }  // namespace crbm

@@ -642,9 +642,10 @@ cudaError_t launch_sweep_stream(const SweepArgs& a, cudaStream_t st, int64_t* la
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    const RowCut cut = row_cut(a.g, a.n_words, sms);
+    const RowCut cut = row_cut(a.g, a.n_words, sms), ccut = count_cut(a.g, a.n_words, sms);
     const dim3 grid(((a.g.W + kTI - 1) / kTI) * ((a.g.Wc + kTJ - 1) / kTJ), a.n_words);  // bit-plane tiles
     const dim3 row_grid(static_cast<unsigned int>(cut.tiles(a.g, 1)), a.n_words);
+    const dim3 count_grid(static_cast<unsigned int>(ccut.tiles(a.g, 1)), a.n_words);
     const auto hidden = a.g.paper ? k_stream_hidden<true> : k_stream_hidden<false>;
     const auto visible = a.g.paper ? k_stream_visible<true> : k_stream_visible<false>;
     if (!a.g.bitplane && a.n_sweeps > 0) {
@@ -668,7 +669,7 @@ cudaError_t launch_sweep_stream(const SweepArgs& a, cudaStream_t st, int64_t* la
         const bool do_meas = a.measure_every > 0 && (t + 1u) % static_cast<uint32_t>(a.measure_every) == 0u;
         const bool do_swap = a.swap_every > 0 && (t + 1u) % static_cast<uint32_t>(a.swap_every) == 0u;
         if (do_meas || do_swap) {
-            k_stream_count<<<row_grid, kStreamThreads, 0, st>>>(a, cut);
+            k_stream_count<<<count_grid, kStreamThreads, 0, st>>>(a, ccut);
             if (a.swap_every > 0)
                 k_stream_post_pt<<<a.n_words, 32, 0, st>>>(a, meas, t, do_meas ? 1 : 0, do_swap ? 1 : 0);
             else

@@ -21,8 +21,8 @@ int main() {
     char rule[32];
     while (std::scanf("%31s", rule) == 1) {
         int L, Lc, words;
-        if (!std::strcmp(rule, "rows") && std::scanf("%d %d %d", &L, &Lc, &words) == 3) {
-            const crbm::RowCut c = crbm::row_cut(lattice(L, Lc), words, 152);
+        if ((!std::strcmp(rule, "rows") || !std::strcmp(rule, "count")) && std::scanf("%d %d %d", &L, &Lc, &words) == 3) {
+            const crbm::RowCut c = rule[0] == 'r' ? crbm::row_cut(lattice(L, Lc), words, 152) : crbm::count_cut(lattice(L, Lc), words, 152);
             std::printf("%d %d\n", c.seg, c.rows);
         } else {
             return 1;
