@@ -46,6 +46,8 @@
 // Adam.
 #include <algorithm>
 #include <cstring>
+#include <memory>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -1049,14 +1051,14 @@ struct crbm_proposal {
     float* m = nullptr;      // Adam moments
     float* v2 = nullptr;
     double* grad = nullptr;
-    double* loss = nullptr;  // [kLossCap], a training step each
+    double* loss = nullptr;  // [kLossCap] behind grad's [kGradPad]: a training step each
     uint16_t* bmat = nullptr;  // tensor-core B operands (bf16)
     float* bias = nullptr;     // b2, b3
     float* c1 = nullptr;     // folded layer-1 constants
     unsigned long long* stats = nullptr;
     crbm::Example* ex = nullptr;
     int ex_cap = 0;
-    char* raw = nullptr;     // crbm_proposal_loss_grad: the given spins, origins, beta and h
+    char* raw = nullptr;     // crbm_proposal_loss_grad: a slice of the given spins, origins, beta and h
     size_t raw_cap = 0;
     int train_sms = 0, train_dev = -1;  // SM count of the device the training kernel was set up on
     int64_t adam_t = 0;
@@ -1162,6 +1164,8 @@ int ensure_examples(crbm_proposal* p, int n) {
     return CRBM_OK;
 }
 
+constexpr int kGradPad = 3360;  // kNP rounded up to 256 bytes: gradient and first loss are one copy, both aligned
+static_assert(kGradPad >= kNP, "");
 constexpr int kLossCap = 1024;  // steps whose losses stay on the device before they are read back
 
 int ensure_raw(crbm_proposal* p, size_t bytes) {
@@ -1176,6 +1180,34 @@ int ensure_raw(crbm_proposal* p, size_t bytes) {
     }
     p->raw_cap = bytes;
     return CRBM_OK;
+}
+
+// crbm_proposal_loss_grad's transfers.  A copy from pageable memory takes about 8 us beside its bytes (14 ps a
+// byte), so small calls make one (one example 76 us, 100 in three copies).  Cutting a patch
+// takes the host 0.1 us: faster than copying L x L bytes on lattices of side 128 and more (8192 examples of 96 x 96:
+// whole 689 us, cut 941; 128 x 128: 1011, 932; 256 x 256: 3133, 950).
+constexpr size_t kRawBytes = 64u << 20;  // configurations on the device at a time
+constexpr size_t kOneCopy = 64u << 10;
+constexpr int kWholeSide = 112;
+static_assert(kRawBytes >= static_cast<size_t>(kWholeSide) * kWholeSide, "a slice holds a configuration");
+
+// The patch of the block at `origin` (any integers) of an L x L configuration, L >= kP, as a kP x kP one; the block's
+// place there replaces the origin.
+void cut_patch(const int8_t* v, int L, int32_t* origin, char* out) {
+    const int bR = ((origin[0] % L) + L) % L, bC = ((origin[1] % L) + L) % L;
+    const int r0 = (bR + 1) & 1, c0 = (bC + 1) & 1;  // the patch's first row and column in `out`
+    const int C = (bC - 3 + L) % L, before = std::min(crbm::kP, L - C);  // columns up to the lattice's edge
+    for (int y = 0; y < crbm::kP; ++y) {
+        const int8_t* row = v + static_cast<size_t>((bR - 3 + y + L) % L) * L;
+        char line[crbm::kP];
+        std::memcpy(line, row + C, before);
+        std::memcpy(line + before, row, crbm::kP - before);
+        char* o = out + (r0 + y) % crbm::kP * crbm::kP;
+        std::memcpy(o + c0, line, crbm::kP - c0);
+        if (c0) o[0] = line[crbm::kP - 1];
+    }
+    origin[0] = 3 + r0;
+    origin[1] = 3 + c0;
 }
 
 // Loss and gradient of the n examples in p->ex, added to *loss and p->grad.
@@ -1250,8 +1282,8 @@ int crbm_proposal_create(crbm_proposal** out, int32_t block, uint64_t seed) {
     float** bufs[] = {&p->w, &p->wb, &p->m, &p->v2};
     for (float** b : bufs)
         if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(b), kNP * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&p->grad), kNP * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&p->loss), kLossCap * sizeof(double));
+    if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&p->grad), (kGradPad + kLossCap) * sizeof(double));
+    if (e == cudaSuccess) p->loss = p->grad + kGradPad;
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&p->bmat), crbm::kBElems * sizeof(uint16_t));
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&p->bias), 33 * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&p->c1), crbm::kC1 * sizeof(float));
@@ -1282,7 +1314,7 @@ int crbm_proposal_create(crbm_proposal** out, int32_t block, uint64_t seed) {
 
 void crbm_proposal_destroy(crbm_proposal* p) {
     if (!p) return;
-    void* b[] = {p->w, p->wb, p->m, p->v2, p->grad, p->loss, p->bmat, p->bias, p->c1, p->stats, p->ex, p->raw};
+    void* b[] = {p->w, p->wb, p->m, p->v2, p->grad, p->bmat, p->bias, p->c1, p->stats, p->ex, p->raw};
     for (void* x : b)
         if (x) cudaFree(x);
     delete p;
@@ -1312,27 +1344,49 @@ int crbm_proposal_loss_grad(crbm_proposal* p, const int8_t* spins, int32_t L, co
         return prop_fail(CRBM_EINVAL, "bad arguments");
     int rc = ensure_examples(p, n);
     if (rc) return rc;
-    const size_t b_spins = static_cast<size_t>(n) * L * L, off_o = (b_spins + 15) & ~static_cast<size_t>(15);
-    rc = ensure_raw(p, off_o + 16 * static_cast<size_t>(n));
+    // The configurations go to the device in slices, as they are or, of larger lattices, cut on the host to the
+    // patches that the net reads.  A patch is a periodic lattice of side kP of its own, with the block at row and
+    // column 3 or 4 (the origin's parity).
+    const bool cut = L > kWholeSide;
+    const int side = cut ? crbm::kP : L;
+    const size_t per = static_cast<size_t>(side) * side, nn = static_cast<size_t>(n);
+    const int slice = cut ? n : static_cast<int>(std::min<size_t>(nn, kRawBytes / per));
+    const size_t off = (slice * per + 15) & ~static_cast<size_t>(15);  // origins [n][2], beta and h [n][2] behind a slice
+    rc = ensure_raw(p, off + 16 * nn);
     if (rc) return rc;
-    int32_t* d_origins = reinterpret_cast<int32_t*>(p->raw + off_o);
-    float* d_bh = reinterpret_cast<float*>(d_origins + 2 * static_cast<size_t>(n));
-    cudaError_t e = cudaMemcpy(p->raw, spins, b_spins, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(d_origins, origins, 8 * static_cast<size_t>(n), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(d_bh, beta_h, 8 * static_cast<size_t>(n), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemsetAsync(p->grad, 0, kNP * sizeof(double), nullptr);
-    if (e == cudaSuccess) e = cudaMemsetAsync(p->loss, 0, sizeof(double), nullptr);
-    if (e == cudaSuccess) {
-        crbm::k_prop_gather<<<(n + 3) / 4, 128>>>(reinterpret_cast<const int8_t*>(p->raw), L, d_origins, d_bh, p->ex, n);
-        e = cudaGetLastError();
+    const bool one_copy = off + 16 * nn <= kOneCopy;  // (then n <= slice)
+    const size_t b_host = one_copy || cut ? off + 16 * nn : 16 * nn;
+    const std::unique_ptr<char[]> host(new (std::nothrow) char[b_host]);
+    if (!host) return prop_fail(CRBM_ENOMEM, "host allocation");
+    char* tail = host.get() + b_host - 16 * nn;
+    int32_t* h_origins = reinterpret_cast<int32_t*>(tail);
+    std::memcpy(h_origins, origins, 8 * nn);
+    std::memcpy(tail + 8 * nn, beta_h, 8 * nn);
+    cudaError_t e = cudaMemsetAsync(p->grad, 0, (kGradPad + 1) * sizeof(double), nullptr);  // gradient and loss
+    const int32_t* d_origins = reinterpret_cast<const int32_t*>(p->raw + off);
+    const float* d_bh = reinterpret_cast<const float*>(d_origins + 2 * nn);
+    if (!one_copy && !cut && e == cudaSuccess) e = cudaMemcpy(p->raw + off, tail, 16 * nn, cudaMemcpyHostToDevice);
+    for (int k0 = 0; k0 < n && e == cudaSuccess; k0 += slice) {
+        const int m = std::min(slice, n - k0);
+        const int8_t* v = spins + static_cast<size_t>(k0) * L * L;
+        if (cut)
+            for (int x = 0; x < m; ++x)
+                cut_patch(v + static_cast<size_t>(x) * L * L, L, h_origins + 2 * static_cast<size_t>(x), host.get() + x * per);
+        else if (one_copy)
+            std::memcpy(host.get(), v, m * per);
+        e = cut || one_copy ? cudaMemcpy(p->raw, host.get(), b_host, cudaMemcpyHostToDevice)
+                            : cudaMemcpy(p->raw, v, m * per, cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) {
+            crbm::k_prop_gather<<<(m + 3) / 4, 128>>>(reinterpret_cast<const int8_t*>(p->raw), side, d_origins + 2 * static_cast<size_t>(k0),
+                                                     d_bh + 2 * static_cast<size_t>(k0), p->ex + k0, m);
+            e = cudaGetLastError();
+        }
     }
     if (e == cudaSuccess) e = launch_train(p, n, p->loss, nullptr);
-    double g[kNP];
+    double g[kGradPad + 1];
     if (e == cudaSuccess) e = cudaMemcpy(g, p->grad, sizeof(g), cudaMemcpyDeviceToHost);
-    double sum = 0.0;
-    if (e == cudaSuccess) e = cudaMemcpy(&sum, p->loss, sizeof(sum), cudaMemcpyDeviceToHost);
     if (e == cudaSuccess) {
-        *loss = static_cast<float>(sum);
+        *loss = static_cast<float>(g[kGradPad]);
         for (int i = 0; i < kNP; ++i) grad[i] = static_cast<float>(g[i]);
     }
     return e == cudaSuccess ? CRBM_OK : prop_fail(CRBM_ECUDA, cudaGetErrorString(e));
