@@ -143,8 +143,10 @@ __host__ __device__ inline CanonSmem canon_smem(const Geometry& g, int mode) {
     s.segmask = 160;
     s.seg = 192;
     s.u = 228;
-    const int w = g.n_cells * (mode == kCanonPacked && !g.paper ? 16 : 32);
-    s.w = place(w > canon_corr_scratch(g) ? w : canon_corr_scratch(g));
+    int w = g.n_cells * 32;
+    if (mode == kCanonPacked && !g.paper)  // (the other forms' words always hold a sample)
+        w = g.n_cells * 16 > canon_corr_scratch(g) ? g.n_cells * 16 : canon_corr_scratch(g);
+    s.w = place(w);
     s.pw = place(g.paper && mode != kCanonPacked ? g.n_cells * 64 : 0);
     s.rec = place(mode == kCanonRec ? g.n_cells * kCellRec * 4 : 0);
     s.rows = place(g.W * g.n_seg * 32);
