@@ -6,6 +6,7 @@
 #include <algorithm>
 
 #include "crbm_canon_body.cuh"
+#include "crbm_launch.h"
 
 #ifndef CRBM_SWEEP_MIN_BLOCKS
 #define CRBM_SWEEP_MIN_BLOCKS (CRBM_SWEEP_MAX_THREADS <= 512 ? 2 : 1)  // 64 registers a thread either way
@@ -139,28 +140,6 @@ size_t smem_bytes_canon(const Geometry& g) {
                          32 + 64 + 3;
     return sizeof(uint32_t) * ((words & ~static_cast<size_t>(3)) + (g.paper ? static_cast<size_t>(g.n_cells) * 64 : 0));
 }
-
-namespace {
-// Sweeps per work item: with a CTA per word, all of them; else the chunk with
-// the least (rounds of items over the grid) x (sweeps + the staging of a word,
-// 0.7 sweeps on the L=18 grid: 5.79 ms per 500 sweeps in chunks of 8, 5.56 in
-// chunks of 16).
-int pick_chunk(int n_sweeps, int n_words, int grid) {
-    if (n_words <= grid) return n_sweeps;
-    int best = n_sweeps;
-    double best_cost = 0.0;
-    for (int n_chunks = 1; n_chunks <= 64 && n_chunks <= n_sweeps; ++n_chunks) {
-        const int chunk = (n_sweeps + n_chunks - 1) / n_chunks;
-        const int64_t items = static_cast<int64_t>(n_words) * ((n_sweeps + chunk - 1) / chunk);
-        const double cost = static_cast<double>((items + grid - 1) / grid) * (chunk + 0.7);
-        if (n_chunks == 1 || cost < best_cost) {
-            best = chunk;
-            best_cost = cost;
-        }
-    }
-    return best;
-}
-}  // namespace
 
 // The segments' length.  Warp w takes segments w, w + warps, ... of a half-step
 // and runs on SM sub-partition w % 4, so the half-step takes about what the
@@ -307,8 +286,12 @@ cudaError_t make_plan(const Geometry& g0, int n_words, int warps, int dev, bool 
         p.per_sm = per_sm[0];
     }
     if (p.per_sm < 1) return cudaErrorInvalidConfiguration;
-    if ((e = check_dynamic_smem_base(reinterpret_cast<const void*>(persistent_kernel(p.mode, g.paper, p.cta)), dev)) != cudaSuccess)
-        return e;
+    // a CTA per word: the instantiation with the most CTAs per SM
+    p.all_cta = per_sm[1] >= per_sm[0] ? kCtaPair : kCtaAny;
+    p.resident = std::max(1, std::max(per_sm[0], per_sm[1]));
+    for (const int cta : {p.cta, p.all_cta})
+        if ((e = check_dynamic_smem_base(reinterpret_cast<const void*>(persistent_kernel(p.mode, g.paper, cta)), dev)) != cudaSuccess)
+            return e;
     p.warps = warps;
     p.device = dev;
     return cudaSuccess;
@@ -336,15 +319,22 @@ cudaError_t launch_sweep_canon_persistent(const SweepArgs& a0, int warps_per_cta
     // no more CTAs per SM than whole words: were every word held at once, SMs with one word more
     // than others would finish last with nothing to claim for the rest
     const int per_sm = std::max(1, std::min(plan.per_sm, a.n_words / plan.sms));
-    const int grid = std::min(a.n_words, per_sm * plan.sms);
-    const int chunk = pick_chunk(a.n_sweeps, a.n_words, grid);
+    int grid = std::min(a.n_words, per_sm * plan.sms), cta = plan.cta, chunk = a.n_sweeps;
+    if (grid < a.n_words) {
+        const CanonSchedule sc = canon_schedule(a.n_sweeps, a.n_words, a.g.n_cells, plan.sms, per_sm, plan.resident);
+        chunk = sc.chunk;
+        if (sc.all) {
+            grid = a.n_words;
+            cta = plan.all_cta;
+        }
+    }
     if (grid == a.n_words) {
         sched = nullptr;
     } else {
         e = cudaMemsetAsync(sched, 0, sizeof(int) * (4 + static_cast<size_t>(a.n_words)), st);
         if (e != cudaSuccess) return e;
     }
-    persistent_kernel(plan.mode, a.g.paper, plan.cta)<<<grid, warps_per_cta * 32, plan.smem, st>>>(a, chunk, sched);
+    persistent_kernel(plan.mode, a.g.paper, cta)<<<grid, warps_per_cta * 32, plan.smem, st>>>(a, chunk, sched);
     return cudaGetLastError();
 }
 

@@ -304,6 +304,7 @@ size_t canon_plan(Geometry& g, int warps, int* mode, int bands = 1);
 struct CanonLaunch {
     int warps = 0, device = -1;  // what they were made for
     int mode = 0, seg_cells = 0, n_seg = 0, cta = 0, per_sm = 0, sms = 0, bands = 1;
+    int all_cta = 0, resident = 0;  // a CTA per word, more words than CTAs at once: instantiation, CTAs per SM
     size_t smem = 0;
 };
 // cudaErrorInvalidConfiguration unless dynamic_smem_at_base holds for `kernel` on device `dev` (a row-form

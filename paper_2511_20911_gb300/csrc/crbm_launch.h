@@ -62,4 +62,42 @@ inline RowCut count_cut(const Geometry& g, int n_words, int sms) {
     return c;
 }
 
+// ---- canonical SMEM sweep: how a launch with more words than resident CTAs
+// runs.  `all`: a CTA per word for the whole launch, placed by the hardware;
+// else a persistent grid over (word, chunk of sweeps) items.
+struct CanonSchedule {
+    bool all;
+    int chunk;  // sweeps per item
+};
+// Persistent: the chunk with the least (rounds of items over the grid of per_sm
+// CTAs per SM) x (sweeps + the staging of a word, 0.7 sweeps on the L=18 grid:
+// 5.79 ms per 500 sweeps in chunks of 8, 5.56 in chunks of 16).  It balances the
+// SMs, at a staging and a claim (a scan of every word's state) per item.
+// All: for short launches, of up to eight stagings a word, where the fullest SM's
+// words and their staging, once for every `resident` of them, cost less.  By
+// estimates (us): a word's sweep takes an SM 0.7 + 0.042 a cell, its staging 5 +
+// 0.009 a cell.  us per launch of one sweep, persistent -> all, 1600 words: L = 4
+// 191 -> 19, L = 6 186 -> 21, L = 12 246 -> 43; 384 words of L = 18 34 -> 21.
+inline CanonSchedule canon_schedule(int n_sweeps, int n_words, int n_cells, int sms, int per_sm, int resident) {
+    const int64_t grid = static_cast<int64_t>(per_sm) * sms;
+    CanonSchedule best{false, n_sweeps};
+    int64_t rounds = 0;
+    double best_cost = 0.0;
+    for (int n_chunks = 1; n_chunks <= 64 && n_chunks <= n_sweeps; ++n_chunks) {
+        const int chunk = (n_sweeps + n_chunks - 1) / n_chunks;
+        const int64_t items = static_cast<int64_t>(n_words) * ((n_sweeps + chunk - 1) / chunk);
+        const double cost = static_cast<double>((items + grid - 1) / grid) * (chunk + 0.7);
+        if (n_chunks == 1 || cost < best_cost) {
+            best.chunk = chunk;
+            best_cost = cost;
+            rounds = (items + grid - 1) / grid;
+        }
+    }
+    const double sweep = 0.7 + 0.042 * n_cells, stage = 5.0 + 0.009 * n_cells;
+    if (sweep * n_sweeps > 8.0 * stage) return best;
+    const int most = (n_words + sms - 1) / sms;  // words of the fullest SM
+    const double all = most * sweep * n_sweeps + (most + resident - 1) / resident * stage;
+    return all <= static_cast<double>(rounds) * (best.chunk * per_sm * sweep + stage) ? CanonSchedule{true, n_sweeps} : best;
+}
+
 }  // namespace crbm

@@ -24,6 +24,11 @@ int main() {
         if ((!std::strcmp(rule, "rows") || !std::strcmp(rule, "count")) && std::scanf("%d %d %d", &L, &Lc, &words) == 3) {
             const crbm::RowCut c = rule[0] == 'r' ? crbm::row_cut(lattice(L, Lc), words, 152) : crbm::count_cut(lattice(L, Lc), words, 152);
             std::printf("%d %d\n", c.seg, c.rows);
+        } else if (!std::strcmp(rule, "schedule")) {
+            int sweeps, cells, per_sm, resident;
+            if (std::scanf("%d %d %d %d %d", &sweeps, &words, &cells, &per_sm, &resident) != 5) return 1;
+            const crbm::CanonSchedule c = crbm::canon_schedule(sweeps, words, cells, 152, per_sm, resident);
+            std::printf("%d %d\n", c.all ? 1 : 0, c.chunk);
         } else {
             return 1;
         }

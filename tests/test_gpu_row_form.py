@@ -75,3 +75,38 @@ def test_split_ladders_match_whole_words(orc, ladders, precision):
     assert np.array_equal(few.series(), many.series()[:, :n])
     assert np.array_equal(few.permutation(), many.permutation()[:n])
     assert np.array_equal(few.first_hits(), many.first_hits()[:n])
+
+
+@pytest.mark.parametrize("L,words,precision,splits", [(4, 161, EXACT, [1, 2, 40]), (6, 310, PAPER, [1, 40]), (4, 700, EXACT, [1, 3, 30]),
+                                                      (18, 160, EXACT, [1, 3]), (30, 305, PAPER, [1, 2])])
+def test_more_words_than_ctas(orc, L, words, precision, splits, monkeypatch):
+    """Short launches give every word a CTA, long ones claim chunks of words from a persistent grid."""
+    monkeypatch.delenv("CRBM_WARPS", raising=False)
+    n = 32 * words - 5
+    params = workloads.random_params(np.random.default_rng(L + words), 3)
+    cp = (np.arange(n) // 7 % 3).astype(np.int32)
+    s = crbm.Sampler(L, params, n, chain_param=cp, seed=words, measure_every=2, precision=precision)
+    ids = np.arange(n, dtype=np.uint32)
+    spins, sums, t = orc.init_spins(L, ids, words), None, 0
+    for k in splits:
+        s.sweep(k)
+        sums, _, _ = orc.run(L, params, cp, spins, words, t, k, 2, chain_ids=ids, sums=sums, precision=precision)
+        t += k
+        assert np.array_equal(s.get_spins(), spins), f"spins after {t} sweeps"
+    assert np.array_equal(s.observables(), sums)
+
+
+# records from global memory and 16-bit hidden words, more words than CTAs: a CTA's second word finds the first's expansion table
+@pytest.mark.parametrize("L,precision", [(64, EXACT), (68, EXACT), (38, PAPER), (52, PAPER)])
+def test_large_lattices_on_a_persistent_grid(L, precision, monkeypatch):
+    """A context of 170 words against the same chains in a context of 2 (split, or a CTA per word)."""
+    monkeypatch.delenv("CRBM_WARPS", raising=False)
+    params = workloads.random_params(np.random.default_rng(L), 3)
+    cp = (np.arange(32 * 170) % 3).astype(np.int32)
+    many = crbm.Sampler(L, params, 32 * 170, chain_param=cp, seed=9, measure_every=3, precision=precision)
+    few = crbm.Sampler(L, params, 64, chain_param=cp[:64], seed=9, measure_every=3, precision=precision)
+    for s in (many, few):
+        s.sweep(1)
+        s.sweep(60)
+    assert np.array_equal(many.get_spins()[:64], few.get_spins())
+    assert np.array_equal(many.observables()[:64], few.observables())

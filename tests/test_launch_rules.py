@@ -48,3 +48,20 @@ def test_streamed_tiles_cover_every_lattice(rule):
                                              (100, 100, 2, 4), (64, 64, 2, 4), (100, 100, 32, 8)])
 def test_streamed_count_rows(rule, L, Lc, words, rows):
     assert rule("count", L, Lc, words)[1] == rows
+
+
+# sweeps, words, cells, CTAs per SM of the persistent grid, resident CTAs of a CTA per word: a one-sweep launch of 1600
+# words of L = 4 took 191 us through the scheduler, 46 with a CTA per word; long launches balance the SMs in chunks
+@pytest.mark.parametrize("sweeps,words,cells,per_sm,resident,everything", [
+    (1, 1600, 4, 4, 4, 1), (1, 1600, 9, 4, 4, 1), (4, 384, 9, 2, 4, 1), (1, 250, 81, 1, 2, 1), (4, 384, 81, 2, 3, 1),
+    (1, 384, 225, 2, 2, 1), (500, 384, 81, 2, 3, 0), (2000, 384, 81, 2, 3, 0), (500, 250, 81, 1, 2, 0)])
+def test_short_launches_take_a_cta_per_word(rule, sweeps, words, cells, per_sm, resident, everything):
+    every, chunk = rule("schedule", sweeps, words, cells, per_sm, resident)
+    assert every == everything
+    assert chunk == sweeps if every else 1 <= chunk < sweeps
+
+
+def test_schedule_chunks_at_any_size(rule):
+    for args in [(1, 153, 4, 1, 1), (1 << 20, 1 << 20, 2304, 1, 1), (7, 100000, 4, 4, 4), (1 << 20, 153, 4, 4, 4)]:
+        every, chunk = rule("schedule", *args)
+        assert 1 <= chunk <= args[0] and (not every or chunk == args[0])
