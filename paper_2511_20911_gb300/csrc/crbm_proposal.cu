@@ -1401,8 +1401,20 @@ int crbm_proposal_train(crbm_proposal* p, crbm_ctx* ctx, int32_t steps, int32_t 
     if (!rc) rc = ensure_examples(p, batch);
     if (rc) return rc;
     cudaStream_t st = ctx->stream;
+    // the losses of steps s0 .. s0 + k - 1 (k <= kLossCap, of one filling of p->loss) to the caller
+    auto read_losses = [&](int s0, int k) {
+        double sums[kLossCap];
+        cudaError_t e = cudaMemcpyAsync(sums, p->loss, sizeof(double) * static_cast<size_t>(k), cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        for (int i = 0; e == cudaSuccess && i < k; ++i) losses[s0 + i] = static_cast<float>(sums[i]);
+        return e;
+    };
     for (int s = 0; s < steps; ++s) {
-        if (sweeps_between > 0 && (rc = crbm_sweep(ctx, sweeps_between))) return prop_fail(rc, crbm_last_error(ctx));
+        if (sweeps_between > 0 && (rc = crbm_sweep(ctx, sweeps_between))) {
+            const std::string what = crbm_last_error(ctx);
+            if (losses && s % kLossCap) read_losses(s - s % kLossCap, s % kLossCap);  // the finished steps' losses
+            return prop_fail(rc, what);
+        }
         double* step_loss = p->loss + s % kLossCap;  // read back kLossCap steps at a time
         crbm::k_prop_extract<<<(batch + 3) / 4, 128, 0, st>>>(
             ctx->g, ctx->d.v, ctx->d.chain_bh, ctx->n_chains, p->ex, batch,
@@ -1420,13 +1432,7 @@ int crbm_proposal_train(crbm_proposal* p, crbm_ctx* ctx, int32_t steps, int32_t 
                                                                   b1, b2, 1e-8f, c1, c2);
             e = cudaGetLastError();
         }
-        if (e == cudaSuccess && losses && (s % kLossCap == kLossCap - 1 || s == steps - 1)) {
-            const int s0 = s - s % kLossCap;
-            double sums[kLossCap];
-            e = cudaMemcpyAsync(sums, p->loss, sizeof(double) * static_cast<size_t>(s - s0 + 1), cudaMemcpyDeviceToHost, st);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-            for (int k = s0; e == cudaSuccess && k <= s; ++k) losses[k] = static_cast<float>(sums[k - s0]);
-        }
+        if (e == cudaSuccess && losses && (s % kLossCap == kLossCap - 1 || s == steps - 1)) e = read_losses(s - s % kLossCap, s % kLossCap + 1);
         if (e != cudaSuccess) return prop_fail(CRBM_ECUDA, std::string("train: ") + cudaGetErrorString(e));
     }
     const cudaError_t e = refresh_fragments(p, st);

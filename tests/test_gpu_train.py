@@ -81,3 +81,20 @@ def test_loss_grad_memory_does_not_grow_with_the_lattice():
     free = torch.cuda.mem_get_info()[0]
     p.loss_grad(spins, np.zeros((200, 2), np.int32), np.ones((200, 2), np.float32))
     assert free - torch.cuda.mem_get_info()[0] <= 32 << 20
+
+
+def test_losses_of_the_steps_before_a_failing_one():
+    """A training step whose sweeps fail (here the 32-bit sweep counter) leaves the finished steps' losses written."""
+    import ctypes
+    n = 64
+    s = crbm.Sampler(10, dict(J=[1.0], Jp=[1.0], h=[0.5], beta=[1.0]), n, seed=3, measure_every=0)
+    ck = s.save()
+    ck[:128].view(np.int64)[6] = 2 ** 32 - 1 - 5   # sweeps so far: two steps of two sweeps still fit
+    s.load(ck)
+    p = crbm.Proposal(seed=2)
+    losses = np.full(4, np.nan, np.float32)
+    lib = crbm.load_library()
+    rc = lib.crbm_proposal_train(p._p, s._ctx, 4, 32, ctypes.c_float(1e-2), 2,
+                                 losses.ctypes.data_as(ctypes.POINTER(ctypes.c_float)))
+    assert rc == crbm.CRBM_EINVAL
+    assert np.isfinite(losses[:2]).all() and (losses[:2] > 0).all() and np.isnan(losses[2:]).all()
