@@ -73,7 +73,8 @@ struct CanonSchedule {
 // CTAs per SM) x (sweeps + the staging of a word, 0.7 sweeps on the L=18 grid:
 // 5.79 ms per 500 sweeps in chunks of 8, 5.56 in chunks of 16).  It balances the
 // SMs, at a staging and a claim (a scan of every word's state) per item.
-// All: for short launches, of up to eight stagings a word, where the fullest SM's
+// All: where one chunk per word is the best anyway (265 sweeps of 600 words of
+// L = 14 on 304 CTAs, us per sweep: claimed 14.5, placed 11.7), and for short launches, of up to eight stagings a word, where the fullest SM's
 // words and their staging, once for every `resident` of them, cost less.  By
 // estimates (us): a word's sweep takes an SM 0.7 + 0.042 a cell, its staging 5 +
 // 0.009 a cell.  us per launch of one sweep, persistent -> all, 1600 words: L = 4
@@ -93,6 +94,7 @@ inline CanonSchedule canon_schedule(int n_sweeps, int n_words, int n_cells, int 
             rounds = (items + grid - 1) / grid;
         }
     }
+    if (best.chunk >= n_sweeps) return {true, n_sweeps};
     const double sweep = 0.7 + 0.042 * n_cells, stage = 5.0 + 0.009 * n_cells;
     if (sweep * n_sweeps > 8.0 * stage) return best;
     const int most = (n_words + sms - 1) / sms;  // words of the fullest SM

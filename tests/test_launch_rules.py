@@ -54,7 +54,7 @@ def test_streamed_count_rows(rule, L, Lc, words, rows):
 # words of L = 4 took 191 us through the scheduler, 46 with a CTA per word; long launches balance the SMs in chunks
 @pytest.mark.parametrize("sweeps,words,cells,per_sm,resident,everything", [
     (1, 1600, 4, 4, 4, 1), (1, 1600, 9, 4, 4, 1), (4, 384, 9, 2, 4, 1), (1, 250, 81, 1, 2, 1), (4, 384, 81, 2, 3, 1),
-    (1, 384, 225, 2, 2, 1), (500, 384, 81, 2, 3, 0), (2000, 384, 81, 2, 3, 0), (500, 250, 81, 1, 2, 0)])
+    (1, 384, 225, 2, 2, 1), (265, 600, 49, 2, 2, 1), (500, 384, 81, 2, 3, 0), (2000, 384, 81, 2, 3, 0), (500, 250, 81, 1, 2, 0)])
 def test_short_launches_take_a_cta_per_word(rule, sweeps, words, cells, per_sm, resident, everything):
     every, chunk = rule("schedule", sweeps, words, cells, per_sm, resident)
     assert every == everything
