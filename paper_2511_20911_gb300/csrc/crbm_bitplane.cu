@@ -37,7 +37,7 @@ constexpr int kBpMaxThreads = CRBM_SWEEP_MAX_THREADS;  // largest CTA the launch
 // What bounds it: the half-steps' barriers and the ALU pipe (L=18, 384 words:
 // ALU 47 %, with the wide multiplies' share 74 % of its slots; 5.7 of 13.6
 // stalled warps at barriers).
-// Default CTA (default_warps): with less than three words per SM one round of
+// Default CTA (sweep_warps, crbm_launch.h): with less than three words per SM one round of
 // node groups, up to 16 warps, finishes a word's half-step soonest; with more,
 // smaller CTAs, of which more are resident, fill each other's barriers.  us per
 // sweep, a warp per six cells always -> by this rule: L=6 3.2 -> 2.8 (152

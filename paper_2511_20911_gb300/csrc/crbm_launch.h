@@ -9,6 +9,42 @@
 
 namespace crbm {
 
+// ---- warps per CTA of the SMEM sweeps
+// Bit-plane sweep: with less than three words per SM one round of node groups, up
+// to 16 warps, finishes a word's half-step soonest; with more, smaller CTAs, of
+// which more are resident, fill each other's barriers; the smallest lattices
+// take so few warps that every word is resident, else the words queue at the
+// scheduler (us per sweep with 4, 3, 1 warps,
+// 1600 words: L = 4 9.1 4.4 4.4, L = 6 9.6 5.8 6.0, L = 8 10.4 7.0 7.4, L = 12 13.8
+// 14.0 14.4; 3000 words: 12.3 10.8 7.5, 14.0 12.4 10.2, 15.6 14.0 12.5, 23.9
+// 23.1 24.0).
+// Generic sweep (us per sweep with 4, 8, 16 warps, 48 words of 18 x 12
+// spins: 8.8 6.2 5.4, 304 words: 11.7 9.8 10.7, 600 words: 18.7 19.1 21.1, of 9 x 9
+// spins 9.1 10.0 11.5): fewer warps the more words an SM has.  The canonical sweep, by whether every SM has two
+// words or more (us per sweep of 384 words with 4, 8, 12, 16 warps: L = 6 2.65
+// 2.81, L = 12 6.07 6.07 5.42 5.50, L = 18 11.5 10.6 11.0 11.4, L = 24 21.1 18.7 -
+// 18.5, L = 30 32.6 29.1 28.8 28.4; of 152 words with 8, 16, 32: L = 18 5.1 4.6
+// 4.7, L = 48 30.1 26.6 26.4, L = 64 74.4 50.2 47.6; L = 6, every sweep measured:
+// 1.29 with 9 warps, 1.20 with 12, one of them free to finish the measurements).
+inline int sweep_warps(const Geometry& g, int n_words, int sms) {
+    if (g.bitplane) {
+        const int groups = (g.n_cells * 10 + 31) / 32;
+        const int round = (groups + 3) & ~3;  // one round of hidden groups
+        const int per = (n_words + sms - 1) / sms;  // words of the fullest SM; 36 warps of 56 registers a thread fit
+        const int w = n_words >= 5 * sms   ? (groups > 12 ? 8 : groups > 8 || per <= 9 ? 4 : per <= 12 || groups > 5 ? 3 : 1)
+                      : n_words >= 3 * sms ? (groups <= 12 ? std::min(8, round) : 12)
+                      : groups <= 16       ? std::min(12, round)
+                                           : std::min(16, (g.n_cells + 5) / 6);
+        return std::max(1, std::min(kMaxSweepWarps, w));
+    }
+    if (!g.canonical)
+        return std::max(1, std::min(std::min(n_words <= sms ? 16 : n_words < 3 * sms || g.n_cells >= 64 ? 8 : 4, kMaxSweepWarps),
+                                    g.n_cells));
+    if (n_words >= 2 * sms && g.n_cells <= 400)  // (larger ones hold one CTA per SM)
+        return std::min(kMaxSweepWarps, g.n_cells < 16 ? 4 : g.n_cells < 30 || (g.n_cells >= 50 && g.n_cells <= 144) ? 8 : 12);
+    return std::min(kMaxSweepWarps, g.n_cells < 8 ? 8 : g.n_cells <= 16 ? 12 : g.n_cells <= 600 || 2 * n_words <= sms ? 16 : 32);
+}
+
 // ---- streamed lane-uniform sweep: tiles of `rows` rows of cells by `seg`
 // segments of three, rows in {4, 8, 16}, seg in {4, 5, 6}
 constexpr int kTileRows = 16, kMaxTileSeg = 6;

@@ -24,6 +24,10 @@ int main() {
         if ((!std::strcmp(rule, "rows") || !std::strcmp(rule, "count")) && std::scanf("%d %d %d", &L, &Lc, &words) == 3) {
             const crbm::RowCut c = rule[0] == 'r' ? crbm::row_cut(lattice(L, Lc), words, 152) : crbm::count_cut(lattice(L, Lc), words, 152);
             std::printf("%d %d\n", c.seg, c.rows);
+        } else if (!std::strcmp(rule, "bitplane") && std::scanf("%d %d %d", &L, &Lc, &words) == 3) {
+            crbm::Geometry g = lattice(L, Lc);
+            g.bitplane = 1;
+            std::printf("%d\n", crbm::sweep_warps(g, words, 152));
         } else if (!std::strcmp(rule, "schedule")) {
             int sweeps, cells, per_sm, resident;
             if (std::scanf("%d %d %d %d %d", &sweeps, &words, &cells, &per_sm, &resident) != 5) return 1;
