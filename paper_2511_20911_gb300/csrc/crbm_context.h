@@ -13,6 +13,7 @@ struct crbm_ctx {
     int n_chains = 0, n_words = 0, n_params = 0;
     int layout = CRBM_LAYOUT_SMEM;
     int warps = 8;
+    bool tuned = false;     // warps: from CRBM_WARPS, the cache or crbm_autotune, not by the rule
     uint64_t seed = 0;
     int measure_every = 0, series_len = 0, sq_every = 0, swap_every = 0;
     int64_t sweeps = 0;     // global sweep counter

@@ -238,13 +238,15 @@ void free_device(DeviceState& d) {
     d = DeviceState{};
 }
 
-// Warps per CTA of the SMEM sweeps unless the context is tuned: CRBM_WARPS, or
-// the rule of crbm_launch.h for the device's SMs.
+// CRBM_WARPS, or 0.
+int env_warps() {
+    const char* env = std::getenv("CRBM_WARPS");
+    const int w = env ? std::atoi(env) : 0;
+    return w >= 1 && w <= kMaxSweepWarps ? w : 0;
+}
+
+// The warps per CTA by the rule of crbm_launch.h, for the current device's SMs.
 int default_warps(const Geometry& g, int n_words) {
-    if (const char* env = std::getenv("CRBM_WARPS")) {
-        const int w = std::atoi(env);
-        if (w >= 1 && w <= kMaxSweepWarps) return w;
-    }
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
@@ -398,7 +400,9 @@ int crbm_create(crbm_ctx** out, const crbm_params* p) {
     ctx->series_len = p->series_len;
     ctx->sq_every = p->sq_every;
     ctx->stream = static_cast<cudaStream_t>(p->stream);
-    ctx->warps = default_warps(g, ctx->n_words);
+    ctx->warps = env_warps();
+    ctx->tuned = ctx->warps > 0;
+    if (!ctx->tuned) ctx->warps = default_warps(g, ctx->n_words);
     for (int k = 0; k < 3; ++k) ctx->q[k].resize(p->n_params);
     ctx->q_odd.resize(p->n_params);
     ctx->beta.assign(p->beta, p->beta + p->n_params);
@@ -777,7 +781,10 @@ int crbm_create(crbm_ctx** out, const crbm_params* p) {
     }
     ctx->launches = 1;
     if (!std::getenv("CRBM_WARPS") && ctx->layout == CRBM_LAYOUT_SMEM)
-        if (const int w = autotune_lookup(ctx)) ctx->warps = w;  // shape tuned earlier on this GPU
+        if (const int w = autotune_lookup(ctx)) {  // shape tuned earlier on this GPU
+            ctx->warps = w;
+            ctx->tuned = true;
+        }
     *out = ctx;
     return CRBM_OK;
 }

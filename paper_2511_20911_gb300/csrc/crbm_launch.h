@@ -45,6 +45,20 @@ inline int sweep_warps(const Geometry& g, int n_words, int sms) {
     return std::min(kMaxSweepWarps, g.n_cells < 8 ? 8 : g.n_cells <= 16 ? 12 : g.n_cells <= 600 || 2 * n_words <= sms ? 16 : 32);
 }
 
+// ---- batched launch: warps per CTA of members at their rules' shapes
+// With a CTA per SM at most, the largest member's (`warps`).  With more, so many
+// that registers (128 a thread) let as many CTAs share an SM as shared memory
+// does, up to four and to the CTAs per SM: a CTA alone on its SM waits at its
+// barriers, and CTAs wait for SMs (us per sweep, 16 or 12 warps -> by this rule:
+// 600 words of L = 12 37.9 -> 14.9, 150 of L = 18 and 100 of L = 12 31.2 -> 13.7,
+// 300 of L = 6 and 300 of L = 8 4.3 -> 3.3, 200 of L = 30 39.7 -> 23.7, 400 of
+// 9 x 9 7.9 -> 7.3, 300 of L = 18 in paper precision 5.8 -> 5.7).
+inline int batch_warps(int warps, int n_ctas, size_t smem, int sms) {
+    const int per = (n_ctas + sms - 1) / sms, fit = static_cast<int>(228 * 1024 / (smem + kReservedSmem));
+    const int share = std::min(std::min(per, fit), 4);
+    return share <= 1 ? warps : std::min(warps, share == 2 ? 8 : 4);
+}
+
 // ---- streamed lane-uniform sweep: tiles of `rows` rows of cells by `seg`
 // segments of three, rows in {4, 8, 16}, seg in {4, 5, 6}
 constexpr int kTileRows = 16, kMaxTileSeg = 6;

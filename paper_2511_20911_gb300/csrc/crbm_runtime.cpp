@@ -17,6 +17,7 @@
 #include <sys/stat.h>
 
 #include "crbm_context.h"
+#include "crbm_launch.h"
 
 using namespace crbm;
 
@@ -161,6 +162,7 @@ int crbm_autotune(crbm_ctx* ctx, int64_t probe_sweeps, int32_t* best_warps) {
         return CRBM_ECUDA;
     }
     ctx->warps = best;
+    ctx->tuned = true;
     if (best_warps) *best_warps = best;
     std::lock_guard<std::mutex> lock(g_cache_mutex);
     const std::string path = cache_path();
@@ -237,6 +239,7 @@ int crbm_batch_create(crbm_batch** out, crbm_ctx* const* ctxs, int32_t n_ctx) {
     crbm_batch* b = new (std::nothrow) crbm_batch();
     if (!b) return CRBM_ENOMEM;
     int warps = 1;
+    bool tuned = false;
     for (int c = 0; c < n_ctx; ++c) {
         crbm_ctx* x = ctxs[c];
         if (!x || x->layout != CRBM_LAYOUT_SMEM || x->stream != ctxs[0]->stream ||
@@ -247,6 +250,7 @@ int crbm_batch_create(crbm_batch** out, crbm_ctx* const* ctxs, int32_t n_ctx) {
         }
         b->ctx.push_back(x);
         warps = std::max(warps, x->warps);
+        tuned = tuned || x->tuned;
         if (x->g.paper) b->modes |= kBatchPaper;
         if (x->g.bitplane) b->modes |= kBatchBitplane;
     }
@@ -307,6 +311,12 @@ int crbm_batch_create(crbm_batch** out, crbm_ctx* const* ctxs, int32_t n_ctx) {
     for (auto& p : whole) items.push_back(p.second);
     while (items.size() % static_cast<size_t>(cluster)) items.push_back(make_int4(-1, 0, 0, 1));
     b->cluster = cluster;
+    if (!tuned) {  // more CTAs than SMs: of a size that lets them share an SM
+        int sms = 0;
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctxs[0]->device) != cudaSuccess || sms < 1) sms = 152;
+        const int w = batch_warps(warps, static_cast<int>(items.size()), b->smem, sms);
+        if (w != warps) set_threads(b, 32 * w);
+    }
     std::vector<int> every;
     for (auto* x : b->ctx) every.push_back(x->measure_every);
     b->stream = ctxs[0]->stream;

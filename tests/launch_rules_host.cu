@@ -28,6 +28,10 @@ int main() {
             crbm::Geometry g = lattice(L, Lc);
             g.bitplane = 1;
             std::printf("%d\n", crbm::sweep_warps(g, words, 152));
+        } else if (!std::strcmp(rule, "batch")) {
+            int warps, ctas, smem;
+            if (std::scanf("%d %d %d", &warps, &ctas, &smem) != 3) return 1;
+            std::printf("%d\n", crbm::batch_warps(warps, ctas, smem, 152));
         } else if (!std::strcmp(rule, "schedule")) {
             int sweeps, cells, per_sm, resident;
             if (std::scanf("%d %d %d %d %d", &sweeps, &words, &cells, &per_sm, &resident) != 5) return 1;

@@ -303,3 +303,35 @@ def test_autotune_probes_do_the_work_of_the_context(tmp_path, monkeypatch):
     before = s.correlations()[0]
     assert seconds(lambda: s.autotune(20)) > 3 * sweeps
     assert np.array_equal(s.correlations()[0], before)
+
+
+def test_batch_of_more_ctas_than_sms():
+    """Small CTAs (four to an SM) of split, whole, generic, paper-precision and bit-plane words; a tuned member keeps
+    its shape."""
+    rng = np.random.default_rng(80)
+    specs = [dict(L=L, params=workloads.random_params(rng, 3), n_chains=n, chain_param=rng.integers(0, 3, n).astype(np.int32),
+                  seed=40 + k, measure_every=3, **kw)
+             for k, (L, n, kw) in enumerate([(12, 2550, {}), (18, 1000, {}), (9, 640, {}), (10, 640, dict(precision=crbm.CRBM_PRECISION_PAPER)),
+                                             (8, 640, dict(rng=crbm.CRBM_RNG_BITPLANE))])]
+    batched = [make(s) for s in specs]
+    twins = [make(s) for s in specs]
+    batch = crbm.Batch(batched)
+    assert batch.threads <= 256
+    for n in (1, 4, 9):
+        batch.sweep(n)
+        for t in twins:
+            t.sweep(n)
+    for a, b in zip(batched, twins):
+        same(a, b)
+    batch.close()
+
+
+def test_batch_keeps_a_tuned_shape(monkeypatch):
+    specs = [dict(L=12, params=workloads.random_params(np.random.default_rng(81), 2), n_chains=32 * 200, seed=50 + k) for k in range(2)]
+    monkeypatch.setenv("CRBM_WARPS", "12")
+    tuned = make(specs[0])
+    monkeypatch.delenv("CRBM_WARPS")
+    other = make(specs[1])
+    batch = crbm.Batch([tuned, other])
+    assert batch.threads == 32 * max(12, other.warps)
+    batch.close()

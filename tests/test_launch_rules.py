@@ -73,3 +73,11 @@ def test_schedule_chunks_at_any_size(rule):
                                            (48, 250, 16), (48, 160, 16), (40, 250, 16), (4, 250, 4)])
 def test_bitplane_warps(rule, L, words, warps):
     assert rule("bitplane", L, L, words) == (warps,)
+
+
+# warps of the largest member, CTAs, shared memory of a CTA: 1200 CTAs of half words of L = 12 took 37.9 us a sweep at 12
+# warps, a CTA per SM, and 14.9 at 4, four per SM; L = 48 (170 KB) is alone on its SM at any size
+@pytest.mark.parametrize("warps,ctas,smem,chosen", [(12, 1200, 56320, 4), (16, 120, 174000, 16), (16, 480, 174000, 16), (16, 152, 57000, 16),
+                                                    (16, 160, 60000, 8), (16, 1600, 95000, 8), (4, 800, 56320, 4), (16, 400, 70000, 4)])
+def test_batch_warps(rule, warps, ctas, smem, chosen):
+    assert rule("batch", warps, ctas, smem) == (chosen,)
