@@ -177,26 +177,31 @@ __device__ __forceinline__ void sweep_canon_body(const SweepArgs& a, int word, u
                              : "memory");
         };
         stage(tab + kRowVis, reinterpret_cast<const uint4*>(gt + kCanonTh), 4 * 32 * 32 / 4);
-        if (kMode == kCanonRec && first) stage(rec_addr, a.crec, g.n_cells * kCellRec);
+        if (kMode == kCanonRec && first) {
+            const int c0 = kCluster ? row0 * Wc : 0, c1 = kCluster ? row1 * Wc : g.n_cells;
+            stage(rec_addr + 16u * kCellRec * static_cast<uint32_t>(c0), a.crec + static_cast<size_t>(c0) * kCellRec, (c1 - c0) * kCellRec);
+        }
         // spins to row form: the site words of a segment's word (lane = bit), bit-transposed (lane = chain)
         const uint32_t* gv = a.v + static_cast<size_t>(word) * g.N;
         const Transpose32 transpose(lane);
         const SegmentSites site(g.Lc, lane);
-        for (int u0 = warp; u0 < W * nseg; u0 += 4 * nwarp) {
+        // (a band: its own rows and the one below them; the rest of the lattice is never read)
+        const int n_staged = kCluster ? min(u_end - u_begin + nseg, W * nseg) : W * nseg;
+        auto staged = [&](int x) { return !kCluster ? x : u_begin + x < W * nseg ? u_begin + x : u_begin + x - W * nseg; };
+        for (int u0 = warp; u0 < n_staged; u0 += 4 * nwarp) {
             uint32_t v[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const int u = u0 + k * nwarp;
                 v[k] = 0u;
-                if (u < W * nseg) {
-                    const Segment sg = segment(u);
+                if (u0 + k * nwarp < n_staged) {
+                    const Segment sg = segment(staged(u0 + k * nwarp));
                     const int sx = site(lane, sg.i, sg.j0, sg.n, sg.j0 + sg.n == Wc ? 0 : sg.j0 + sg.n);
                     if (lane >= 14 && lane < 16 + 4 * sg.n) v[k] = __ldcg(gv + sx);
                 }
             }
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                if (u0 + k * nwarp < W * nseg) sts32(row_addr(u0 + k * nwarp), transpose(v[k]));
+                if (u0 + k * nwarp < n_staged) sts32(row_addr(staged(u0 + k * nwarp)), transpose(v[k]));
         }
         build_threshold_tables(s_tab, gt, threadIdx.x, blockDim.x);
         if (kPacked && first)
