@@ -246,12 +246,12 @@ int env_warps() {
 }
 
 // The warps per CTA by the rule of crbm_launch.h, for the current device's SMs.
-int default_warps(const Geometry& g, int n_words) {
+int default_warps(const Geometry& g, int n_words, bool correlations) {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
         sms = 152;
-    return sweep_warps(g, n_words, sms);
+    return sweep_warps(g, n_words, sms, correlations);
 }
 
 }  // namespace
@@ -402,7 +402,7 @@ int crbm_create(crbm_ctx** out, const crbm_params* p) {
     ctx->stream = static_cast<cudaStream_t>(p->stream);
     ctx->warps = env_warps();
     ctx->tuned = ctx->warps > 0;
-    if (!ctx->tuned) ctx->warps = default_warps(g, ctx->n_words);
+    if (!ctx->tuned) ctx->warps = default_warps(g, ctx->n_words, p->sq_every > 0);
     for (int k = 0; k < 3; ++k) ctx->q[k].resize(p->n_params);
     ctx->q_odd.resize(p->n_params);
     ctx->beta.assign(p->beta, p->beta + p->n_params);

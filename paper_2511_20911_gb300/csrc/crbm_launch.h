@@ -26,7 +26,11 @@ namespace crbm {
 // 18.5, L = 30 32.6 29.1 28.8 28.4; of 152 words with 8, 16, 32: L = 18 5.1 4.6
 // 4.7, L = 48 30.1 26.6 26.4, L = 64 74.4 50.2 47.6; L = 6, every sweep measured:
 // 1.29 with 9 warps, 1.20 with 12, one of them free to finish the measurements).
-inline int sweep_warps(const Geometry& g, int n_words, int sms) {
+// With correlations beyond L = 34, 32 warps: a sample takes as long as 20 to 40
+// sweeps there, waiting for its popcounts, and the sweep itself loses nothing (us
+// per sweep with a sample each, 16 -> 32 warps: L = 36, 1 word 228 -> 156, L = 48,
+// 384 words 1730 -> 1133; a sample every 100: 16.9 -> 16.6, 84.8 -> 79.3).
+inline int sweep_warps(const Geometry& g, int n_words, int sms, bool correlations) {
     if (g.bitplane) {
         const int groups = (g.n_cells * 10 + 31) / 32;
         const int round = (groups + 3) & ~3;  // one round of hidden groups
@@ -40,6 +44,7 @@ inline int sweep_warps(const Geometry& g, int n_words, int sms) {
     if (!g.canonical)
         return std::max(1, std::min(std::min(n_words <= sms ? 16 : n_words < 3 * sms || g.n_cells >= 64 ? 8 : 4, kMaxSweepWarps),
                                     g.n_cells));
+    if (correlations && g.L > 34) return std::min(kMaxSweepWarps, 32);
     if (n_words >= 2 * sms && g.n_cells <= 400)  // (larger ones hold one CTA per SM)
         return std::min(kMaxSweepWarps, g.n_cells < 16 ? 4 : g.n_cells < 30 || (g.n_cells >= 50 && g.n_cells <= 144) ? 8 : 12);
     return std::min(kMaxSweepWarps, g.n_cells < 8 ? 8 : g.n_cells <= 16 ? 12 : g.n_cells <= 600 || 2 * n_words <= sms ? 16 : 32);

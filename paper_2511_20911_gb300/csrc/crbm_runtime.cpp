@@ -238,8 +238,9 @@ int crbm_batch_create(crbm_batch** out, crbm_ctx* const* ctxs, int32_t n_ctx) {
     *out = nullptr;
     crbm_batch* b = new (std::nothrow) crbm_batch();
     if (!b) return CRBM_ENOMEM;
-    int warps = 1;
+    int warps = 1, sms = 0;
     bool tuned = false;
+    if (!ctxs[0] || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctxs[0]->device) != cudaSuccess || sms < 1) sms = 152;
     for (int c = 0; c < n_ctx; ++c) {
         crbm_ctx* x = ctxs[c];
         if (!x || x->layout != CRBM_LAYOUT_SMEM || x->stream != ctxs[0]->stream ||
@@ -249,7 +250,8 @@ int crbm_batch_create(crbm_batch** out, crbm_ctx* const* ctxs, int32_t n_ctx) {
             return CRBM_EINVAL;
         }
         b->ctx.push_back(x);
-        warps = std::max(warps, x->warps);
+        // (not the warps that a context of its own takes for its correlations: they would be every member's)
+        warps = std::max(warps, x->tuned ? x->warps : sweep_warps(x->g, x->n_words, sms, false));
         tuned = tuned || x->tuned;
         if (x->g.paper) b->modes |= kBatchPaper;
         if (x->g.bitplane) b->modes |= kBatchBitplane;
@@ -312,8 +314,6 @@ int crbm_batch_create(crbm_batch** out, crbm_ctx* const* ctxs, int32_t n_ctx) {
     while (items.size() % static_cast<size_t>(cluster)) items.push_back(make_int4(-1, 0, 0, 1));
     b->cluster = cluster;
     if (!tuned) {  // more CTAs than SMs: of a size that lets them share an SM
-        int sms = 0;
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctxs[0]->device) != cudaSuccess || sms < 1) sms = 152;
         const int w = batch_warps(warps, static_cast<int>(items.size()), b->smem, sms);
         if (w != warps) set_threads(b, 32 * w);
     }

@@ -27,7 +27,11 @@ int main() {
         } else if (!std::strcmp(rule, "bitplane") && std::scanf("%d %d %d", &L, &Lc, &words) == 3) {
             crbm::Geometry g = lattice(L, Lc);
             g.bitplane = 1;
-            std::printf("%d\n", crbm::sweep_warps(g, words, 152));
+            std::printf("%d\n", crbm::sweep_warps(g, words, 152, false));
+        } else if (!std::strcmp(rule, "canonical")) {
+            int correlations;
+            if (std::scanf("%d %d %d %d", &L, &Lc, &words, &correlations) != 4) return 1;
+            std::printf("%d\n", crbm::sweep_warps(lattice(L, Lc), words, 152, correlations != 0));
         } else if (!std::strcmp(rule, "batch")) {
             int warps, ctas, smem;
             if (std::scanf("%d %d %d", &warps, &ctas, &smem) != 3) return 1;

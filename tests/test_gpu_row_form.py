@@ -110,3 +110,21 @@ def test_large_lattices_on_a_persistent_grid(L, precision, monkeypatch):
         s.sweep(60)
     assert np.array_equal(many.get_spins()[:64], few.get_spins())
     assert np.array_equal(many.observables()[:64], few.observables())
+
+
+@pytest.mark.parametrize("L,n", [(36, 40), (48, 33), (68, 32)])
+def test_correlations_of_a_large_lattice(L, n, monkeypatch):
+    """One sample, after the last sweep, against the spins read back (CTAs of 32 warps beyond L = 34)."""
+    monkeypatch.delenv("CRBM_WARPS", raising=False)
+    monkeypatch.setenv("CRBM_AUTOTUNE_CACHE", "/nonexistent/none.txt")
+    params = workloads.random_params(np.random.default_rng(L), 3)
+    cp = (np.arange(n) % 3).astype(np.int32)
+    s = crbm.Sampler(L, params, n, chain_param=cp, seed=L, measure_every=2, sq_every=5)
+    assert s.warps == 32
+    s.sweep(5)
+    v = s.get_spins().astype(np.int64)
+    corr, samples = s.correlations()
+    assert np.array_equal(samples, np.bincount(cp, minlength=3))
+    for dR, dC in [(0, 0), (0, 1), (1, 0), (L // 2, L // 2), (L - 1, 3), (7, L - 2), (L // 2 - 1, 33)]:
+        c = (v * np.roll(v, (-dR, -dC), axis=(1, 2))).sum(axis=(1, 2))
+        assert np.array_equal(corr[:, dR, dC], np.bincount(cp, c, minlength=3).astype(np.int64)), (dR, dC)
