@@ -286,9 +286,13 @@ cudaError_t make_plan(const Geometry& g0, int n_words, int warps, int dev, bool 
         p.per_sm = per_sm[0];
     }
     if (p.per_sm < 1) return cudaErrorInvalidConfiguration;
-    // a CTA per word: the instantiation with the most CTAs per SM
-    p.all_cta = per_sm[1] >= per_sm[0] ? kCtaPair : kCtaAny;
-    p.resident = std::max(1, std::max(per_sm[0], per_sm[1]));
+    // a CTA per word: the instantiation with the most CTAs per SM (of as many, the one above)
+    p.all_cta = p.cta;
+    p.resident = p.per_sm;
+    if (std::max(per_sm[0], per_sm[1]) > p.per_sm) {
+        p.all_cta = per_sm[1] >= per_sm[0] ? kCtaPair : kCtaAny;
+        p.resident = std::max(per_sm[0], per_sm[1]);
+    }
     for (const int cta : {p.cta, p.all_cta})
         if ((e = check_dynamic_smem_base(reinterpret_cast<const void*>(persistent_kernel(p.mode, g.paper, cta)), dev)) != cudaSuccess)
             return e;

@@ -128,3 +128,9 @@ def test_correlations_of_a_large_lattice(L, n, monkeypatch):
     for dR, dC in [(0, 0), (0, 1), (1, 0), (L // 2, L // 2), (L - 1, 3), (7, L - 2), (L // 2 - 1, 33)]:
         c = (v * np.roll(v, (-dR, -dC), axis=(1, 2))).sum(axis=(1, 2))
         assert np.array_equal(corr[:, dR, dC], np.bincount(cp, c, minlength=3).astype(np.int64)), (dR, dC)
+
+
+@pytest.mark.parametrize("L,Lc,precision", [(14, 14, EXACT), (14, 14, PAPER), (4, 20, EXACT), (20, 4, EXACT), (12, 14, PAPER)])
+def test_words_split_in_two(orc, L, Lc, precision, monkeypatch):
+    """40 to 79 cells: bands of half the rows, each the other's neighbour above and below (two rows of cells: of one row)."""
+    check(orc, L, Lc, precision, 64, [1, 2, 5], 8, monkeypatch)
