@@ -43,13 +43,17 @@ __global__ void k_init(const Geometry g, uint32_t* v, int n_words, uint32_t k0, 
 // loads the words of sites 4 l .. 4 l + 3 and writes, chain by chain, their four
 // bytes, 128 bytes a row (N a multiple of 4, as every even lattice's; other
 // lattices write byte by byte).  Bound by the write: 113 MB in 200 us with a
-// thread per byte, two 64-bit divisions and a byte store each, 25 now.
-__global__ void k_unpack(const Geometry g, const uint32_t* v, int8_t* out, int n_words) {
-    const int lane = threadIdx.x & 31, N = g.N, blocks = (N + 127) / 128;
-    const long long n = static_cast<long long>(n_words) * blocks, step = static_cast<long long>(gridDim.x) * (blockDim.x >> 5);
+// thread per byte, two 64-bit divisions and a byte store each, 25 now.  Few words
+// wait for a warp's 32 stores in turn: they go to `parts` warps, 32 / parts chains
+// each (a call on 16 words of 18 x 18: 18.2 us with one part, 16.5 now).
+__global__ void k_unpack(const Geometry g, const uint32_t* v, int8_t* out, int n_words, int parts) {
+    const int lane = threadIdx.x & 31, N = g.N, blocks = (N + 127) / 128, chains = 32 / parts;
+    const long long n = static_cast<long long>(n_words) * blocks * parts, step = static_cast<long long>(gridDim.x) * (blockDim.x >> 5);
     const bool by4 = N % 4 == 0;
     for (long long x = blockIdx.x * static_cast<long long>(blockDim.x >> 5) + (threadIdx.x >> 5); x < n; x += step) {
-        const int word = static_cast<int>(x / blocks), s0 = static_cast<int>(x - static_cast<long long>(word) * blocks) * 128;
+        const long long y = x / parts;
+        const int word = static_cast<int>(y / blocks), s0 = static_cast<int>(y - static_cast<long long>(word) * blocks) * 128;
+        const int c0 = static_cast<int>(x - y * parts) * chains;
         uint32_t w[4];
         int site[4];
 #pragma unroll
@@ -57,9 +61,9 @@ __global__ void k_unpack(const Geometry g, const uint32_t* v, int8_t* out, int n
             site[k] = by4 ? s0 + 4 * lane + k : s0 + lane + 32 * k;
             w[k] = site[k] < N ? v[word_index(g.vil, word, N, site[k])] : 0u;
         }
-        int8_t* o = out + static_cast<size_t>(word) * 32 * N;
+        int8_t* o = out + (static_cast<size_t>(word) * 32 + c0) * N;
 #pragma unroll 4
-        for (int c = 0; c < 32; ++c, o += N) {
+        for (int c = c0; c < c0 + chains; ++c, o += N) {
             if (by4) {  // bytes 0xFF, or 0x01 where the bit is set
                 const uint32_t b = ((w[0] >> c) & 1u) | ((w[1] >> c) & 1u) << 8 | ((w[2] >> c) & 1u) << 16 | ((w[3] >> c) & 1u) << 24;
                 if (site[0] < N) *reinterpret_cast<uint32_t*>(o + site[0]) = ~(b * 0xFEu);
@@ -171,8 +175,10 @@ cudaError_t launch_sweep_generic(const SweepArgs& a, int warps_per_cta, cudaStre
 cudaError_t launch_unpack(const Geometry& g, const uint32_t* v, int8_t* out, int n_words,
                           cudaStream_t st) {
     const long long warps = static_cast<long long>(n_words) * ((g.N + 127) / 128);
-    const int blocks = static_cast<int>(std::min<long long>((warps + 7) / 8, 152 * 32));
-    k_unpack<<<blocks, 256, 0, st>>>(g, v, out, n_words);
+    int parts = 1;
+    while (parts < 8 && warps * parts < 152 * 8) parts *= 2;
+    const int blocks = static_cast<int>(std::min<long long>((warps * parts + 7) / 8, 152 * 32));
+    k_unpack<<<blocks, 256, 0, st>>>(g, v, out, n_words, parts);
     return cudaGetLastError();
 }
 
