@@ -48,8 +48,8 @@ CALLS_PER_CELL_PAPER_STREAM = 3  # streamed paper precision: the visible half-st
 # launch of k_sweep_canon_persistent (2000 sweeps of the L=18 grid), and one
 # streamed sweep of the L=384 lattice (k_stream_hidden + k_stream_visible).
 MEASURED_TRAFFIC = {
-    "grid": (8.96e6 + 0.09e6, "per launch; profiles/launches_L18_grid.md"),
-    "grid_sq": (10.60e6 + 0.11e6, "per launch with S(q) every 100 sweeps; profiles/launches_L18_grid.md"),
+    "grid": (8.34e6 + 0.05e6, "per launch; profiles/launches_L18_grid.md"),
+    "grid_sq": (10.55e6 + 0.06e6, "per launch with S(q) every 100 sweeps; profiles/launches_L18_grid.md"),
     "stream": (56.93e6 + 390.50e6 + 454.58e6 + 45.85e6, "per sweep (two launches); profiles/k_stream_L384.md"),
     "grid_paper": (8.66e6 + 0.10e6, "per launch; profiles/k_sweep_canon_persistent_L18_grid_paper.md"),
     "grid_paper_sq": (10.77e6 + 0.09e6,

@@ -251,7 +251,9 @@ int crbm_layout(const crbm_ctx* ctx);
  * spins (its chains, counters and observables are untouched), keep the
  * fastest for this context and append it to the cache file
  * ($CRBM_AUTOTUNE_CACHE, default $HOME/.cache/crbm_autotune.txt), which
- * crbm_create consults for contexts of the same shape on the same GPU model.
+ * crbm_create consults for contexts of the same shape (and with correlations
+ * or without) on the same GPU model; shapes cached by a library whose kernels
+ * differ are not taken.  Probes take correlations where the context does.
  * best_warps may be NULL.  Synchronises the stream.  Errors: CRBM_EINVAL,
  * CRBM_EUNSUPPORTED (streamed layout), CRBM_ECUDA. */
 int crbm_autotune(crbm_ctx* ctx, int64_t probe_sweeps, int32_t* best_warps);

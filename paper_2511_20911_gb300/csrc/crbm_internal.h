@@ -18,7 +18,7 @@ __host__ __device__ inline size_t word_index(int vil, int w, int N, int s) {
 #endif
 constexpr int kMaxSweepWarps = CRBM_SWEEP_MAX_THREADS / 32;  // warps per CTA of the SMEM sweeps
 #ifndef CRBM_CHUNKS_PER_WORD
-#define CRBM_CHUNKS_PER_WORD 64  // persistent SMEM sweep: a launch is about this many chunks per word
+#define CRBM_CHUNKS_PER_WORD 64  // bit-plane SMEM sweep: a launch is about this many chunks per word
 #endif
 constexpr int kMaxBonds = 16;  // filters per 3x3 window -> at most 4 hidden Philox calls
 constexpr int kNSum = 11;      // per-chain observable sums
@@ -83,7 +83,7 @@ struct Geometry {
     int8_t r1[kMaxBonds], c1[kMaxBonds], r2[kMaxBonds], c2[kMaxBonds];
     uint8_t cls[kMaxBonds];
     // canonical SMEM sweep: a row of cells is cut into n_seg segments of seg_cells cells (the last
-    // may be shorter), the unit of work of a warp; set per launch (canon_segments)
+    // may be shorter), the unit of work of a warp; set per launch (canon_plan)
     int seg_cells, n_seg;
 };
 
@@ -223,7 +223,7 @@ struct DeviceState {
     int32_t* swap_off = nullptr;  // [n_words][32]
     int32_t* swap_len = nullptr;  // [n_words][32]: thresholds for dE = 1 .. len-1 (0 beyond)
     int32_t* wq = nullptr;        // [n_words][3] Q.4 couplings (J, J', h) of each word
-    uint32_t* h = nullptr;        // streamed layout: [n_words][n_cells][10] hidden words
+    uint32_t* h = nullptr;        // streamed layout: hidden words, [n_words][n_cells][32] per lane, or [n_words][n_cells][10] with bit-plane uniforms
     int* cnt = nullptr;           // streamed layout: [n_words * 32][3] measurement counts
     float* chain_bh = nullptr;    // block proposals: [n_words * 32][2] beta, h (bf16-rounded)
     int32_t* chain_q = nullptr;   // block proposals: [n_words * 32][3] Q.4 J, J', h
@@ -251,7 +251,7 @@ struct SweepArgs {
     const int32_t* swap_len;
     const int32_t* wq;
     int swap_every;       // 0 = no replica exchange
-    int n_bands;          // batched cluster launch: CTAs (bands of cell rows) per word, else 1
+    int n_bands;          // cluster launches (few words, batches): CTAs (bands of cell rows) per word, else 1
     const int64_t* clock; // batch launches: device {sweep, measurements} (else t0 / meas0)
     int64_t* hit;         // time to solution (nullptr = off): per chain {target energy, first hitting sweep}
     const int32_t* hit_q; // per chain {Q.4 J, J', h, 0}

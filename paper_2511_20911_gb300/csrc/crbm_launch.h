@@ -26,6 +26,9 @@ namespace crbm {
 // 18.5, L = 30 32.6 29.1 28.8 28.4; of 152 words with 8, 16, 32: L = 18 5.1 4.6
 // 4.7, L = 48 30.1 26.6 26.4, L = 64 74.4 50.2 47.6; L = 6, every sweep measured:
 // 1.29 with 9 warps, 1.20 with 12, one of them free to finish the measurements).
+// Between L = 12 and 18 the 8 and 12 warps are close (304 words of L = 14, 49 cells:
+// 6.10, 5.97; 600 words of L = 16, 64 cells: 12.9, 13.1; in paper precision 4.24,
+// 4.23; 8.98, 9.43), which is where the line lies; paper precision keeps the order.
 // With correlations beyond L = 34, 32 warps: a sample takes as long as 20 to 40
 // sweeps there, waiting for its popcounts, and the sweep itself loses nothing (us
 // per sweep with a sample each, 16 -> 32 warps: L = 36, 1 word 228 -> 156, L = 48,
@@ -129,11 +132,12 @@ struct CanonSchedule {
 // 5.79 ms per 500 sweeps in chunks of 8, 5.56 in chunks of 16).  It balances the
 // SMs, at a staging and a claim (a scan of every word's state) per item.
 // All: where one chunk per word is the best anyway (265 sweeps of 600 words of
-// L = 14 on 304 CTAs, us per sweep: claimed 14.5, placed 11.7), and for short launches, of up to eight stagings a word, where the fullest SM's
-// words and their staging, once for every `resident` of them, cost less.  By
-// estimates (us): a word's sweep takes an SM 0.7 + 0.042 a cell, its staging 5 +
-// 0.009 a cell.  us per launch of one sweep, persistent -> all, 1600 words: L = 4
-// 191 -> 19, L = 6 186 -> 21, L = 12 246 -> 43; 384 words of L = 18 34 -> 21.
+// L = 14 on 304 CTAs, us per sweep: claimed 14.5, placed 11.7), and for short
+// launches, of up to eight stagings a word, where the fullest SM's words and their
+// staging, once for every `resident` of them, cost less.  By estimates (us): a
+// word's sweep takes an SM 0.7 + 0.042 a cell, its staging 5 + 0.009 a cell.  us
+// per launch of one sweep, persistent -> all, 1600 words: L = 4 191 -> 19, L = 6
+// 186 -> 21, L = 12 246 -> 43; 384 words of L = 18 34 -> 21.
 inline CanonSchedule canon_schedule(int n_sweeps, int n_words, int n_cells, int sms, int per_sm, int resident) {
     const int64_t grid = static_cast<int64_t>(per_sm) * sms;
     CanonSchedule best{false, n_sweeps};

@@ -568,7 +568,7 @@ __device__ __forceinline__ void fill_example(Example& x, int L, int bR, int bC, 
 }
 
 // Draw examples from a context's chains: chain and block origin from Philox;
-// one warp per example (38 us for 4096 examples with one thread each, 4 now).
+// one warp per example (38 us for 4096 examples with one thread each, 6 now).
 __global__ void k_prop_extract(Geometry g, const uint32_t* v, const float* chain_bh, int n_chains,
                                Example* ex, int n, uint32_t step, uint32_t k0, uint32_t k1) {
     const int e = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;

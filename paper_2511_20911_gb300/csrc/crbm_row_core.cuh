@@ -91,8 +91,7 @@ __device__ __forceinline__ void build_threshold_tables(char* tab, const uint32_t
     }
 }
 
-// w | K when q < t, as one compare and one predicated OR (the conditional
-// expression form compiles to a compare, a select and an OR).
+// w | K when q < t, as one compare and one predicated OR.
 template <uint32_t K>
 __device__ __forceinline__ uint32_t or_if_less(uint32_t w, uint32_t q, uint32_t t) {
     asm("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t@p or.b32 %0, %0, %3;\n\t}"
@@ -102,9 +101,8 @@ __device__ __forceinline__ uint32_t or_if_less(uint32_t w, uint32_t q, uint32_t 
 }
 
 // Shared-memory access by 32-bit shared address plus an immediate offset: the
-// address is an operand of the load as it is (through pointers the compiler
-// added the base of shared memory to each address, 21 additions per cell on
-// the pipe of the multiplies).  tab32, tab64: thresholds, constant while a
+// address is an operand of the load as it is, where a pointer is the base of
+// shared memory plus an index.  tab32, tab64: thresholds, constant while a
 // word is swept; lds32, lds64, lds128: state, ordered with the barriers.
 template <int kOff>
 __device__ __forceinline__ uint32_t tab32(uint32_t addr) {
